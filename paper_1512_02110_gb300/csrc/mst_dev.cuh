@@ -174,6 +174,11 @@ __device__ __forceinline__ int pad_index(const Geo& g, int ix, int iy, int iz) {
     return (ix + kHalo) + g.p0 * (iy + kHalo) + g.p01 * (iz + kHalo);
 }
 
+// padded index of linear voxel k
+__device__ __forceinline__ int pad_of(const Geo& g, int k) {
+    return pad_index(g, k % g.nx, (k / g.nx) % g.ny, k / (g.nx * g.ny));
+}
+
 // (ix, iy, iz) of padded index q, each in [-kHalo, n + kHalo). The quotients come from FP32 reciprocals and
 // are corrected by one step: q < 2^31 and the quotients are below 2^12, so the FP32 estimate is
 // off by at most one.
