@@ -149,6 +149,7 @@ TransportArgs transport_args(mst_grid* g, const mst_params* p) {
     a.omega = g->omega;
     a.adj = g->adj;
     a.gacc = g->gacc;
+    a.gbrk = g->gbrk;
     a.wbuf = g->wbuf;
     a.nevbuf = g->nevbuf;
     a.plist = g->plist;
@@ -168,6 +169,16 @@ void set_fold(TransportArgs& a, uint64_t bins) {
     const uint64_t batches = kFoldSweep / kTicketBatch;
     uint64_t slice = (bins + batches - 1) / batches;
     slice = std::max<uint64_t>(128, (slice + 31) / 32 * 32);
+    a.fold_bins = bins;
+    a.fold_slice = (uint32_t)slice;
+    a.fold_nslices = (uint32_t)((bins + slice - 1) / slice);
+}
+
+// The score kernel folds one slice of its brick tile per chunk of stored events. A photon makes
+// a few events at most on average; counting one per photon keeps a sweep within kFoldSweep photons.
+void set_score_fold(TransportArgs& a) {
+    const uint64_t bins = (uint64_t)brick_bins(a.g), chunks = kFoldSweep / kEventChunk;
+    const uint64_t slice = std::max<uint64_t>(32, ((bins + chunks - 1) / chunks + 31) / 32 * 32);
     a.fold_bins = bins;
     a.fold_slice = (uint32_t)slice;
     a.fold_nslices = (uint32_t)((bins + slice - 1) / slice);
@@ -200,8 +211,8 @@ int run_photons(mst_grid* g, const mst_params* p, bool replay, double* cimg, cud
         a.evrec = g->evrec;
         a.ev_cap = g->ev_cap;
         a.ev_count = g->ev_count;
-        a.ch_next = g->ch_next;
-        a.warp_head = g->warp_head;
+        a.ch_prev = g->ch_prev;
+        a.warp_tail = g->warp_tail;
         g->ev_warps = (uint32_t)b_fwd * kTransportWarps;
         MST_CK(cudaMemsetAsync(g->ev_count, 0, sizeof(unsigned long long), st));
     }
@@ -218,7 +229,7 @@ int run_photons(mst_grid* g, const mst_params* p, bool replay, double* cimg, cud
             }
             {
                 Phase ph(g, MST_PH_REPLAY_LIST, st);
-                MST_CK(launch_score_list(g, a.n, st));
+                MST_CK(launch_score_list(g, a.n, false, st));
             }
             a.ticket = g->tickets + 2 * l + 1;
             {
@@ -249,48 +260,38 @@ int run_photons(mst_grid* g, const mst_params* p, bool replay, double* cimg, cud
     return MST_OK;
 }
 
-// The replay of a call whose forward stored its events: W per photon from the stored events
-// (replay pass 1 over all photons instead, on the device, when they did not fit), the list of
-// photons with W != 0 over the whole call, and one pass-2 launch over it.
+// The replay of a call whose forward stored its events: the score kernel, and, on the device when
+// the events did not fit, replay pass 1 over all photons, the list of photons with W != 0 over the
+// whole call and one pass-2 launch over it.
 int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
     TransportArgs a = transport_args(g, p);
     const uint64_t n = p->n_photons;
-    set_fold(a, (uint64_t)g->geo.npad);
     a.evrec = g->evrec;
     a.ev_cap = g->ev_cap;
     a.ev_count = g->ev_count;
-    a.wseq = g->wseq;
-    a.evoff = g->evoff;
-    a.ch_next = g->ch_next;
-    a.warp_head = g->warp_head;
+    a.ch_prev = g->ch_prev;
+    a.warp_tail = g->warp_tail;
     a.n_warps = g->ev_warps;
     a.first_id = p->photon_offset;
     a.out_base = 0;
     a.n = (uint32_t)n;
     MST_CK(cudaMemsetAsync(g->tickets, 0, sizeof(unsigned int) * 3, st));
     MST_CK(cudaMemsetAsync(g->wbuf, 0, sizeof(double) * n, st));
-    {
-        Phase ph(g, MST_PH_EVENT_ADJOINT, st);
-        MST_CK(launch_event_offsets(g, a.n, st));
-        // the counts are spent: the adjoint leaves in them each photon's last event with w_s != 0
-        MST_CK(cudaMemsetAsync(g->nevbuf, 0, sizeof(uint32_t) * n, st));
-        a.ticket = g->tickets + 2;  // the adjoint's blocks take the forward warps' lists from it
-        MST_CK(launch_event_adjoint(g, a, p->grid_dtype, st));
-    }
     auto blocks = [&](int mode) { return transport_blocks(g, p->grid_dtype, mode); };
+    {
+        Phase ph(g, MST_PH_REPLAY2, st);
+        set_score_fold(a);
+        a.ticket = g->tickets + 2;  // its warps take the forward warps' lists from it
+        MST_CK(launch_score(g, a, p->grid_dtype, blocks(4), st));
+        MST_CK(launch_fold_bricks(g, st));
+    }
+    set_fold(a, (uint64_t)g->geo.npad);
     a.ticket = g->tickets;
     {
-        Phase ph(g, MST_PH_REPLAY, st);  // returns at once when the events fitted
+        Phase ph(g, MST_PH_REPLAY, st);  // these return at once when the events fitted
         MST_CK(launch_transport(g, a, p->grid_dtype, 3, blocks(3), st));
-    }
-    {
-        Phase ph(g, MST_PH_REPLAY_LIST, st);
-        MST_CK(launch_score_list(g, a.n, st));
-    }
-    a.ticket = g->tickets + 1;
-    {
-        Phase ph(g, MST_PH_REPLAY2, st);  // on the stored w_s (mode 4), or recomputing them when they did not fit
-        MST_CK(launch_transport(g, a, p->grid_dtype, 4, blocks(4), st));
+        MST_CK(launch_score_list(g, a.n, true, st));
+        a.ticket = g->tickets + 1;
         MST_CK(launch_transport(g, a, p->grid_dtype, 2, blocks(2), st));
     }
     Phase ph(g, MST_PH_FOLD, st);
@@ -303,30 +304,32 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
 int ensure_replay(mst_grid* g, uint64_t n) {
     n = std::max<uint64_t>(n, kReplayChunk);
     if (g->wbuf && g->replay_cap >= n) return MST_OK;
-    cudaFree(g->wbuf);
-    cudaFree(g->nevbuf);
-    cudaFree(g->plist);
-    cudaFree(g->evoff);
-    g->wbuf = nullptr;
-    g->nevbuf = nullptr;
-    g->plist = nullptr;
-    g->evoff = nullptr;
-    g->replay_cap = 0;
-    if (cudaMalloc(&g->wbuf, n * 8) != cudaSuccess || cudaMalloc(&g->nevbuf, n * 4) != cudaSuccess ||
-        cudaMalloc(&g->plist, n * sizeof(ScoreRec)) != cudaSuccess || cudaMalloc(&g->evoff, n * 4) != cudaSuccess) {
-        cudaGetLastError();
+    auto drop = [g]() {
         cudaFree(g->wbuf);
         cudaFree(g->nevbuf);
         cudaFree(g->plist);
-        cudaFree(g->evoff);
         g->wbuf = nullptr;
         g->nevbuf = nullptr;
         g->plist = nullptr;
-        g->evoff = nullptr;
+    };
+    drop();
+    g->replay_cap = 0;
+    if (cudaMalloc(&g->wbuf, n * 8) != cudaSuccess || cudaMalloc(&g->nevbuf, n * 4) != cudaSuccess ||
+        cudaMalloc(&g->plist, n * sizeof(ScoreRec)) != cudaSuccess) {
+        cudaGetLastError();
+        drop();
         return fail(g, MST_ERR_OOM, "replay buffers: out of device memory");
     }
     g->replay_cap = n;
     return MST_OK;
+}
+
+void drop_records(mst_grid* g) {
+    cudaFree(g->evrec);
+    cudaFree(g->ch_prev);
+    g->evrec = nullptr;
+    g->ch_prev = nullptr;
+    g->ev_cap = 0;
 }
 
 // Whether the forward of a full-gradient call of n photons stores its events, with the buffer
@@ -361,7 +364,7 @@ bool ensure_records(mst_grid* g, uint64_t n, int dtype) {
             cudaGetLastError();  // not ready yet: size from the last count that arrived
         }
     }
-    const uint64_t max_ev = std::min<uint64_t>(g->rec_budget / rec_bytes, 0xFFFFFFFFull);  // 32-bit slot indices
+    const uint64_t max_ev = std::min<uint64_t>(g->rec_budget / rec_bytes, 0xFFFFFF00ull);  // 32-bit slot indices, kNoEvent free
     // the forward reserves slots in per-warp chunks: one chunk per resident warp of headroom
     const uint64_t tails = (uint64_t)g->sm_count * transport_blocks_per_sm(dtype, 0, g->air != nullptr) *
                            kTransportWarps * kEventChunk;
@@ -370,10 +373,10 @@ bool ensure_records(mst_grid* g, uint64_t n, int dtype) {
     // few chunks from call to call do not reallocate it every time
     const uint64_t need = std::min<uint64_t>(std::max<uint64_t>((g->ev_last ? g->ev_last : 4 * n) + tails, 1024), max_ev);
     uint64_t want = std::min<uint64_t>(need + need / 4, max_ev);
-    if (!g->warp_head) {  // the forward's warps: at most kMaxWarpsPerSm per SM
-        if (cudaMalloc(&g->warp_head, sizeof(uint32_t) * (size_t)g->sm_count * kMaxWarpsPerSm) != cudaSuccess) {
+    if (!g->warp_tail) {  // the forward's warps: at most kMaxWarpsPerSm per SM
+        if (cudaMalloc(&g->warp_tail, sizeof(uint32_t) * (size_t)g->sm_count * kMaxWarpsPerSm) != cudaSuccess) {
             cudaGetLastError();
-            g->warp_head = nullptr;
+            g->warp_tail = nullptr;
             return false;
         }
     }
@@ -381,13 +384,7 @@ bool ensure_records(mst_grid* g, uint64_t n, int dtype) {
         (uint64_t)g->sm_count * kMaxWarpsPerSm)
         return false;
     if (g->evrec && g->ev_cap >= need) return true;
-    cudaFree(g->evrec);
-    cudaFree(g->wseq);
-    cudaFree(g->ch_next);
-    g->evrec = nullptr;
-    g->wseq = nullptr;
-    g->ch_next = nullptr;
-    g->ev_cap = 0;
+    drop_records(g);
     // leave a sixteenth of the device (at least 4 GiB) free for the call's other buffers, other
     // handles (a batch sizes all of its handles before it runs) and the caller: a buffer that
     // would not leave it is made smaller, and one below the need is not made (W by replay)
@@ -399,16 +396,10 @@ bool ensure_records(mst_grid* g, uint64_t n, int dtype) {
     const uint64_t reserve = std::max<uint64_t>(total_b / 16, 4ull << 30);
     want = std::min<uint64_t>(want, free_b > reserve ? (free_b - reserve) / rec_bytes : 0);
     if (want < need) return false;
-    if (cudaMalloc(&g->evrec, want * kEventWords * 4) != cudaSuccess ||
-        cudaMalloc(&g->wseq, want * sizeof(EventStep)) != cudaSuccess ||
-        cudaMalloc(&g->ch_next, sizeof(uint32_t) * (want / kEventChunk + 1)) != cudaSuccess) {
+    if (cudaMalloc(&g->evrec, want * kEventBytes) != cudaSuccess ||
+        cudaMalloc(&g->ch_prev, sizeof(uint32_t) * (want / kEventChunk + 1)) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(g->evrec);
-        cudaFree(g->wseq);
-        cudaFree(g->ch_next);
-        g->evrec = nullptr;
-        g->wseq = nullptr;
-        g->ch_next = nullptr;
+        drop_records(g);
         return false;
     }
     g->ev_cap = want;
@@ -445,11 +436,9 @@ void free_all(mst_grid* g) {
                     g->resid, g->cimg, g->lap, g->omega, g->Qw, g->stats, g->tickets, g->wbuf, g->nevbuf, g->plist, g->score_cnt};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    cudaFree(g->evrec);
-    cudaFree(g->wseq);
-    cudaFree(g->ch_next);
-    cudaFree(g->warp_head);
-    cudaFree(g->evoff);
+    drop_records(g);
+    cudaFree(g->warp_tail);
+    cudaFree(g->gbrk);
     cudaFree(g->reg_wz);
     cudaFree(g->ch_beta);
     cudaFree(g->ch_grad);
@@ -586,6 +575,7 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         }
         t.ix = iv[0]; t.iy = iv[1]; t.iz = iv[2];
         t.lx = lv[0]; t.ly = lv[1]; t.lz = lv[2];
+        g->cams.pos[c] = {(float)iv[0], (float)iv[1], (float)iv[2], 0.f, lv[0], lv[1], lv[2], 0.f};
         t.inside = inside ? 1 : 0;
         t.rx = (float)s.rot[0]; t.ry = (float)s.rot[1]; t.rz = (float)s.rot[2];
         t.ux = (float)s.rot[3]; t.uy = (float)s.rot[4]; t.uz = (float)s.rot[5];
@@ -620,6 +610,7 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         {(void**)&g->gT, C * geo.npad * 4},
         {(void**)&g->adj, nvox * g->cp * 4},
         {(void**)&g->gacc, (size_t)geo.npad * 4},
+        {(void**)&g->gbrk, (size_t)brick_bins(geo) * 4},
         {(void**)&g->score_cnt, (2 * kScoreBins + 1) * 4},
         {(void**)&g->g64, nvox * 8},
         {(void**)&g->resid, (size_t)off * 8},
@@ -654,6 +645,7 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     if (e == cudaSuccess) e = cudaMemset(g->R, 0xFF, C * geo.npad * 4);  // the halo's mark (k_los writes the rest)
     if (e == cudaSuccess) e = cudaMemset(g->Lacc, 0, nvox * g->cp * 4);
     if (e == cudaSuccess) e = cudaMemset(g->gacc, 0, (size_t)geo.npad * 4);
+    if (e == cudaSuccess) e = cudaMemset(g->gbrk, 0, (size_t)brick_bins(geo) * 4);
     if (e == cudaSuccess) e = cudaMemset(g->stats, 0, MST_NSTATS * 8 + 64);
     if (e != cudaSuccess) {
         free_all(g);
@@ -1245,13 +1237,7 @@ int mst_set_replay_memory(mst_grid* g, uint64_t bytes) {
     if (g->evrec && g->ev_cap * (uint64_t)kEventBytes > bytes) {  // shrink to the new budget at the next call
         DeviceGuard dg(g->device);
         MST_CK(cudaDeviceSynchronize());
-        cudaFree(g->evrec);
-        cudaFree(g->wseq);
-        cudaFree(g->ch_next);
-        g->evrec = nullptr;
-        g->wseq = nullptr;
-        g->ch_next = nullptr;
-        g->ev_cap = 0;
+        drop_records(g);
     }
     return MST_OK;
 }
@@ -1291,7 +1277,7 @@ struct mst_batch {
     int form = MST_BATCH_BRANCHES;    // requested form
     bool persistent = false;          // form of the captured graph
     int trip_fwd = 0, blocks_fwd = 0, trip_p2 = 0, blocks_p2 = 0;  // its wavefront (0: defaults)
-    TransportArgs* tables = nullptr;  // device [4][n]: forward, event adjoint, pass 1, pass 2
+    TransportArgs* tables = nullptr;  // device [4][n]: forward, score, pass 1, pass 2
 };
 
 namespace {
@@ -1336,7 +1322,7 @@ bool persistent_ok(const mst_batch* b, const mst_params* params) {
 }
 
 // Arguments of the persistent launches, one per scene and launch, as mst_render_grad builds them
-// for one handle (forward storing its events; event adjoint, pass 1 and pass 2 with their tickets).
+// for one handle (forward storing its events; score, pass 1 and pass 2 with their tickets).
 int persistent_tables(mst_batch* b, const float* const* betas, const mst_params* params) {
     const int n = b->n;
     std::vector<TransportArgs> t(4 * (size_t)n);
@@ -1349,8 +1335,8 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         f.evrec = g->evrec;
         f.ev_cap = g->ev_cap;
         f.ev_count = g->ev_count;
-        f.ch_next = g->ch_next;
-        f.warp_head = g->warp_head;
+        f.ch_prev = g->ch_prev;
+        f.warp_tail = g->warp_tail;
         g->ev_warps = (uint32_t)batch_launch_blocks(b, 0, b->blocks_fwd) * kTransportWarps;
         f.first_id = p->photon_offset;
         f.out_base = 0;
@@ -1358,20 +1344,19 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         f.ticket = g->tickets;
         t[i] = f;
         TransportArgs r = transport_args(g, p);
-        set_fold(r, (uint64_t)g->geo.npad);
+        set_score_fold(r);
         r.evrec = g->evrec;
         r.ev_cap = g->ev_cap;
         r.ev_count = g->ev_count;
-        r.wseq = g->wseq;
-        r.evoff = g->evoff;
-        r.ch_next = g->ch_next;
-        r.warp_head = g->warp_head;
+        r.ch_prev = g->ch_prev;
+        r.warp_tail = g->warp_tail;
         r.n_warps = g->ev_warps;
         r.first_id = p->photon_offset;
         r.out_base = 0;
         r.n = (uint32_t)p->n_photons;
-        r.ticket = g->tickets + 2;  // the event adjoint's blocks take the forward warps' lists from it
+        r.ticket = g->tickets + 2;  // the score kernel's warps take the forward warps' lists from it
         t[n + i] = r;
+        set_fold(r, (uint64_t)g->geo.npad);
         r.ticket = g->tickets;      // pass 1 (returns at once when the events fitted)
         t[2 * n + i] = r;
         r.ticket = g->tickets + 1;  // pass 2
@@ -1392,7 +1377,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
 
 // The persistent form of one batch call, enqueued while the capture stream records: each scene's
 // small kernels run on its own branch (the steps of mst_render_grad for one handle, in order),
-// and the photon transport, the stored-event adjoint and both replay passes of all scenes run as
+// and the photon transport, the score and both replay passes of all scenes run as
 // single persistent launches on the capture stream between them.
 int persistent_sequence(mst_batch* b, const float* const* betas, const mst_params* params, const double* const* meas,
                         const uint8_t* const* masks, double* const* images, double* const* grads, double* losses) {
@@ -1400,7 +1385,7 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
     mst_grid* g = nullptr;  // the scene in hand, for the error messages of MST_CK
     cudaStream_t cap = b->cap;
     const TransportArgs* t_fwd = b->tables;
-    const TransportArgs* t_adj = b->tables + n;
+    const TransportArgs* t_sco = b->tables + n;
     const TransportArgs* t_p1 = b->tables + 2 * n;
     const TransportArgs* t_p2 = b->tables + 3 * n;
     auto fork = [&]() {
@@ -1413,7 +1398,6 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
             cudaStreamWaitEvent(cap, b->join[i], 0);
         }
     };
-    const int sm = b->grids[0]->sm_count;
     auto blocks = [&](int mode, int per_sm) { return batch_launch_blocks(b, mode, per_sm); };
     // 1. staging and the counters of the forward
     fork();
@@ -1430,7 +1414,7 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
     join();
     g = b->grids[0];
     MST_CK(launch_transport_batch(t_fwd, n, 0, b->trip_fwd, blocks(0, b->blocks_fwd), cap));
-    // 2. L, images, loss, back-projection, LOS adjoint, adjoint tiles, the event slots
+    // 2. L, images, loss, back-projection, LOS adjoint, adjoint tiles
     fork();
     for (int i = 0; i < n; ++i) {
         g = b->grids[i];
@@ -1452,28 +1436,26 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
         MST_CK(cudaMemsetAsync(g->g64, 0, sizeof(double) * g->geo.nvox, st));
         MST_CK(cudaMemsetAsync(g->tickets, 0, sizeof(unsigned int) * 3, st));
         MST_CK(cudaMemsetAsync(g->wbuf, 0, sizeof(double) * np, st));
-        MST_CK(launch_event_offsets(g, (uint32_t)np, st));
-        MST_CK(cudaMemsetAsync(g->nevbuf, 0, sizeof(uint32_t) * np, st));
     }
     join();
     g = b->grids[0];
-    MST_CK(launch_event_adjoint_batch(t_adj, n, sm * 8, cap));
-    MST_CK(launch_transport_batch(t_p1, n, 3, 0, blocks(3, 0), cap));  // only scenes whose events overflowed
-    // 3. the pass-2 lists
+    MST_CK(launch_score_batch(t_sco, n, b->trip_p2, blocks(4, b->blocks_p2), cap));
+    // 3. only scenes whose events overflowed: pass 1, the pass-2 lists, pass 2
+    MST_CK(launch_transport_batch(t_p1, n, 3, 0, blocks(3, 0), cap));
     fork();
     for (int i = 0; i < n; ++i) {
         g = b->grids[i];
-        MST_CK(launch_score_list(g, (uint32_t)params[i].n_photons, b->branch[i]));
+        MST_CK(launch_score_list(g, (uint32_t)params[i].n_photons, true, b->branch[i]));
     }
     join();
     g = b->grids[0];
-    MST_CK(launch_transport_batch(t_p2, n, 4, b->trip_p2, blocks(4, b->blocks_p2), cap));
-    MST_CK(launch_transport_batch(t_p2, n, 2, 0, blocks(2, 0), cap));  // only scenes whose events overflowed
+    MST_CK(launch_transport_batch(t_p2, n, 2, 0, blocks(2, 0), cap));
     // 4. gradient: fold, W^T term, regulariser
     fork();
     for (int i = 0; i < n; ++i) {
         g = b->grids[i];
         cudaStream_t st = b->branch[i];
+        MST_CK(launch_fold_bricks(g, st));
         MST_CK(launch_fold_grad(g, st));
         MST_CK(launch_combine_full(g, g->gT, g->g64, grads[i], st));
         if (params[i].reg_eta != 0.0)
@@ -1692,8 +1674,8 @@ int mst_batch_render_grad(mst_batch* b, const float* const* betas, const mst_par
             key_add(k, g->air);
             key_add(k, g->albedo_air);
             key_add(k, g->reg_wz);
-            const void* bufs[] = {g->wbuf, g->nevbuf, g->plist, g->evoff, g->evrec, g->wseq, g->ch_next,
-                                  g->warp_head, g->Qw, g->btot, g->btot_ref};
+            const void* bufs[] = {g->wbuf, g->nevbuf, g->plist, g->evrec, g->ch_prev,
+                                  g->warp_tail, g->Qw, g->btot, g->btot_ref};
             for (const void* q : bufs) key_add(k, q);
             key_add(k, g->ev_cap);
             key_add(k, g->batch_stored);

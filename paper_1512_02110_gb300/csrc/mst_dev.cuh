@@ -44,7 +44,15 @@ struct Cam {
     int w, h, pix_off;
 };
 
+// What the local estimates need of a camera, apart and in 16-byte words: (ix, iy, iz) as floats
+// (exact: the centre lies within 1e6 voxels of the grid) and the offset (lx, ly, lz).
+struct __align__(16) CamPos {
+    float jx, jy, jz, pad0;
+    float lx, ly, lz, pad1;
+};
+
 struct CamSet {
+    CamPos pos[kMaxCams];
     int n;
     Cam c[kMaxCams];
 };
@@ -200,6 +208,26 @@ __device__ __forceinline__ bool interior_lin(const Geo& g, int q, int& k) {
     unpad(g, q, ix, iy, iz);
     k = lin_index(g, ix, iy, iz);
     return (unsigned)ix < (unsigned)g.nx && (unsigned)iy < (unsigned)g.ny && (unsigned)iz < (unsigned)g.nz;
+}
+
+// The score kernel's gradient tile keeps 2 x 2 x 2 voxels in one 32-byte sector: a straight flight
+// crosses two of them per brick on average, and atomics of one instruction on different words of a
+// sector go out as one transaction. Bin of voxel (ix, iy, iz), number of bins, voxel of a bin
+// (false: a bin past the grid's odd edge).
+__host__ __device__ __forceinline__ int brick_bins(const Geo& g) {
+    return ((g.nx + 1) >> 1) * ((g.ny + 1) >> 1) * ((g.nz + 1) >> 1) * 8;
+}
+
+__device__ __forceinline__ unsigned brick_bin(const Geo& g, unsigned ix, unsigned iy, unsigned iz) {
+    const unsigned b = (ix >> 1) + ((g.nx + 1) >> 1) * ((iy >> 1) + ((g.ny + 1) >> 1) * (iz >> 1));
+    return b * 8u + (ix & 1u) + 2u * (iy & 1u) + 4u * (iz & 1u);
+}
+
+__device__ __forceinline__ bool brick_voxel(const Geo& g, int i, int& k) {
+    const int bx = (g.nx + 1) >> 1, by = (g.ny + 1) >> 1, b = i >> 3;
+    const int ix = 2 * (b % bx) + (i & 1), iy = 2 * (b / bx % by) + (i >> 1 & 1), iz = 2 * (b / (bx * by)) + (i >> 2 & 1);
+    k = lin_index(g, ix, iy, iz);
+    return ix < g.nx && iy < g.ny && iz < g.nz;
 }
 
 template <int DT>

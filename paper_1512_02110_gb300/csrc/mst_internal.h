@@ -23,23 +23,13 @@ constexpr uint64_t kReplayChunk = 1ull << 24;    // photons per replay pass-1 / 
 // for calls of at most kRecordMaxPhotons photons; W then comes from the stored events and the
 // replay is one pass-2 launch over the call's photons.
 constexpr uint64_t kRecordMaxPhotons = 1ull << 27;
-// packed voxel, offset (3), incoming direction (3), albedo * weight, photon, event number, and the
-// free path left when the flight entered the event's voxel
-constexpr int kEventWords = 11;
-// What replay pass 2 needs of each stored event, in the photon's slot (event order): w_s, the
-// event's packed voxel and the free path left on entering it. Pass 2 then walks each flight to
-// that voxel without loading the extinction of the voxels before it.
-struct EventStep {
-    float w;
-    uint32_t vox;
-    float tau_in;
-    uint32_t pad;
-};
-constexpr int kEventBytes = kEventWords * 4 + (int)sizeof(EventStep);  // the record and its slot
+// packed voxel, offset (3) | incoming direction (3), albedo * weight | photon, event number, the free
+// path left when the flight entered the event's voxel, the photon's previous record
+constexpr int kEventBytes = 3 * 16;
 constexpr unsigned kEventChunk = 256;  // record slots a warp of the forward reserves at a time
 constexpr int kTransportWarps = 8;     // warps per transport block (256 threads)
 constexpr uint32_t kEndChunk = 0xFFFFFFFFu;  // end of a warp's chunk list
-constexpr int kMaxWarpsPerSm = 64;     // warp_head entries per SM (the forward runs 24)
+constexpr int kMaxWarpsPerSm = 64;     // warp_tail entries per SM (the forward runs 24)
 constexpr uint64_t kDefaultRecordBytes = 32ull << 30;
 constexpr uint64_t kFoldSweep = 1ull << 21;
 constexpr int kTicketBatch = 64;  // photon ids a warp takes from the global ticket at a time
@@ -76,17 +66,16 @@ struct TransportArgs {
     const double* cres;        // [total pix] dE/di of the classic images (classic-estimator gradient)
     const float* adj;          // [nvox][cp] a_c(k) = T_c(k) b_c(k) (replay)
     float* gacc;               // [npad] FP32 gradient accumulator on the padded grid (replay)
-    double* wbuf;              // [photons of the chunk] W per photon (replay pass 1, stored-event adjoint)
-    uint32_t* nevbuf;          // [photons of the chunk] events per photon (replay pass 1, or the forward
-                               // when it stores events)
-    uint32_t* evrec;           // stored events [kEventWords][ev_cap] (forward), or NULL
+    float* gbrk;               // FP32 gradient accumulator in 2 x 2 x 2 bricks (score of the stored events)
+    double* wbuf;              // [photons of the chunk] W per photon (replay pass 1; the score kernel's
+                               // running sum of each photon's later w_s)
+    uint32_t* nevbuf;          // [photons of the chunk] events per photon (replay pass 1)
+    uint4* evrec;              // stored events [3][ev_cap] (forward), or NULL
     unsigned long long ev_cap;     // capacity of evrec in events (0: no events stored)
     unsigned long long* ev_count;  // events offered for storage; > ev_cap: they did not fit
-    EventStep* wseq;           // [ev_cap] the stored events' steps, photon after photon (event order)
-    uint32_t* ch_next;         // [ev_cap / kEventChunk] next chunk of the same forward warp (kEndChunk: none)
-    uint32_t* warp_head;       // [warps of the forward launch] each warp's first chunk (kEndChunk: none)
+    uint32_t* ch_prev;         // [ev_cap / kEventChunk] previous chunk of the same forward warp (kEndChunk: none)
+    uint32_t* warp_tail;       // [warps of the forward launch] each warp's last chunk (kEndChunk: none)
     uint32_t n_warps;          // warps of the forward launch that stored the events
-    const uint32_t* evoff;     // [photons of the call] each photon's first slot in wseq
     const ScoreRec* plist;     // [kReplayChunk] photons with W != 0 (replay pass 2)
     const unsigned int* plist_n;  // entries in plist
     double* L64;               // [C][nvox] FP64 result the L tile folds into
@@ -124,13 +113,12 @@ struct mst_grid {
     float* gT = nullptr;          // [C][npad]  W_c^T (L T b)
     float* adj = nullptr;         // [nvox][cp] T_c b_c
     float* gacc = nullptr;        // [npad] gradient tile on the padded grid
+    float* gbrk = nullptr;        // [brick_bins] gradient tile in 2 x 2 x 2 bricks
     double* wbuf = nullptr;       // [replay_cap], allocated by the first full-gradient call
     uint32_t* nevbuf = nullptr;   // [replay_cap]
     mst::ScoreRec* plist = nullptr;     // [replay_cap]
-    uint32_t* evoff = nullptr;          // [replay_cap] first step slot of each photon (stored events)
-    uint64_t replay_cap = 0;            // photons the four buffers above hold
-    uint32_t* evrec = nullptr;          // [kEventWords][ev_cap] stored events (full gradient)
-    mst::EventStep* wseq = nullptr;     // [ev_cap] their steps (w_s, voxel, free path), grouped by photon
+    uint64_t replay_cap = 0;            // photons the three buffers above hold
+    uint4* evrec = nullptr;             // [3][ev_cap] stored events (full gradient)
     unsigned long long ev_cap = 0;
     unsigned long long* ev_count = nullptr;  // device counter of the last recording forward
     unsigned long long* ev_seen = nullptr;   // pinned host copy of it, read at the next call
@@ -152,8 +140,8 @@ struct mst_grid {
     const float* air = nullptr;   // [nvox] air extinction (borrowed, mst_set_air), NULL: one species
     double albedo_air = 1.0;      // single-scattering albedo of air
     const float* beta_in = nullptr;  // the running call's beta (the aerosol field with air)
-    uint32_t* ch_next = nullptr;  // [ev_cap / kEventChunk] chunk lists of the stored events
-    uint32_t* warp_head = nullptr;  // [sm_count * kMaxWarpsPerSm] first chunk of each forward warp
+    uint32_t* ch_prev = nullptr;  // [ev_cap / kEventChunk] chunk lists of the stored events
+    uint32_t* warp_tail = nullptr;  // [sm_count * kMaxWarpsPerSm] last chunk of each forward warp
     uint32_t ev_warps = 0;        // warps of the last storing forward launch
     float* btot = nullptr;        // [nvox] two species: beta + beta_air in FP32, written by the staging
     float* btot_ref = nullptr;    // [nvox] two species: beta_ref + beta_air (mst_surrogate_grad)
@@ -192,21 +180,22 @@ cudaError_t launch_channel_beta(const mst_grid* g, const float* ref, double sigm
 cudaError_t launch_channel_add(const mst_grid* g, double* grad, double sigma, const double* gmu, double* loss,
                                const double* loss_mu, cudaStream_t st);
 // transport kernel modes: 0 forward voxel LE, 1 forward classic LE, 3 replay pass 1, 2 replay pass 2,
-// 4 replay pass 2 reading w_s from the stored events, 5 / 6 passes 1 / 2 of the classic-estimator
-// gradient
+// 5 / 6 passes 1 / 2 of the classic-estimator gradient (4, the score of the stored events, is
+// launch_score)
 cudaError_t launch_transport(const mst_grid* g, const TransportArgs& a, int dtype, int mode, int blocks,
                              cudaStream_t st);
 cudaError_t launch_fold_L(const mst_grid* g, cudaStream_t st);
 cudaError_t launch_fold_grad(const mst_grid* g, cudaStream_t st);
-cudaError_t launch_score_list(const mst_grid* g, uint32_t n, cudaStream_t st);
-// W per photon from the stored events (returns at once when they did not fit)
-cudaError_t launch_event_adjoint(const mst_grid* g, const TransportArgs& a, int dtype, cudaStream_t st);
+// the pass-2 list; with `stored` its kernels return at once when the stored events fitted
+cudaError_t launch_score_list(const mst_grid* g, uint32_t n, bool stored, cudaStream_t st);
+// the score gradient from the stored events (returns at once when they did not fit), and what it
+// left in the brick tile
+cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, int blocks, cudaStream_t st);
+cudaError_t launch_fold_bricks(const mst_grid* g, cudaStream_t st);
 // backward MC images (Eq. ble): n paths per pixel, sums into sum / sum2, then sum <- means and
 // var <- variances of the means (var may be NULL)
 cudaError_t launch_bmc(const mst_grid* g, const mst_params* p, uint32_t n, double* sum, double* sum2, double* var,
                        cudaStream_t st);
-// evoff = exclusive prefix sum of the n photons' event counts (nevbuf)
-cudaError_t launch_event_offsets(const mst_grid* g, uint32_t n, cudaStream_t st);
 cudaError_t launch_los(const mst_grid* g, int dtype, const double* L, const double* jfix, const float* beta_ref,
                        const float* beta, float* T_out, float* R_out, cudaStream_t st);
 cudaError_t launch_images(const mst_grid* g, const float* R, double* images, const double* meas, const uint8_t* mask,
@@ -224,12 +213,12 @@ cudaError_t launch_classic_residual(const mst_grid* g, const double* img, const 
 cudaError_t launch_regularizer(const mst_grid* g, const float* beta, double eta, double* lap, double* psi,
                                double* loss, double* grad, cudaStream_t st);
 int transport_blocks_per_sm(int dtype, int mode, bool two);
-// The batched form (FP32 grid, one species): one persistent launch of transport mode `mode` (0, 3,
-// 4 or 2) over n scenes whose arguments sit in the device table, scene after scene in every warp;
+// The batched form (FP32 grid, one species): one persistent launch of transport mode `mode` (0, 3
+// or 2) over n scenes whose arguments sit in the device table, scene after scene in every warp;
 // trip as in the handle's wavefront setting (0: the mode's default).
 cudaError_t launch_transport_batch(const TransportArgs* table, int n, int mode, int trip, int blocks,
                                    cudaStream_t st);
-cudaError_t launch_event_adjoint_batch(const TransportArgs* table, int n, int blocks, cudaStream_t st);
+cudaError_t launch_score_batch(const TransportArgs* table, int n, int trip, int blocks, cudaStream_t st);
 // Resident blocks per SM of the batched kernels of a mode; the first call sets the attributes of
 // every batched instantiation (call it before a stream capture).
 int transport_batch_blocks_per_sm(int mode);

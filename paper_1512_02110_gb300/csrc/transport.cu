@@ -25,7 +25,7 @@ struct Photon {
     int ix, iy, iz;
     float I, tau;
     uint32_t s;      // scattering events so far
-    uint32_t hash;   // forward: path checksum; replay pass 2 on the stored events: the photon's first step slot
+    uint32_t hash;   // forward: path checksum
     uint64_t id;     // global photon id (Philox counter)
     uint32_t idx;    // call-relative index (hash / skip arrays)
 };
@@ -149,7 +149,6 @@ struct Flight {
     int lin;
     float bn;  // extinction of voxel lin, loaded ahead
     int left;  // voxel steps left before a flight is abandoned (only a non-finite direction gets there)
-    int tgt;   // replay pass 2 on the stored events: padded index of the voxel the flight ends in
 };
 
 // 1 / |d| by the hardware reciprocal (__fdividef, within 2 ulp)
@@ -183,22 +182,6 @@ __device__ __forceinline__ void flight_init(Flight& f, const TransportArgs& A, c
     f.left = g.max_steps;
 }
 
-// Replay pass 2 on the stored events: the same flight, told by the step the stored-event adjoint
-// wrote for the event that ends it (slot evoff + events so far, ph.hash holding evoff) where it
-// ends and how much free path it has left on entering that voxel (tau). Its voxels before that
-// one need no extinction: the flight crosses them.
-__device__ __forceinline__ void flight_init_stored(Flight& f, const TransportArgs& A, const Photon& ph, float& tau) {
-    const Geo& g = A.g;
-    const uint4 st = __ldg(reinterpret_cast<const uint4*>(A.wseq) + (ph.hash + ph.s));
-    flight_axis(fminf(fmaxf(ph.p.x, 0.f), g.hx), ph.d.x, g.hx, 1, f.tx, f.qx, f.dx);
-    flight_axis(fminf(fmaxf(ph.p.y, 0.f), g.hy), ph.d.y, g.hy, g.p0, f.ty, f.qy, f.dy);
-    flight_axis(fminf(fmaxf(ph.p.z, 0.f), g.hz), ph.d.z, g.hz, g.p01, f.tz, f.qz, f.dz);
-    f.lin = pad_index(g, ph.ix, ph.iy, ph.iz);
-    f.left = g.max_steps;
-    f.tgt = pad_index(g, (int)(st.y & 0x7FFu), (int)((st.y >> 11) & 0x7FFu), (int)(st.y >> 22));
-    tau = __uint_as_float(st.z);
-}
-
 // One voxel of a free flight (Eq. MCextinct): the free path tau runs out in this voxel when
 // tau <= beta * (distance to the next face). Returns true then, or when the voxel is the halo
 // (beta = +inf; the caller tells the two apart by b), with b and the face distance m of the voxel;
@@ -227,27 +210,6 @@ __device__ __forceinline__ bool flight_step(const TransportArgs& A, Flight& f, f
     f.ty = py ? f.qy : f.ty - m;
     f.tz = (px || py) ? f.tz - m : f.qz;
     f.lin = next;
-    return false;
-}
-
-// One voxel of a replay pass-2 flight whose end is known (flight_init_stored): true in the voxel
-// the flight ends in (the caller loads its extinction there), else the voxel receives -S *
-// length in the gradient tile and the flight crosses into the next one, by the arithmetic of
-// flight_step, so that it visits the same voxels.
-__device__ __forceinline__ bool flight_step_stored(const TransportArgs& A, Flight& f, float S, unsigned& nsc) {
-    // (a voxel index past the padded grid would mean the walk missed its end: it stops there)
-    if (f.lin == f.tgt || (unsigned)f.lin >= (unsigned)A.g.npad) return true;
-    const float m = fminf(f.tx, fminf(f.ty, f.tz));
-    const bool px = f.tx <= m;
-    const bool py = !px && f.ty <= m;
-    if (S != 0.f && m > 0.f) {
-        atomicAdd(A.gacc + f.lin, -S * m);
-        ++nsc;
-    }
-    f.tx = px ? f.qx : f.tx - m;
-    f.ty = py ? f.qy : f.ty - m;
-    f.tz = (px || py) ? f.tz - m : f.qz;
-    f.lin += px ? f.dx : (py ? f.dy : f.dz);
     return false;
 }
 
@@ -293,9 +255,12 @@ __device__ __forceinline__ int flight_end(const TransportArgs& A, Photon& ph, co
 }
 
 // cosine between the photon direction and the direction from the photon to camera c, and the
-// squared distance; r2 = 0 when the photon sits on the centre of projection
-__device__ __forceinline__ float cam_cosine(const TransportArgs& A, const Photon& ph, const Cam& cm, float& r2) {
-    const float3 v = local_delta(A.g, ph.ix, ph.iy, ph.iz, ph.p, cm.ix, cm.iy, cm.iz, make_float3(cm.lx, cm.ly, cm.lz));
+// squared distance; r2 = 0 when the photon sits on the centre of projection. `at` holds the
+// photon's voxel indices as floats: whole numbers below 2^24, so the difference to the camera's
+// is exact and needs no conversion per camera.
+__device__ __forceinline__ float cam_cosine(const TransportArgs& A, const Photon& ph, float3 at, const CamPos& cm, float& r2) {
+    const float3 v = make_float3((cm.jx - at.x) * A.g.hx + (cm.lx - ph.p.x), (cm.jy - at.y) * A.g.hy + (cm.ly - ph.p.y),
+                                 (cm.jz - at.z) * A.g.hz + (cm.lz - ph.p.z));
     r2 = v.x * v.x + v.y * v.y + v.z * v.z;
     return r2 > 0.f ? (ph.d.x * v.x + ph.d.y * v.y + ph.d.z * v.z) * rsqrtf(r2) : 0.f;
 }
@@ -328,20 +293,22 @@ __device__ __forceinline__ float phase_of(const TransportArgs& A, float mu) {
 template <bool AIR>
 __device__ __forceinline__ void le_voxel_p(const TransportArgs& A, const Photon& ph, float w, int k) {
     float* row = A.Lacc + (size_t)k * A.cp;
-    for (int c0 = 0; c0 < A.cams.n; c0 += 4) {
+    const float3 at = make_float3((float)ph.ix, (float)ph.iy, (float)ph.iz);
+#pragma unroll 1  // (unrolled, the forward outgrows the instruction cache: 38.1 -> 41.9 ms)
+    for (int q = 0; 4 * q < A.cams.n; ++q) {
         float v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int c = c0 + j;
+            const int c = 4 * q + j;
             float val = 0.f;
             if (c < A.cams.n) {
                 float r2;
-                const float mu = cam_cosine(A, ph, A.cams.c[c], r2);
+                const float mu = cam_cosine(A, ph, at, A.cams.pos[c], r2);
                 if (r2 > 0.f) val = w * phase_of<AIR>(A, mu);
             }
             v[j] = val;
         }
-        atomicAdd(reinterpret_cast<float4*>(row + c0), make_float4(v[0], v[1], v[2], v[3]));
+        atomicAdd(reinterpret_cast<float4*>(row + 4 * q), make_float4(v[0], v[1], v[2], v[3]));
     }
 }
 
@@ -354,20 +321,29 @@ __device__ __forceinline__ void le_voxel(const TransportArgs& A, const Photon& p
 template <bool AIR>
 __device__ __forceinline__ float le_adjoint_p(const TransportArgs& A, const Photon& ph, float w, int k) {
     const float4* row = reinterpret_cast<const float4*>(A.adj + (size_t)k * A.cp);
+    const float3 at = make_float3((float)ph.ix, (float)ph.iy, (float)ph.iz);
     float acc = 0.f;
-    for (int c0 = 0; c0 < A.cams.n; c0 += 4) {
-        const float4 a4 = __ldg(row + (c0 >> 2));
+    auto group = [&](int q) {
+        const float4 a4 = __ldg(row + q);
         const float aa[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int c = c0 + j;
-            if (c < A.cams.n && aa[j] != 0.f) {
+            const int c = 4 * q + j;
+            if (c < A.cams.n) {
                 float r2;
-                const float mu = cam_cosine(A, ph, A.cams.c[c], r2);
-                if (r2 > 0.f) acc += aa[j] * w * phase_of<AIR>(A, mu);
+                const float mu = cam_cosine(A, ph, at, A.cams.pos[c], r2);
+                const float v = aa[j] * w * phase_of<AIR>(A, mu);
+                acc += aa[j] != 0.f && r2 > 0.f ? v : 0.f;
             }
         }
-    }
+    };
+    // the first groups unrolled: their cameras' constants are operands of the arithmetic then
+    // instead of loads (score of 3.7e8 events with 9 cameras: 20.8 -> 19.5 ms)
+    group(0);
+    if (A.cams.n > 4) group(1);
+    if (A.cams.n > 8) group(2);
+#pragma unroll 1
+    for (int q = 3; 4 * q < A.cams.n; ++q) group(q);
     return acc;
 }
 
@@ -619,28 +595,19 @@ __device__ __forceinline__ void finish_photon(const TransportArgs& A, const Phot
     if (A.point)
         A.point[ph.idx] = make_float4(ph.p.x, ph.p.y, ph.p.z,
                                       __uint_as_float((uint32_t)ph.ix | ((uint32_t)ph.iy << 11) | ((uint32_t)ph.iz << 22)));
-    if (A.ev_cap) A.nevbuf[ph.idx - A.out_base] = ph.s;  // forward storing events: the count pass 2 stops at
 }
 
-// One stored event (forward, full gradient): what w_s = sum_c a_c(k) albedo I_s P_c(s) needs.
-// Word 9 holds the event number, with the particle (1: air) in bit 31; word 10 the free path left
-// when the flight entered the event's voxel (e.tau, set at the collision), with which replay
-// pass 2 ends the flight there.
+// One stored event (forward, full gradient), three 16-byte words: where it happened; the incoming
+// direction and albedo * weight; the photon, the event number with the particle (1: air) in bit
+// 31, the free path left when the flight entered the event's voxel (e.tau, set at the collision),
+// and the record of the photon's previous event (kNoEvent: none), where this event's flight began.
 __device__ __forceinline__ void store_event(const TransportArgs& A, unsigned long long i, const Photon& e, float wgt,
-                                            bool air) {
-    const unsigned long long C = A.ev_cap;
-    uint32_t* r = A.evrec + i;
-    r[0] = (uint32_t)e.ix | ((uint32_t)e.iy << 11) | ((uint32_t)e.iz << 22);
-    r[C] = __float_as_uint(e.p.x);
-    r[2 * C] = __float_as_uint(e.p.y);
-    r[3 * C] = __float_as_uint(e.p.z);
-    r[4 * C] = __float_as_uint(e.d.x);
-    r[5 * C] = __float_as_uint(e.d.y);
-    r[6 * C] = __float_as_uint(e.d.z);
-    r[7 * C] = __float_as_uint(wgt);
-    r[8 * C] = e.idx - A.out_base;
-    r[9 * C] = e.s | (air ? 0x80000000u : 0u);
-    r[10 * C] = __float_as_uint(e.tau);  // the free path left on entering the event's voxel
+                                            bool air, uint32_t prev) {
+    uint4* r = A.evrec + i;
+    r[0] = make_uint4((uint32_t)e.ix | ((uint32_t)e.iy << 11) | ((uint32_t)e.iz << 22), __float_as_uint(e.p.x),
+                      __float_as_uint(e.p.y), __float_as_uint(e.p.z));
+    r[A.ev_cap] = make_uint4(__float_as_uint(e.d.x), __float_as_uint(e.d.y), __float_as_uint(e.d.z), __float_as_uint(wgt));
+    r[2 * A.ev_cap] = make_uint4(e.idx - A.out_base, e.s | (air ? 0x80000000u : 0u), __float_as_uint(e.tau), prev);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -656,13 +623,14 @@ __device__ __forceinline__ void store_event(const TransportArgs& A, unsigned lon
 
 constexpr int kScoreTile = 4096;   // photons per block in the list kernels
 // Stored events are written in per-warp chunks of kEvChunk slots (one reservation on the global
-// counter per chunk). A warp's photons come from its own ticket batches, so a chunk holds the
-// events of a few dozen photons, and the adjoint that walks a chunk finds their W and step slots
-// together in cache instead of scattered over all photons in flight. The buffer keeps one chunk
-// per resident warp of headroom for the chunks' unused tails.
+// counter per chunk). A warp's photons come from its own ticket batches and all events of a photon
+// lie in its warp's chunks in the order they happened, so the score kernel can walk a warp's
+// chunks backwards and meet every photon's events from the last to the first. The buffer keeps
+// one chunk per resident warp of headroom for the chunks' unused tails.
 constexpr unsigned kEvChunk = kEventChunk;
 static_assert(kTB / 32 == kTransportWarps, "transport block size");
 constexpr uint32_t kNoPhoton = 0xFFFFFFFFu;  // photon word of a chunk's unused tail slots
+constexpr uint32_t kNoEvent = 0xFFFFFFFFu;   // previous record of a photon's first event
 constexpr int kSlots = 64;
 // Voxels a flying lane advances per loop trip, and minimum resident blocks per SM (register
 // budget), per kernel mode; set from sweeps on the 64^3 cumulus workload.
@@ -673,11 +641,13 @@ constexpr int kMinBlocksForward = 3;
 constexpr int kMinBlocksClassic = 3;
 constexpr int kMinBlocksPass1 = 3;
 constexpr int kMinBlocksPass2 = 3;
+constexpr int kMinBlocksScore = 3;
+constexpr int kStepsScore = 6;  // list entries a score lane adds per loop trip
 
 // kernel modes
-// kPass2W: replay pass 2 reading w_s from the stored events instead of recomputing them;
-// kPass1C, kPass2C: passes 1 and 2 of the classic-estimator gradient
-constexpr int kFwdVoxel = 0, kFwdClassic = 1, kPass2 = 2, kPass1 = 3, kPass2W = 4, kPass1C = 5, kPass2C = 6;
+// kScore: the score of the stored events (k_score); kPass1C, kPass2C: passes 1 and 2 of the
+// classic-estimator gradient
+constexpr int kFwdVoxel = 0, kFwdClassic = 1, kPass2 = 2, kPass1 = 3, kScore = 4, kPass1C = 5, kPass2C = 6;
 
 template <int NW>
 struct Stack {
@@ -685,9 +655,10 @@ struct Stack {
     int cap;
 };
 
-template <bool REPLAY>
+// words of a stack slot: the photon; the forward's previous record, or a replay's event count and sum
+template <int MODE>
 struct Rec {
-    static constexpr int NW = REPLAY ? 15 : 12;
+    static constexpr int NW = MODE >= kPass2 ? 15 : (MODE == kFwdVoxel ? 13 : 12);
 };
 
 template <int NW>
@@ -706,8 +677,8 @@ __device__ __forceinline__ void put(const Stack<NW>& q, int slot, const Photon& 
     b[9 * c] = ph.s;
     b[10 * c] = ph.hash;
     b[11 * c] = ph.idx;
-    if (NW > 12) {
-        b[12 * c] = nev;
+    if (NW > 12) b[12 * c] = nev;
+    if (NW > 13) {
         b[13 * c] = (uint32_t)__double_as_longlong(acc);
         b[14 * c] = (uint32_t)((unsigned long long)__double_as_longlong(acc) >> 32);
     }
@@ -730,11 +701,10 @@ __device__ __forceinline__ void get(const Stack<NW>& q, int slot, const Transpor
     ph.hash = b[10 * c];
     ph.idx = b[11 * c];
     ph.id = A.first_id + (ph.idx - A.out_base);
-    if (NW > 12) {
-        nev = b[12 * c];
+    nev = NW > 12 ? b[12 * c] : 0u;
+    if (NW > 13) {
         acc = __longlong_as_double((long long)((unsigned long long)b[13 * c] | ((unsigned long long)b[14 * c] << 32)));
     } else {
-        nev = 0u;
         acc = 0.0;
     }
 }
@@ -764,7 +734,7 @@ __device__ __forceinline__ uint4 unstash_block(const Stack<NW>& q, int slot) {
 // 32-bit atomics, so nothing added is lost; each bin's FP32 partial covers at most one sweep.
 template <int MODE>
 __device__ __forceinline__ void fold_slice(const TransportArgs& A, uint32_t batch, unsigned lane) {
-    if constexpr (MODE == kFwdVoxel || MODE == kPass2 || MODE == kPass2W || MODE == kPass2C) {
+    if constexpr (MODE == kFwdVoxel || MODE == kPass2 || MODE == kPass2C) {
         if (A.fold_bins == 0u) return;
         const uint64_t i0 = (uint64_t)(batch % A.fold_nslices) * A.fold_slice;
         const uint64_t i1 = min(i0 + A.fold_slice, A.fold_bins);
@@ -863,7 +833,7 @@ __device__ __forceinline__ void flush_tally(const TransportArgs& A, const Tally&
 // code. TRIP: voxels a flying lane advances per loop trip (0: the mode's default), a compile-time
 // constant (a run-time bound cost the forward 2 %); the autotuner picks among the instantiated ones.
 constexpr int min_blocks(int mode) {
-    return (mode == kPass2 || mode == kPass2W)
+    return mode == kPass2
                ? kMinBlocksPass2
                : (mode == kPass1 ? kMinBlocksPass1
                                  : ((mode == kFwdClassic || mode == kPass1C || mode == kPass2C) ? kMinBlocksClassic
@@ -875,11 +845,11 @@ constexpr int min_blocks(int mode) {
 template <int DT, int MODE, bool TWO, int TRIP>
 __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* smem) {
     constexpr bool PASS1 = MODE == kPass1 || MODE == kPass1C;
-    constexpr bool PASS2 = MODE == kPass2 || MODE == kPass2W || MODE == kPass2C;
+    constexpr bool PASS2 = MODE == kPass2 || MODE == kPass2C;
     constexpr bool CLASSIC = MODE == kFwdClassic || MODE == kPass1C || MODE == kPass2C;
     constexpr bool REPLAY = PASS1 || PASS2;
     constexpr int kStepsPerTrip = TRIP > 0 ? TRIP : (PASS2 ? kStepsPass2 : (PASS1 ? kStepsPass1 : kStepsForward));
-    constexpr int NW = Rec<REPLAY>::NW;
+    constexpr int NW = Rec<MODE>::NW;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned warp = threadIdx.x >> 5;
     const Stack<NW> stk{smem + warp * NW * kSlots, kSlots};  // events at slot i, ready photons at kSlots-1-i
@@ -912,18 +882,15 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     Photon ph;
     Flight w;
     float tau = 0.f;
-    uint32_t nev = 0u;  // pass 2: events of pass 1
+    uint32_t nev = 0u;  // pass 2: events of pass 1; forward: the photon's last record
     double acc = 0.0;   // pass 1: W; pass 2: S
     bool fly = false, dry = false;
     uint32_t wbase = 0u, wend = 0u;
     unsigned segments = 0u, scatters = 0u, events = 0u;
     EventCount<TWO && !REPLAY> air_events;  // two species: forward events on air
     const uint32_t pool_n = PASS2 ? *A.plist_n : A.n;  // pass 2 walks the list built from pass 1
-    if (A.ev_cap) {  // a call whose forward stored its events: one of each pair of kernels works
-        const bool fit = *A.ev_count <= A.ev_cap;
-        if ((PASS1 || MODE == kPass2) && fit) return;  // W and w_s come from the stored events
-        if (MODE == kPass2W && !fit) return;           // they did not fit: pass 1 and kPass2 run
-    }
+    // a call whose forward stored its events: the score kernel did the replay unless they did not fit
+    if ((PASS1 || MODE == kPass2) && A.ev_cap && *A.ev_count <= A.ev_cap) return;
 
     for (;;) {
         // (1) fill: ready photons first, new photons only when the ready stack is empty
@@ -933,12 +900,8 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             const int take = min(__popc(empty), rd_n);
             if (!fly && rank < take) {
                 get(stk, kSlots - rd_n + rank, A, ph, nev, acc);
-                if constexpr (MODE == kPass2W) {
-                    flight_init_stored(w, A, ph, tau);
-                } else {
-                    flight_init<DT>(w, A, ph);
-                    tau = ph.tau;
-                }
+                flight_init<DT>(w, A, ph);
+                tau = ph.tau;
                 fly = true;
             }
             rd_n -= take;
@@ -946,7 +909,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
         }
         refill(A, pool_n, fly, dry, wbase, wend, lane, [&](uint32_t j) -> bool {
             uint32_t pid = j;
-            nev = 0u;
+            nev = MODE == kFwdVoxel ? kNoEvent : 0u;
             acc = 0.0;
             if (PASS2) {  // item j of the pass-1 list
                 const ScoreRec r = A.plist[j];
@@ -956,17 +919,12 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             } else if (A.skip && A.skip[A.out_base + j]) {
                 if (A.hash) A.hash[A.out_base + j] = 0u;
                 if (PASS1) A.wbuf[j] = 0.0;
-                if (PASS1 || A.ev_cap) A.nevbuf[j] = 0u;
+                if (PASS1) A.nevbuf[j] = 0u;
                 return false;
             }
             launch_photon(A, ph, pid);
-            if constexpr (MODE == kPass2W) {
-                ph.hash = A.evoff[pid];
-                flight_init_stored(w, A, ph, tau);
-            } else {
-                flight_init<DT>(w, A, ph);
-                tau = ph.tau;
-            }
+            flight_init<DT>(w, A, ph);
+            tau = ph.tau;
             t.add_launch(A.I0);
             return true;
         }, [&](uint32_t t0) { fold_slice<MODE>(A, t0 / (uint32_t)kTicketBatch, lane); });
@@ -980,38 +938,18 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             int nstep = 0;
             bool stop = false;
             float b = 0.f, m = 0.f;
-            if constexpr (MODE == kPass2W) {  // the flight's last voxel is known: no extinction before it
 #pragma unroll 1
-                while (nstep < kStepsPerTrip) {
-                    ++nstep;
-                    if (flight_step_stored(A, w, S, scatters)) {
-                        stop = true;
-                        break;
-                    }
+            while (nstep < kStepsPerTrip) {
+                ++nstep;
+                if (flight_step<DT, PASS2>(A, w, tau, b, m, S, scatters)) {
+                    stop = true;
+                    break;
                 }
-                if (stop) {
-                    r = (unsigned)w.lin < (unsigned)A.g.npad
-                            ? flight_end<TWO>(A, ph, w, tau, BetaFetch<DT>::get(A.beta_pad, w.lin), S, scatters)
-                            : kWalkOverflow;
-                    // a stored flight ends in its event; any other end is a replay that left the
-                    // forward's path, counted as lost (0 in valid use; the fold drops what such a
-                    // walk added to the halo)
-                    if (r != kCollided) atomicAdd(A.stats + MST_ST_LOST, 1.0);
-                }
-            } else {
-#pragma unroll 1
-                while (nstep < kStepsPerTrip) {
-                    ++nstep;
-                    if (flight_step<DT, PASS2>(A, w, tau, b, m, S, scatters)) {
-                        stop = true;
-                        break;
-                    }
-                }
-                if (stop) {
-                    r = flight_end<TWO>(A, ph, w, tau, b, S, scatters);
-                    if (r >= 0) --nstep;  // the halo voxel is no segment of the path
-                    if (MODE == kFwdVoxel && r == kCollided) ph.tau = tau;  // kept for the stored event
-                }
+            }
+            if (stop) {
+                r = flight_end<TWO>(A, ph, w, tau, b, S, scatters);
+                if (r >= 0) --nstep;  // the halo voxel is no segment of the path
+                if (MODE == kFwdVoxel && r == kCollided) ph.tau = tau;  // kept for the stored event
             }
             segments += nstep;
             // a flight longer than any straight walk through the grid is abandoned
@@ -1050,12 +988,12 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             if (MODE == kFwdVoxel && A.ev_cap) {
                 // the round's slots continue the warp's chunk and spill into a new one
                 unsigned long long nb = 0ull;
-                if (ch_fill + (unsigned)n > kEvChunk) {  // a new chunk, linked after the warp's last one
+                if (ch_fill + (unsigned)n > kEvChunk) {  // a new chunk, linked to the warp's last one
                     if (lane == 0u) {
                         nb = atomicAdd(A.ev_count, (unsigned long long)kEvChunk);
-                        const uint32_t nc = (uint32_t)(nb / kEvChunk);
-                        if (ch_base == ~0ull) A.warp_head[gwarp] = nc;
-                        else if (ch_base + kEvChunk <= A.ev_cap) A.ch_next[ch_base / kEvChunk] = nc;
+                        // (a chunk past the buffer is not linked: the call then replays instead)
+                        if (nb + kEvChunk <= A.ev_cap)
+                            A.ch_prev[nb / kEvChunk] = ch_base == ~0ull ? kEndChunk : (uint32_t)(ch_base / kEvChunk);
                     }
                     nb = __shfl_sync(kFull, nb, 0);
                 }
@@ -1133,15 +1071,14 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                     const float wgt = (air ? A.albedo_air : A.albedo) * e.I;
                     if (!REPLAY) {
                         e.hash = (e.hash ^ (uint32_t)k) * kFnvPrime;
-                        if (MODE == kFwdVoxel && A.ev_cap && ev_slot < A.ev_cap) store_event(A, ev_slot, e, wgt, air);
+                        if (MODE == kFwdVoxel && A.ev_cap && ev_slot < A.ev_cap) store_event(A, ev_slot, e, wgt, air, enev);
+                        if (MODE == kFwdVoxel) enev = (uint32_t)ev_slot;
                         le_voxel(A, e, wgt, k, air);
                         if constexpr (TWO) xb = unstash_block(stk, slot);
                         term = after_event<TWO>(A, e, t, air, xb);
                         if (term) finish_photon(A, e, term);
                     } else {
-                        float we;
-                        if constexpr (MODE == kPass2W) we = A.wseq[e.hash + e.s - 1u].w;
-                        else we = le_adjoint(A, e, wgt, k, air);
+                        const float we = le_adjoint(A, e, wgt, k, air);
                         if (PASS1) {
                             eacc += (double)we;
                             if constexpr (TWO) xb = unstash_block(stk, slot);
@@ -1159,7 +1096,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                             }
                             if constexpr (TWO) xb = unstash_block(stk, slot);
                             term = e.s == enev ? 1 : after_event<TWO>(A, e, t, air, xb);  // stop at pass 1's last event
-                            eacc -= (double)we;  // after the scattering step, which hides the w_s load
+                            eacc -= (double)we;
                         }
                     }
                 }
@@ -1189,14 +1126,11 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     } else {
         flush_tally(A, t.load(), segments, events, lane);
         air_events.flush(A.stats + MST_ST_AIR_EVENTS, lane);
-        if (MODE == kFwdVoxel && A.ev_cap) {  // close the warp's list; its last chunk's tail holds no event
-            if (ch_base == ~0ull) {
-                if (lane == 0u) A.warp_head[gwarp] = kEndChunk;
-            } else {
-                if (lane == 0u && ch_base + kEvChunk <= A.ev_cap) A.ch_next[ch_base / kEvChunk] = kEndChunk;
+        if (MODE == kFwdVoxel && A.ev_cap) {  // the warp's last chunk; its tail holds no event
+            if (lane == 0u) A.warp_tail[gwarp] = ch_base == ~0ull ? kEndChunk : (uint32_t)(ch_base / kEvChunk);
+            if (ch_base != ~0ull)
                 for (unsigned f = ch_fill + lane; f < kEvChunk; f += 32u)
-                    if (ch_base + f < A.ev_cap) A.evrec[8ull * A.ev_cap + ch_base + f] = kNoPhoton;
-            }
+                    if (ch_base + f < A.ev_cap) A.evrec[2ull * A.ev_cap + ch_base + f].x = kNoPhoton;
         }
     }
 }
@@ -1220,205 +1154,268 @@ __global__ void __launch_bounds__(kTB, min_blocks(MODE))
     }
 }
 
-// w_s of every event the forward stored, instead of replay pass 1: the same arithmetic
-// (le_adjoint) on the same event state, written with the event's voxel and free path to the
-// photon's step slot in wseq for pass 2, and added to W in FP64; nevbuf (zeroed after the slot
-// scan) receives each photon's last event with w_s != 0. Does nothing when the events did not
-// fit (pass 1 then walks the paths).
-template <bool TWO>
-__device__ __forceinline__ void event_adjoint_run(const TransportArgs& A) {
-    const unsigned long long cnt = *A.ev_count;  // reserved slots: whole chunks
-    if (cnt > A.ev_cap) return;
-    const unsigned long long C = A.ev_cap;
-    unsigned long long stored = 0ull;
-    // A block follows one forward warp's chunks in the order the warp wrote them (lists taken
-    // from a ticket): a photon's events lie in one or two neighbouring chunks of its warp, so its
-    // W, offset and step slots are used while they are still cached.
-    __shared__ uint32_t list;
+// ------------------------------------------------------------------------------------------
+// The score gradient from the stored events. The flight that ended in event s of a photon scores
+// S_s = sum_{s' >= s} w_s' (Eq. DirectJacob on the residual), w_s = sum_c a_c(k) albedo I_s P_c(s):
+// every voxel it crossed receives -S_s * length, its last voxel S_s (1/beta - length). Each flight is
+// told by two records (where the event before it happened, and its own direction, last voxel and
+// free path there), so nothing is walked from the Philox keys, and flights need not follow one
+// another: a warp takes one forward warp's chunks from the last to the first, so that it meets
+// every photon's events in falling order and S is a running sum per photon (FP64), and its lanes
+// walk whatever flights are queued.
+//
+// A batch is 32 records: w_s, S, the last voxel's term, and the flight's set-up (the number of faces
+// it crosses is known: the sum of the index differences of its end voxels), queued in shared
+// memory; the next batch's records are on their way meanwhile (cp.async). A trip refills idle lanes
+// from the queue and walks K voxels per lane; the (bin, term) entries go through a shared-memory
+// strip and out transposed, so that one atomic instruction holds consecutive voxels of a few
+// flights. Random FP32 atomics run at 2.0e11 a second on this chip whatever the tile's size, but
+// the words of one 32-byte sector go out together, and the tile keeps 2 x 2 x 2 voxels in a sector.
+
+constexpr int kFlightWords = 10;  // of a queued flight
+constexpr int kScoreSlots = 64;   // flights a warp queues: fewer than 32 left when a batch adds 32
+constexpr uint32_t kNoEntry = 0xFFFFFFFFu;
+
+template <int K>
+constexpr int score_words() {  // shared words per warp: a batch of records, the queue, the strip
+    return 3 * 4 * 32 + kFlightWords * kScoreSlots + 2 * 32 * K;
+}
+
+// One axis of a score flight: the distance to the next face and between faces, as flight_axis
+// computes them, without its branches (32 flights are set up at once).
+__device__ __forceinline__ void score_axis(float p, float d, float h, float& t, float& q) {
+    const float inv = __fdividef(1.f, fabsf(d));
+    p = fminf(fmaxf(p, 0.f), h);
+    const float u = (d > 0.f ? h - p : p) * inv;
+    t = d == 0.f ? CUDART_INF_F : u;
+    q = h * inv;
+}
+
+__device__ __forceinline__ void copy16_async(uint32_t* dst, const uint4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <int DT, bool TWO, int K>
+__device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem) {
+    if (*A.ev_count > A.ev_cap) return;  // the events did not fit: the replay passes run instead
+    const unsigned lane = threadIdx.x & 31u;
+    uint32_t* rec = smem + (threadIdx.x >> 5) * score_words<K>();  // the lane's record words f at rec[(f * 32 + lane) * 4]
+    uint32_t* q = rec + 3 * 4 * 32;                                // queue: word f of slot i at q[f * kScoreSlots + i]
+    float2* strip = reinterpret_cast<float2*>(q + kFlightWords * kScoreSlots);
+    const unsigned nbins = (unsigned)brick_bins(A.g);
+    const uint32_t by8 = 8u * (unsigned)((A.g.nx + 1) >> 1), bz8 = by8 * (unsigned)((A.g.ny + 1) >> 1);
+    unsigned stored = 0u, flights = 0u, entries = 0u, lost = 0u;
+
+    // The flight in hand: t and q as in Flight, and per axis the step of its bin (the stride of the
+    // bricks, signed, with the axis' bit of the voxel inside the brick). `at` is the bin with the
+    // bits of the axes the flight descends mirrored (`flip`): a crossing toggles the axis' bit and
+    // enters the next brick when it was set.
+    float tx = 0.f, ty = 0.f, tz = 0.f, qx = 0.f, qy = 0.f, qz = 0.f, nS = 0.f;
+    uint32_t sx = 0u, sy = 0u, sz = 0u, at = 0u, flip = 0u, goal = 0u;
+    int left = 0;  // faces still to cross; 0: no flight
+
+    // the next batch: its records are being copied (pending), or the lists are used up
+    uint32_t ch = kEndChunk, prev = kEndChunk;
+    int base = -1;
+    bool pending = false;
+    auto fetch = [&]() {
+        if (base < 0) {  // the next chunk of the list, or the next list
+            ch = prev;
+            while (ch == kEndChunk) {
+                unsigned l = 0u;
+                if (lane == 0u) l = atomicAdd(A.ticket, 1u);
+                l = __shfl_sync(kFull, l, 0);
+                if (l >= A.n_warps) break;
+                ch = A.warp_tail[l];
+            }
+            pending = ch != kEndChunk;
+            if (!pending) return;
+            prev = A.ch_prev[ch];
+            base = (int)kEvChunk - 32;
+            // one slice of the rolling fold (see kFoldSweep) per chunk
+            const uint32_t i0 = ch % A.fold_nslices * A.fold_slice;
+            const uint32_t i1 = min(i0 + A.fold_slice, (uint32_t)A.fold_bins);
+            for (uint32_t i = i0 + lane; i < i1; i += 32) {
+                const float v = atomicExch(A.gbrk + i, 0.f);
+                int k;
+                if (v != 0.f && brick_voxel(A.g, (int)i, k)) atomicAdd(A.g64 + k, (double)v);
+            }
+        }
+        const uint4* r = A.evrec + ((unsigned long long)ch * kEvChunk + (unsigned)base + lane);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) copy16_async(rec + (f * 32 + lane) * 4, r + f * A.ev_cap);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        base -= 32;
+        pending = true;
+    };
+    fetch();
+
+    int qn = 0;  // queued flights (warp-uniform)
     for (;;) {
-        if (threadIdx.x == 0) list = atomicAdd(A.ticket, 1u);
-        __syncthreads();
-        const uint32_t gw = list;
-        __syncthreads();
-        if (gw >= A.n_warps) break;
-        for (uint32_t ch = A.warp_head[gw], next; ch != kEndChunk; ch = next) {
-            next = A.ch_next[ch];  // issued first, so its latency overlaps the chunk's work
-            for (unsigned q = threadIdx.x; q < kEvChunk; q += kTB) {
-                const uint32_t* r = A.evrec + (unsigned long long)ch * kEvChunk + q;
-                const uint32_t j = r[8 * C];
-                if (j == kNoPhoton) continue;
-                ++stored;
-                const uint32_t v = r[0];
-                Photon e;
-                e.ix = (int)(v & 2047u);
-                e.iy = (int)((v >> 11) & 2047u);
-                e.iz = (int)(v >> 22);
-                e.p = make_float3(__uint_as_float(r[C]), __uint_as_float(r[2 * C]), __uint_as_float(r[3 * C]));
-                e.d = make_float3(__uint_as_float(r[4 * C]), __uint_as_float(r[5 * C]), __uint_as_float(r[6 * C]));
-                const uint32_t sw = r[9 * C];  // event number, particle in bit 31
-                const float w = le_adjoint(A, e, __uint_as_float(r[7 * C]), lin_index(A.g, e.ix, e.iy, e.iz),
-                                           TWO && (sw >> 31) != 0u);
-                const uint32_t s = sw & 0x7FFFFFFFu;
-                // event s of photon j: slot evoff[j] + s - 1 (one 16-byte store)
-                reinterpret_cast<uint4*>(A.wseq)[A.evoff[j] + s - 1u] = make_uint4(__float_as_uint(w), v, r[10 * C], 0u);
-                if (w != 0.f) {
-                    atomicAdd(A.wbuf + j, (double)w);
-                    // S_j = sum_{s >= j} w_s vanishes past the photon's last event with w_s != 0,
-                    // so pass 2 stops there (its list and its walks use this in place of the count)
-                    atomicMax(A.nevbuf + j, s);
+        const unsigned idle = __ballot_sync(kFull, left == 0);
+        const int want = __popc(idle);
+        while (qn < want && pending) {  // batches until the queue can fill the idle lanes
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            const uint4 r0 = *reinterpret_cast<const uint4*>(rec + lane * 4);
+            const uint4 r1 = *reinterpret_cast<const uint4*>(rec + (32 + lane) * 4);
+            const uint4 r2 = *reinterpret_cast<const uint4*>(rec + (64 + lane) * 4);
+            const bool on = r2.x != kNoPhoton;
+            Photon e;
+            e.ix = (int)(r0.x & 2047u);
+            e.iy = (int)((r0.x >> 11) & 2047u);
+            e.iz = (int)(r0.x >> 22);
+            e.p = make_float3(__uint_as_float(r0.y), __uint_as_float(r0.z), __uint_as_float(r0.w));
+            e.d = make_float3(__uint_as_float(r1.x), __uint_as_float(r1.y), __uint_as_float(r1.z));
+            const bool air = TWO && (r2.y >> 31) != 0u;
+            const int k = lin_index(A.g, e.ix, e.iy, e.iz);
+            // where the flight began: the previous event, or the launch point
+            uint4 o = make_uint4(0u, 0u, 0u, 0u);
+            float b = 1.f;
+            if (on) {
+                if (r2.w != kNoEvent) o = A.evrec[r2.w];
+                b = BetaFetch<DT>::get(A.beta_pad, pad_index(A.g, e.ix, e.iy, e.iz));
+            }
+            fetch();
+            const float w = on ? le_adjoint(A, e, __uint_as_float(r1.w), k, air) : 0.f;
+            // S: later events first. A batch may hold two events of a photon (rounds of fewer than
+            // 32 while the forward's warp drained): they take turns, the later record first.
+            const unsigned same = __match_any_sync(kFull, r2.x);
+            const int turn = on ? __popc(same & ~(lanemask_lt() | (1u << lane))) : -1;
+            const int turns = __reduce_max_sync(kFull, turn);
+            double S = 0.0;
+            for (int t = 0; t <= turns; ++t) {
+                if (turn == t) {
+                    S = A.wbuf[r2.x];
+                    if (w != 0.f) A.wbuf[r2.x] = S += (double)w;
                 }
+                __syncwarp();
+            }
+            const float Sf = (float)S;
+            const bool go = on && Sf != 0.f;
+            int n = 0;
+            if (on && r2.w == kNoEvent) {
+                Photon l;
+                launch_photon(A, l, r2.x);
+                o = make_uint4((uint32_t)l.ix | ((uint32_t)l.iy << 11) | ((uint32_t)l.iz << 22), __float_as_uint(l.p.x),
+                               __float_as_uint(l.p.y), __float_as_uint(l.p.z));
+            }
+            const int ox = (int)(o.x & 2047u), oy = (int)((o.x >> 11) & 2047u), oz = (int)(o.x >> 22);
+            const uint32_t bin = brick_bin(A.g, (unsigned)e.ix, (unsigned)e.iy, (unsigned)e.iz);
+            if (go) {
+                n = abs(e.ix - ox) + abs(e.iy - oy) + abs(e.iz - oz);
+                // the last voxel: the length there is the stored free path over the extinction
+                const float ib = 1.f / b;
+                float is = ib;  // [aerosol] / beta_aer with two species
+                if constexpr (TWO) is = air ? 0.f : 1.f / __ldg(A.beta_aer + k);
+                atomicAdd(A.gbrk + bin, Sf * (is - __uint_as_float(r2.z) * ib));
+                ++flights;
+                entries += (unsigned)n + 1u;
+            }
+            if (on) ++stored;
+            const unsigned gm = __ballot_sync(kFull, n > 0);
+            if (n > 0) {
+                float3 t, f;
+                score_axis(__uint_as_float(o.y), e.d.x, A.g.hx, t.x, f.x);
+                score_axis(__uint_as_float(o.z), e.d.y, A.g.hy, t.y, f.y);
+                score_axis(__uint_as_float(o.w), e.d.z, A.g.hz, t.z, f.z);
+                const uint32_t fl = (e.d.x < 0.f ? 1u : 0u) | (e.d.y < 0.f ? 2u : 0u) | (e.d.z < 0.f ? 4u : 0u);
+                uint32_t* s = q + (qn + __popc(gm & lanemask_lt()));
+                s[0] = __float_as_uint(t.x);
+                s[1 * kScoreSlots] = __float_as_uint(t.y);
+                s[2 * kScoreSlots] = __float_as_uint(t.z);
+                s[3 * kScoreSlots] = __float_as_uint(f.x);
+                s[4 * kScoreSlots] = __float_as_uint(f.y);
+                s[5 * kScoreSlots] = __float_as_uint(f.z);
+                s[6 * kScoreSlots] = __float_as_uint(-Sf);
+                s[7 * kScoreSlots] = brick_bin(A.g, (unsigned)ox, (unsigned)oy, (unsigned)oz) ^ fl;
+                s[8 * kScoreSlots] = bin ^ fl;
+                s[9 * kScoreSlots] = (uint32_t)n | (fl << 16);
+            }
+            qn += __popc(gm);
+            __syncwarp();
+        }
+        if (qn == 0 && want == 32) break;
+        // refill from the top of the queue
+        if (left == 0) {
+            if (at != goal) ++lost;  // a walk that missed its event's voxel (none in valid use)
+            goal = at;
+            const int slot = qn - 1 - __popc(idle & lanemask_lt());
+            if (slot >= 0) {
+                const uint32_t* s = q + slot;
+                tx = __uint_as_float(s[0]);
+                ty = __uint_as_float(s[1 * kScoreSlots]);
+                tz = __uint_as_float(s[2 * kScoreSlots]);
+                qx = __uint_as_float(s[3 * kScoreSlots]);
+                qy = __uint_as_float(s[4 * kScoreSlots]);
+                qz = __uint_as_float(s[5 * kScoreSlots]);
+                nS = __uint_as_float(s[6 * kScoreSlots]);
+                at = s[7 * kScoreSlots];
+                goal = s[8 * kScoreSlots];
+                const uint32_t nf = s[9 * kScoreSlots];
+                left = (int)(nf & 0xFFFFu);
+                flip = nf >> 16;
+                sx = (flip & 1u ? 0u - 8u : 8u) | 1u;
+                sy = (flip & 2u ? 0u - by8 : by8) | 2u;
+                sz = (flip & 4u ? 0u - bz8 : bz8) | 4u;
             }
         }
+        qn = max(0, qn - want);
+        // K voxels per lane into the strip (entry j of a lane at [j][lane ^ 2j]: neither the writes
+        // nor the transposed reads meet in a bank)
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            uint32_t key = kNoEntry;
+            const float m = fminf(tx, fminf(ty, tz));
+            if (left > 0) {
+                key = at ^ flip;
+                const bool px = tx <= m;
+                const bool py = !px && ty <= m;
+                const uint32_t s = px ? sx : (py ? sy : sz);
+                const bool over = (at & s & 7u) != 0u;
+                at ^= s & 7u;
+                if (over) at += s & ~7u;
+                tx = px ? qx : tx - m;
+                ty = py ? qy : ty - m;
+                tz = (px || py) ? tz - m : qz;
+                --left;
+            }
+            strip[j * 32 + ((lane ^ (2 * j)) & 31)] = make_float2(__uint_as_float(key), nS * m);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const int i = r * 32 + (int)lane, j = i % K, l = i / K;  // entry j of lane l
+            const float2 en = strip[j * 32 + ((l ^ (2 * j)) & 31)];
+            const uint32_t key = __float_as_uint(en.x);
+            if (key < nbins) atomicAdd(A.gbrk + key, en.y);
+        }
+        __syncwarp();
     }
-    stored = warp_sumu(stored);
-    if ((threadIdx.x & 31u) == 0u && stored) atomicAdd(A.stats + MST_ST_EVENTS_STORED, (double)stored);
+    const unsigned long long se = warp_sumu(stored), sf = warp_sumu(flights), sn = warp_sumu(entries), sl = warp_sumu(lost);
+    if (lane == 0u) {
+        if (se) atomicAdd(A.stats + MST_ST_EVENTS_STORED, (double)se);
+        atomicAdd(A.stats + MST_ST_REPLAY_EVENTS, (double)sf);
+        atomicAdd(A.stats + MST_ST_REPLAY_SEGMENTS, (double)sn);
+        atomicAdd(A.stats + MST_ST_REPLAY_SCATTERS, (double)sn);
+        if (sl) atomicAdd(A.stats + MST_ST_LOST, (double)sl);
+    }
 }
 
-template <bool TWO>
-__global__ void __launch_bounds__(kTB) k_event_adjoint(const TransportArgs A) {
-    event_adjoint_run<TWO>(A);
+template <int DT, bool TWO, int K>
+__global__ void __launch_bounds__(kTB, kMinBlocksScore) k_score(const TransportArgs A) {
+    extern __shared__ uint32_t smem[];
+    score_run<DT, TWO, K>(A, smem);
 }
 
-// the batched form: the scenes of a table one after the other (block-uniform)
-template <bool TWO>
-__global__ void __launch_bounds__(kTB) k_event_adjoint_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
+// the batched form: the scenes of a table one after the other
+template <int K>
+__global__ void __launch_bounds__(kTB, kMinBlocksScore)
+    k_score_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
+    extern __shared__ uint32_t smem[];
     for (int s = 0; s < n_scenes; ++s) {
-        event_adjoint_run<TWO>(scenes[s]);
-        __syncthreads();
-    }
-}
-
-// Exclusive prefix sum of the photons' event counts (three passes over tiles of kScanTile):
-// photon j's steps go to wseq[evoff[j] + s - 1], so pass 2 reads each photon's in event order.
-constexpr int kScanPer = 16;                 // consecutive counts per thread
-constexpr int kScanTile = kTB * kScanPer;    // counts per block
-
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t& total) {
-    __shared__ uint32_t wsum[kTB / 32 + 1];
-    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(kFull, incl, o);
-        if (lane >= (unsigned)o) incl += u;
-    }
-    if (lane == 31u) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t x = lane < kTB / 32 ? wsum[lane] : 0u;
-        uint32_t xi = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(kFull, xi, o);
-            if (lane >= (unsigned)o) xi += u;
-        }
-        if (lane < kTB / 32) wsum[lane] = xi - x;  // exclusive offset of each warp
-        if (lane == 31u) wsum[kTB / 32] = xi;      // block total
-    }
-    __syncthreads();
-    total = wsum[kTB / 32];
-    return wsum[warp] + incl - v;
-}
-
-// A thread's kScanPer consecutive counts: four 16-byte loads when all lie below n (lo is a
-// multiple of 16 counts, the array 16-byte aligned), else one by one.
-__device__ __forceinline__ void load_counts(const uint32_t* __restrict__ x, uint32_t n, uint32_t lo,
-                                            uint32_t (&v)[kScanPer]) {
-    static_assert(kScanPer == 16, "four uint4 per thread");
-    if (lo + kScanPer <= n) {
-        const uint4* p = reinterpret_cast<const uint4*>(x + lo);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 u = __ldg(p + q);
-            v[4 * q] = u.x;
-            v[4 * q + 1] = u.y;
-            v[4 * q + 2] = u.z;
-            v[4 * q + 3] = u.w;
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < kScanPer; ++q) v[q] = lo + q < n ? x[lo + q] : 0u;
-    }
-}
-
-__global__ void __launch_bounds__(kTB) k_scan_tiles(const uint32_t* __restrict__ x, uint32_t n,
-                                                    uint32_t* __restrict__ tsum) {
-    const uint32_t lo = blockIdx.x * (uint32_t)kScanTile + threadIdx.x * kScanPer;
-    uint32_t c[kScanPer];
-    load_counts(x, n, lo, c);
-    uint32_t v = 0u;
-#pragma unroll
-    for (int q = 0; q < kScanPer; ++q) v += c[q];
-    uint32_t total = 0u;
-    block_exclusive_scan(v, total);
-    if (threadIdx.x == 0) tsum[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_top(uint32_t* __restrict__ tsum, uint32_t nt) {
-    // one block: exclusive scan of the tile sums in place, ceil(nt / 1024) consecutive per thread
-    __shared__ uint32_t wsum[32];
-    const uint32_t per = (nt + 1023u) / 1024u, lo = threadIdx.x * per;
-    uint32_t v = 0u;
-    for (uint32_t q = 0; q < per; ++q)
-        if (lo + q < nt) v += tsum[lo + q];
-    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t incl = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(kFull, incl, o);
-        if (lane >= (unsigned)o) incl += u;
-    }
-    if (lane == 31u) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t x = wsum[lane];
-        uint32_t xi = x;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(kFull, xi, o);
-            if (lane >= (unsigned)o) xi += u;
-        }
-        wsum[lane] = xi - x;
-    }
-    __syncthreads();
-    uint32_t run = wsum[warp] + incl - v;
-    for (uint32_t q = 0; q < per; ++q)
-        if (lo + q < nt) {
-            const uint32_t t = tsum[lo + q];
-            tsum[lo + q] = run;
-            run += t;
-        }
-}
-
-__global__ void __launch_bounds__(kTB) k_scan_apply(const uint32_t* __restrict__ x, uint32_t n,
-                                                    const uint32_t* __restrict__ tsum, uint32_t* __restrict__ out) {
-    const uint32_t lo = blockIdx.x * (uint32_t)kScanTile + threadIdx.x * kScanPer;
-    uint32_t v[kScanPer], sum = 0u;
-    load_counts(x, n, lo, v);
-#pragma unroll
-    for (int q = 0; q < kScanPer; ++q) sum += v[q];
-    uint32_t total = 0u;
-    uint32_t run = tsum[blockIdx.x] + block_exclusive_scan(sum, total);
-    if (lo + kScanPer <= n) {  // four 16-byte stores
-        uint4* o = reinterpret_cast<uint4*>(out + lo);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint4 u;
-            u.x = run;
-            run += v[4 * q];
-            u.y = run;
-            run += v[4 * q + 1];
-            u.z = run;
-            run += v[4 * q + 2];
-            u.w = run;
-            run += v[4 * q + 3];
-            o[q] = u;
-        }
-    } else {
-#pragma unroll
-        for (int q = 0; q < kScanPer; ++q)
-            if (lo + q < n) {
-                out[lo + q] = run;
-                run += v[q];
-            }
+        score_run<0, false, K>(scenes[s], smem);
+        __syncwarp();
     }
 }
 
@@ -1429,8 +1426,10 @@ __device__ __forceinline__ int score_bin(uint32_t nev) { return (int)min(nev, (u
 
 // Step 1: bin counts cnt[b] over the chunk.
 __global__ void __launch_bounds__(kTB) k_score_hist(const double* __restrict__ W, const uint32_t* __restrict__ nev,
-                                                    uint32_t n, unsigned* __restrict__ cnt) {
+                                                    uint32_t n, unsigned* __restrict__ cnt,
+                                                    const unsigned long long* ev_count, unsigned long long ev_cap) {
     __shared__ unsigned h[kScoreBins];
+    if (ev_cap && *ev_count <= ev_cap) return;  // the score kernel did the replay
     for (int b = threadIdx.x; b < kScoreBins; b += kTB) h[b] = 0u;
     __syncthreads();
     const uint32_t lo = blockIdx.x * kScoreTile, hi = min(lo + (uint32_t)kScoreTile, n);
@@ -1448,8 +1447,10 @@ __global__ void __launch_bounds__(kTB) k_score_hist(const double* __restrict__ W
 __global__ void __launch_bounds__(kTB) k_score_scatter(const double* __restrict__ W, const uint32_t* __restrict__ nev,
                                                        uint32_t n, const unsigned* __restrict__ cnt,
                                                        unsigned* __restrict__ fill, unsigned* __restrict__ total,
-                                                       ScoreRec* __restrict__ list) {
+                                                       ScoreRec* __restrict__ list, const unsigned long long* ev_count,
+                                                       unsigned long long ev_cap) {
     __shared__ unsigned h[kScoreBins], pos[kScoreBins];
+    if (ev_cap && *ev_count <= ev_cap) return;
     for (int b = threadIdx.x; b < kScoreBins; b += kTB) h[b] = 0u;
     __syncthreads();
     const uint32_t lo = blockIdx.x * kScoreTile, hi = min(lo + (uint32_t)kScoreTile, n);
@@ -1516,15 +1517,34 @@ __global__ void k_fold_grad(float* __restrict__ gacc, double* __restrict__ g64, 
     }
 }
 
+// what the score kernel left in its brick tile
+__global__ void k_fold_bricks(float* __restrict__ gbrk, double* __restrict__ g64, const Geo g) {
+    const int nb = brick_bins(g);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
+        const float v = gbrk[i];
+        if (v != 0.f) {
+            int k;
+            if (brick_voxel(g, i, k)) g64[k] += (double)v;
+            gbrk[i] = 0.f;
+        }
+    }
+}
+
 // dynamic shared memory of a transport block: the warps' photon stacks, the forward's tallies
 // and the classic estimate's scratch
 template <int MODE>
 constexpr size_t smem_bytes() {
     constexpr bool REPLAY = MODE >= 2;
     constexpr bool CLASSIC = MODE == kFwdClassic || MODE == kPass1C || MODE == kPass2C;
-    return (size_t)(kTB / 32) * Rec<REPLAY>::NW * kSlots * sizeof(uint32_t) +
+    return (size_t)(kTB / 32) * Rec<MODE>::NW * kSlots * sizeof(uint32_t) +
            (REPLAY ? 0 : (size_t)kTB * 15 * sizeof(uint32_t)) +
            (CLASSIC ? (size_t)(kTB / 32) * kClassicWords * sizeof(uint32_t) : 0);
+}
+
+// the score kernel's: the warps' flight queues and entry strips
+template <int K>
+constexpr size_t score_smem() {
+    return (size_t)(kTB / 32) * score_words<K>() * sizeof(uint32_t);
 }
 
 template <typename K>
@@ -1562,7 +1582,7 @@ cudaError_t launch_trip(const TransportArgs& a, int trip, int blocks, cudaStream
             case 16: return launch_mode<0, MODE, TWO, 16>(a, blocks, st);
             default: return launch_mode<0, MODE, TWO>(a, blocks, st);
         }
-    } else {
+    } else {  // pass 2
         switch (trip) {
             case 4: return launch_mode<0, MODE, TWO, 4>(a, blocks, st);
             case 8: return launch_mode<0, MODE, TWO, 8>(a, blocks, st);
@@ -1578,7 +1598,7 @@ int occupancy_mode(int mode) {
         case kFwdVoxel: return occupancy(k_transport<DT, kFwdVoxel, TWO>, smem_bytes<kFwdVoxel>());
         case kFwdClassic: return occupancy(k_transport<DT, kFwdClassic, TWO>, smem_bytes<kFwdClassic>());
         case kPass2: return occupancy(k_transport<DT, kPass2, TWO>, smem_bytes<kPass2>());
-        case kPass2W: return occupancy(k_transport<DT, kPass2W, TWO>, smem_bytes<kPass2W>());
+        case kScore: return occupancy(k_score<DT, TWO, kStepsScore>, score_smem<kStepsScore>());
         case kPass1C: return occupancy(k_transport<DT, kPass1C, TWO>, smem_bytes<kPass1C>());
         case kPass2C: return occupancy(k_transport<DT, kPass2C, TWO>, smem_bytes<kPass2C>());
         default: return occupancy(k_transport<DT, kPass1, TWO>, smem_bytes<kPass1>());
@@ -1589,14 +1609,12 @@ template <int DT, bool TWO>
 cudaError_t launch_dt(const TransportArgs& a, int mode, int trip, int blocks, cudaStream_t st) {
     if constexpr (DT == 0) {
         if (trip > 0 && mode == kFwdVoxel) return launch_trip<kFwdVoxel, TWO>(a, trip, blocks, st);
-        if (trip > 0 && mode == kPass2W) return launch_trip<kPass2W, TWO>(a, trip, blocks, st);
         if (trip > 0 && mode == kPass2) return launch_trip<kPass2, TWO>(a, trip, blocks, st);
     }
     switch (mode) {
         case kFwdVoxel: return launch_mode<DT, kFwdVoxel, TWO>(a, blocks, st);
         case kFwdClassic: return launch_mode<DT, kFwdClassic, TWO>(a, blocks, st);
         case kPass2: return launch_mode<DT, kPass2, TWO>(a, blocks, st);
-        case kPass2W: return launch_mode<DT, kPass2W, TWO>(a, blocks, st);
         case kPass1C: return launch_mode<DT, kPass1C, TWO>(a, blocks, st);
         case kPass2C: return launch_mode<DT, kPass2C, TWO>(a, blocks, st);
         default: return launch_mode<DT, kPass1, TWO>(a, blocks, st);
@@ -1636,13 +1654,6 @@ cudaError_t launch_transport_batch(const TransportArgs* table, int n, int mode, 
                 case 16: return launch_batch_mode<kFwdVoxel, 16>(table, n, blocks, st);
                 default: return launch_batch_mode<kFwdVoxel>(table, n, blocks, st);
             }
-        case kPass2W:
-            switch (trip) {
-                case 4: return launch_batch_mode<kPass2W, 4>(table, n, blocks, st);
-                case 8: return launch_batch_mode<kPass2W, 8>(table, n, blocks, st);
-                case 10: return launch_batch_mode<kPass2W, 10>(table, n, blocks, st);
-                default: return launch_batch_mode<kPass2W>(table, n, blocks, st);
-            }
         case kPass2: return launch_batch_mode<kPass2>(table, n, blocks, st);
         case kPass1: return launch_batch_mode<kPass1>(table, n, blocks, st);
         default: return cudaErrorInvalidValue;
@@ -1657,10 +1668,10 @@ int transport_batch_blocks_per_sm(int mode) {
         batch_occupancy<kFwdVoxel, 8>();
         batch_occupancy<kFwdVoxel, 10>();
         batch_occupancy<kFwdVoxel, 16>();
-        occ[kPass2W] = batch_occupancy<kPass2W>();
-        batch_occupancy<kPass2W, 4>();
-        batch_occupancy<kPass2W, 8>();
-        batch_occupancy<kPass2W, 10>();
+        occ[kScore] = occupancy(k_score_batch<kStepsScore>, score_smem<kStepsScore>());
+        occupancy(k_score_batch<4>, score_smem<4>());
+        occupancy(k_score_batch<8>, score_smem<8>());
+        occupancy(k_score_batch<10>, score_smem<10>());
         occ[kPass2] = batch_occupancy<kPass2>();
         occ[kPass1] = batch_occupancy<kPass1>();
         ready = true;
@@ -1668,8 +1679,13 @@ int transport_batch_blocks_per_sm(int mode) {
     return mode >= 0 && mode < 7 && occ[mode] > 0 ? occ[mode] : 1;
 }
 
-cudaError_t launch_event_adjoint_batch(const TransportArgs* table, int n, int blocks, cudaStream_t st) {
-    k_event_adjoint_batch<false><<<blocks, kTB, 0, st>>>(table, n);
+cudaError_t launch_score_batch(const TransportArgs* table, int n, int trip, int blocks, cudaStream_t st) {
+    switch (trip) {
+        case 4: k_score_batch<4><<<blocks, kTB, score_smem<4>(), st>>>(table, n); break;
+        case 8: k_score_batch<8><<<blocks, kTB, score_smem<8>(), st>>>(table, n); break;
+        case 10: k_score_batch<10><<<blocks, kTB, score_smem<10>(), st>>>(table, n); break;
+        default: k_score_batch<kStepsScore><<<blocks, kTB, score_smem<kStepsScore>(), st>>>(table, n);
+    }
     return cudaGetLastError();
 }
 
@@ -1693,32 +1709,53 @@ cudaError_t launch_transport(const mst_grid* g, const TransportArgs& a, int dtyp
                       : launch_species<false>(a, dtype, mode, trip, blocks, st);
 }
 
-cudaError_t launch_score_list(const mst_grid* g, uint32_t n, cudaStream_t st) {
+cudaError_t launch_score_list(const mst_grid* g, uint32_t n, bool stored, cudaStream_t st) {
+    const unsigned long long cap = stored ? g->ev_cap : 0ull;
     cudaError_t e = cudaMemsetAsync(g->score_cnt, 0, sizeof(unsigned) * (2 * kScoreBins + 1), st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (n + kScoreTile - 1) / kScoreTile;
     if (blocks == 0u) return cudaSuccess;
-    k_score_hist<<<blocks, kTB, 0, st>>>(g->wbuf, g->nevbuf, n, g->score_cnt);
+    k_score_hist<<<blocks, kTB, 0, st>>>(g->wbuf, g->nevbuf, n, g->score_cnt, g->ev_count, cap);
     k_score_scatter<<<blocks, kTB, 0, st>>>(g->wbuf, g->nevbuf, n, g->score_cnt, g->score_cnt + kScoreBins,
-                                            g->score_cnt + 2 * kScoreBins, g->plist);
+                                            g->score_cnt + 2 * kScoreBins, g->plist, g->ev_count, cap);
     return cudaGetLastError();
 }
 
-cudaError_t launch_event_adjoint(const mst_grid* g, const TransportArgs& a, int dtype, cudaStream_t st) {
-    (void)dtype;
-    if (a.beta_air) k_event_adjoint<true><<<g->sm_count * 8, kTB, 0, st>>>(a);
-    else k_event_adjoint<false><<<g->sm_count * 8, kTB, 0, st>>>(a);
+namespace {
+
+template <int DT, bool TWO, int K>
+cudaError_t launch_score_k(const TransportArgs& a, int blocks, cudaStream_t st) {
+    if constexpr (K != kStepsScore) {  // the default's attributes are set by occupancy()
+        static const int once = occupancy(k_score<DT, TWO, K>, score_smem<K>());
+        (void)once;
+    }
+    k_score<DT, TWO, K><<<blocks, kTB, score_smem<K>(), st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_event_offsets(const mst_grid* g, uint32_t n, cudaStream_t st) {
-    const uint32_t nt = (n + kScanTile - 1) / kScanTile;
-    if (nt == 0u) return cudaSuccess;
-    if (nt > 1024u * 64u) return cudaErrorInvalidValue;  // 2^28 photons; calls that store events hold 2^27
-    uint32_t* tsum = reinterpret_cast<uint32_t*>(g->plist);  // the list is built after the offsets are used
-    k_scan_tiles<<<nt, kTB, 0, st>>>(g->nevbuf, n, tsum);
-    k_scan_top<<<1, 1024, 0, st>>>(tsum, nt);
-    k_scan_apply<<<nt, kTB, 0, st>>>(g->nevbuf, n, tsum, g->evoff);
+template <bool TWO>
+cudaError_t launch_score_dt(const TransportArgs& a, int dtype, int trip, int blocks, cudaStream_t st) {
+    if (dtype == 1) return launch_score_k<1, TWO, kStepsScore>(a, blocks, st);
+    if (dtype == 2) return launch_score_k<2, TWO, kStepsScore>(a, blocks, st);
+    switch (trip) {
+        case 4: return launch_score_k<0, TWO, 4>(a, blocks, st);
+        case 8: return launch_score_k<0, TWO, 8>(a, blocks, st);
+        case 10: return launch_score_k<0, TWO, 10>(a, blocks, st);
+        default: return launch_score_k<0, TWO, kStepsScore>(a, blocks, st);
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, int blocks, cudaStream_t st) {
+    const int trip = g->wf_trip[kScore];
+    return a.beta_air ? launch_score_dt<true>(a, dtype, trip, blocks, st)
+                      : launch_score_dt<false>(a, dtype, trip, blocks, st);
+}
+
+cudaError_t launch_fold_bricks(const mst_grid* g, cudaStream_t st) {
+    const int nb = (brick_bins(g->geo) + 255) / 256;
+    k_fold_bricks<<<nb < 4096 ? nb : 4096, 256, 0, st>>>(g->gbrk, g->g64, g->geo);
     return cudaGetLastError();
 }
 
