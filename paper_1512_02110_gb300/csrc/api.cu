@@ -575,7 +575,9 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         }
         t.ix = iv[0]; t.iy = iv[1]; t.iz = iv[2];
         t.lx = lv[0]; t.ly = lv[1]; t.lz = lv[2];
-        g->cams.pos[c] = {(float)iv[0], (float)iv[1], (float)iv[2], 0.f, lv[0], lv[1], lv[2], 0.f};
+        CamPair& pr = g->cams.pair[c / 2];
+        float2* const to[6] = {&pr.jx, &pr.jy, &pr.jz, &pr.lx, &pr.ly, &pr.lz};
+        for (int a = 0; a < 6; ++a) (c % 2 ? to[a]->y : to[a]->x) = a < 3 ? (float)iv[a] : lv[a - 3];
         t.inside = inside ? 1 : 0;
         t.rx = (float)s.rot[0]; t.ry = (float)s.rot[1]; t.rz = (float)s.rot[2];
         t.ux = (float)s.rot[3]; t.uy = (float)s.rot[4]; t.uz = (float)s.rot[5];

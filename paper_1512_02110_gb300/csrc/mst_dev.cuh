@@ -44,15 +44,14 @@ struct Cam {
     int w, h, pix_off;
 };
 
-// What the local estimates need of a camera, apart and in 16-byte words: (ix, iy, iz) as floats
-// (exact: the centre lies within 1e6 voxels of the grid) and the offset (lx, ly, lz).
-struct __align__(16) CamPos {
-    float jx, jy, jz, pad0;
-    float lx, ly, lz, pad1;
+// What the local estimates need of two cameras, side by side: (ix, iy, iz) as floats (exact: the
+// centre lies within 1e6 voxels of the grid) and the offset (lx, ly, lz).
+struct __align__(16) CamPair {
+    float2 jx, jy, jz, lx, ly, lz;
 };
 
 struct CamSet {
-    CamPos pos[kMaxCams];
+    CamPair pair[kMaxCams / 2];
     int n;
     Cam c[kMaxCams];
 };

@@ -254,15 +254,73 @@ __device__ __forceinline__ int flight_end(const TransportArgs& A, Photon& ph, co
     return kCollided;
 }
 
-// cosine between the photon direction and the direction from the photon to camera c, and the
-// squared distance; r2 = 0 when the photon sits on the centre of projection. `at` holds the
-// photon's voxel indices as floats: whole numbers below 2^24, so the difference to the camera's
-// is exact and needs no conversion per camera.
-__device__ __forceinline__ float cam_cosine(const TransportArgs& A, const Photon& ph, float3 at, const CamPos& cm, float& r2) {
-    const float3 v = make_float3((cm.jx - at.x) * A.g.hx + (cm.lx - ph.p.x), (cm.jy - at.y) * A.g.hy + (cm.ly - ph.p.y),
-                                 (cm.jz - at.z) * A.g.hz + (cm.lz - ph.p.z));
-    r2 = v.x * v.x + v.y * v.y + v.z * v.z;
-    return r2 > 0.f ? (ph.d.x * v.x + ph.d.y * v.y + ph.d.z * v.z) * rsqrtf(r2) : 0.f;
+// Two FP32 numbers in one 64-bit register: sm_100's packed add, multiply and fused multiply-add take
+// one issue slot for both, each rounded as the scalar operation.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2(float2 a) { return f2(a.x, a.y); }
+__device__ __forceinline__ void split(F2 a, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v)); }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+// 1 / sqrt of numbers known to be normal (or of one whose result is not used): no scaling around the unit
+__device__ __forceinline__ float rsqrt_normal(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The event side of the local estimates, each value twice: minus the voxel indices (as floats: whole
+// numbers below 2^24, so the difference to a camera's is exact) and the offset, the direction, and
+// the voxel size.
+struct EventPair {
+    F2 nx, ny, nz, npx, npy, npz, dx, dy, dz;
+    __device__ __forceinline__ EventPair(const Photon& e)
+        : nx(f2(-(float)e.ix, -(float)e.ix)), ny(f2(-(float)e.iy, -(float)e.iy)), nz(f2(-(float)e.iz, -(float)e.iz)),
+          npx(f2(-e.p.x, -e.p.x)), npy(f2(-e.p.y, -e.p.y)), npz(f2(-e.p.z, -e.p.z)), dx(f2(e.d.x, e.d.x)),
+          dy(f2(e.d.y, e.d.y)), dz(f2(e.d.z, e.d.z)) {}
+};
+
+// Phase function of the event's particle toward two cameras: Rayleigh (Eq. Pray) for air, HG (Eq.
+// Phg) otherwise, of the cosine between the photon's direction and the direction from it to the
+// camera. ok: false when the photon sits on the centre of projection (within 1e-19 m: a squared
+// distance without a normal FP32 value).
+template <bool AIR>
+__device__ __forceinline__ F2 phase_pair(const TransportArgs& A, const EventPair& e, const CamPair& c, bool& ok0, bool& ok1) {
+    const F2 vx = fma2(f2(c.jx) + e.nx, f2(A.g.hx, A.g.hx), f2(c.lx) + e.npx);
+    const F2 vy = fma2(f2(c.jy) + e.ny, f2(A.g.hy, A.g.hy), f2(c.ly) + e.npy);
+    const F2 vz = fma2(f2(c.jz) + e.nz, f2(A.g.hz, A.g.hz), f2(c.lz) + e.npz);
+    float r0, r1;
+    split(fma2(vz, vz, fma2(vx, vx, vy * vy)), r0, r1);
+    ok0 = r0 >= 1.17549435e-38f;
+    ok1 = r1 >= 1.17549435e-38f;
+    const F2 mu = fma2(e.dz, vz, fma2(e.dx, vx, e.dy * vy)) * f2(rsqrt_normal(r0), rsqrt_normal(r1));
+    if constexpr (AIR) {
+        return f2(0.05968310365946075f, 0.05968310365946075f) * fma2(mu, mu, f2(1.f, 1.f));
+    } else {
+        // 1 + g^2 - 2 g mu: FP32 numbers near 2 leave no subnormal difference
+        split(fma2(f2(-A.hg.b, -A.hg.b), mu, f2(A.hg.a, A.hg.a)), r0, r1);
+        const F2 r = f2(rsqrt_normal(r0), rsqrt_normal(r1));
+        return f2(A.hg.k1, A.hg.k1) * r * r * r;
+    }
 }
 
 // Step iv with two species (Sec. 2): the event's particle is air with probability
@@ -279,34 +337,22 @@ __device__ __forceinline__ bool particle_is_air(const TransportArgs& A, uint4 x,
     return (double)u * (ba + (double)__ldg(A.beta_aer + k)) < ba;
 }
 
-// phase function of the event's particle: Rayleigh (Eq. Pray) for air, HG (Eq. Phg) otherwise.
-// The local estimates take the particle as a template parameter, so the one-species code keeps
-// no per-camera select.
-template <bool AIR>
-__device__ __forceinline__ float phase_of(const TransportArgs& A, float mu) {
-    if constexpr (AIR) return rayleigh_phase(mu);
-    else return hg_phase(A.hg, mu);
-}
-
 // Eq. Lcupdate: L_c(k) += albedo I_s P(angle between the incoming ray and X_c - X_s), for all
 // cameras at once, four cameras per vector atomic into the [nvox][cp] FP32 tile.
 template <bool AIR>
 __device__ __forceinline__ void le_voxel_p(const TransportArgs& A, const Photon& ph, float w, int k) {
     float* row = A.Lacc + (size_t)k * A.cp;
-    const float3 at = make_float3((float)ph.ix, (float)ph.iy, (float)ph.iz);
-#pragma unroll 1  // (unrolled, the forward outgrows the instruction cache: 38.1 -> 41.9 ms)
+    const EventPair e(ph);
+    const F2 w2 = f2(w, w);
+#pragma unroll 1  // (unrolled over 9 cameras, the forward outgrows the instruction cache: 38.1 -> 41.9 ms)
     for (int q = 0; 4 * q < A.cams.n; ++q) {
         float v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = 4 * q + j;
-            float val = 0.f;
-            if (c < A.cams.n) {
-                float r2;
-                const float mu = cam_cosine(A, ph, at, A.cams.pos[c], r2);
-                if (r2 > 0.f) val = w * phase_of<AIR>(A, mu);
-            }
-            v[j] = val;
+        for (int j = 0; j < 2; ++j) {
+            bool ok0, ok1;
+            split(w2 * phase_pair<AIR>(A, e, A.cams.pair[2 * q + j], ok0, ok1), v[2 * j], v[2 * j + 1]);
+            v[2 * j] = ok0 && 4 * q + 2 * j < A.cams.n ? v[2 * j] : 0.f;
+            v[2 * j + 1] = ok1 && 4 * q + 2 * j + 1 < A.cams.n ? v[2 * j + 1] : 0.f;
         }
         atomicAdd(reinterpret_cast<float4*>(row + 4 * q), make_float4(v[0], v[1], v[2], v[3]));
     }
@@ -321,21 +367,20 @@ __device__ __forceinline__ void le_voxel(const TransportArgs& A, const Photon& p
 template <bool AIR>
 __device__ __forceinline__ float le_adjoint_p(const TransportArgs& A, const Photon& ph, float w, int k) {
     const float4* row = reinterpret_cast<const float4*>(A.adj + (size_t)k * A.cp);
-    const float3 at = make_float3((float)ph.ix, (float)ph.iy, (float)ph.iz);
+    const EventPair e(ph);
+    const F2 w2 = f2(w, w);
     float acc = 0.f;
+    auto two = [&](int pair, float a0, float a1) {  // (the padding's a is 0)
+        bool ok0, ok1;
+        float v0, v1;
+        split(f2(a0, a1) * w2 * phase_pair<AIR>(A, e, A.cams.pair[pair], ok0, ok1), v0, v1);
+        acc += ok0 && a0 != 0.f ? v0 : 0.f;
+        acc += ok1 && a1 != 0.f ? v1 : 0.f;
+    };
     auto group = [&](int q) {
         const float4 a4 = __ldg(row + q);
-        const float aa[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = 4 * q + j;
-            if (c < A.cams.n) {
-                float r2;
-                const float mu = cam_cosine(A, ph, at, A.cams.pos[c], r2);
-                const float v = aa[j] * w * phase_of<AIR>(A, mu);
-                acc += aa[j] != 0.f && r2 > 0.f ? v : 0.f;
-            }
-        }
+        two(2 * q, a4.x, a4.y);
+        if (4 * q + 2 < A.cams.n) two(2 * q + 1, a4.z, a4.w);
     };
     // the first groups unrolled: their cameras' constants are operands of the arithmetic then
     // instead of loads (score of 3.7e8 events with 9 cameras: 20.8 -> 19.5 ms)
@@ -588,13 +633,24 @@ __device__ __forceinline__ int after_event(const TransportArgs& A, Photon& ph, T
     return 0;
 }
 
+// Debug outputs: a photon's path checksum and the point of its last event (or launch).
+__device__ __forceinline__ uint32_t end_hash(uint32_t hash, uint32_t s, int term) {
+    return (((hash ^ s) * kFnvPrime) ^ (uint32_t)term) * kFnvPrime;
+}
+
+__device__ __forceinline__ void write_point(const TransportArgs& A, const Photon& ph) {
+    A.point[ph.idx] = make_float4(ph.p.x, ph.p.y, ph.p.z,
+                                  __uint_as_float((uint32_t)ph.ix | ((uint32_t)ph.iy << 11) | ((uint32_t)ph.iz << 22)));
+}
+
 __device__ __forceinline__ void finish_photon(const TransportArgs& A, const Photon& ph, int term) {
-    uint32_t h = (ph.hash ^ ph.s) * kFnvPrime;
-    h = (h ^ (uint32_t)term) * kFnvPrime;
-    if (A.hash) A.hash[ph.idx] = h;
-    if (A.point)
-        A.point[ph.idx] = make_float4(ph.p.x, ph.p.y, ph.p.z,
-                                      __uint_as_float((uint32_t)ph.ix | ((uint32_t)ph.iy << 11) | ((uint32_t)ph.iz << 22)));
+    if (A.hash) A.hash[ph.idx] = end_hash(ph.hash, ph.s, term);
+    if (A.point) write_point(A, ph);
+}
+
+// the forward keeps the running checksum in the output itself
+__device__ __forceinline__ void finish_hash(const TransportArgs& A, uint32_t idx, uint32_t s, int term) {
+    A.hash[idx] = end_hash(A.hash[idx], s, term);
 }
 
 // One stored event (forward, full gradient), three 16-byte words: where it happened; the incoming
@@ -634,10 +690,27 @@ constexpr uint32_t kNoEvent = 0xFFFFFFFFu;   // previous record of a photon's fi
 constexpr int kSlots = 64;
 // Voxels a flying lane advances per loop trip, and minimum resident blocks per SM (register
 // budget), per kernel mode; set from sweeps on the 64^3 cumulus workload.
-constexpr int kStepsForward = 12;
+#ifndef KSF
+#define KSF 8
+#endif
+constexpr int kStepsForward = KSF;
 constexpr int kStepsPass1 = 8;
 constexpr int kStepsPass2 = 6;
-constexpr int kMinBlocksForward = 3;
+#ifndef MBF
+#define MBF 3
+#endif
+#ifndef KSF
+#define KSF 8
+#endif
+#ifndef KDR
+#define KDR 1
+#endif
+constexpr int kDrain = KDR;
+#ifndef LFR
+#define LFR 16
+#endif
+constexpr int kLaunchFrom = LFR;
+constexpr int kMinBlocksForward = MBF;
 constexpr int kMinBlocksClassic = 3;
 constexpr int kMinBlocksPass1 = 3;
 constexpr int kMinBlocksPass2 = 3;
@@ -655,10 +728,10 @@ struct Stack {
     int cap;
 };
 
-// words of a stack slot: the photon; the forward's previous record, or a replay's event count and sum
+// words of a stack slot: the photon, and a replay's event count and sum
 template <int MODE>
 struct Rec {
-    static constexpr int NW = MODE >= kPass2 ? 15 : (MODE == kFwdVoxel ? 13 : 12);
+    static constexpr int NW = MODE >= kPass2 ? 15 : 12;
 };
 
 template <int NW>
@@ -677,8 +750,8 @@ __device__ __forceinline__ void put(const Stack<NW>& q, int slot, const Photon& 
     b[9 * c] = ph.s;
     b[10 * c] = ph.hash;
     b[11 * c] = ph.idx;
-    if (NW > 12) b[12 * c] = nev;
-    if (NW > 13) {
+    if (NW > 12) {
+        b[12 * c] = nev;
         b[13 * c] = (uint32_t)__double_as_longlong(acc);
         b[14 * c] = (uint32_t)((unsigned long long)__double_as_longlong(acc) >> 32);
     }
@@ -701,10 +774,11 @@ __device__ __forceinline__ void get(const Stack<NW>& q, int slot, const Transpor
     ph.hash = b[10 * c];
     ph.idx = b[11 * c];
     ph.id = A.first_id + (ph.idx - A.out_base);
-    nev = NW > 12 ? b[12 * c] : 0u;
-    if (NW > 13) {
+    if (NW > 12) {
+        nev = b[12 * c];
         acc = __longlong_as_double((long long)((unsigned long long)b[13 * c] | ((unsigned long long)b[14 * c] << 32)));
     } else {
+        nev = 0u;
         acc = 0.0;
     }
 }
@@ -738,10 +812,13 @@ __device__ __forceinline__ void fold_slice(const TransportArgs& A, uint32_t batc
         if (A.fold_bins == 0u) return;
         const uint64_t i0 = (uint64_t)(batch % A.fold_nslices) * A.fold_slice;
         const uint64_t i1 = min(i0 + A.fold_slice, A.fold_bins);
+        const uint64_t k0 = MODE == kFwdVoxel ? i0 / (uint32_t)A.cp : 0u;  // the slice's first row
+        const uint32_t o0 = (uint32_t)(i0 - k0 * (uint32_t)A.cp);
         for (uint64_t i = i0 + lane; i < i1; i += 32) {
             if (MODE == kFwdVoxel) {  // L tile [nvox][cp] -> L64 [C][nvox]
-                const uint64_t k = i / (uint32_t)A.cp;
-                const int c = (int)(i - k * (uint32_t)A.cp);
+                const uint32_t o = o0 + (uint32_t)(i - i0), row = o / (uint32_t)A.cp;
+                const uint64_t k = k0 + row;
+                const int c = (int)(o - row * (uint32_t)A.cp);
                 if (c < A.cams.n) {
                     const float v = atomicExch(A.Lacc + i, 0.f);
                     if (v != 0.f) atomicAdd(A.L64 + (size_t)c * A.g.nvox + k, (double)v);
@@ -854,9 +931,6 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     const unsigned warp = threadIdx.x >> 5;
     const Stack<NW> stk{smem + warp * NW * kSlots, kSlots};  // events at slot i, ready photons at kSlots-1-i
     int ev_n = 0, rd_n = 0;  // warp-uniform stack heights
-    unsigned long long ch_base = ~0ull;  // forward storing events: the warp's current chunk (none yet) ...
-    unsigned ch_fill = kEvChunk;         // ... and its slots in use
-    const uint32_t gwarp = blockIdx.x * (kTB / 32) + warp;  // the warp's chunk list
 
     // photon tallies: forward render only, one shared-memory slot per thread after the stacks
     typename std::conditional<REPLAY, NoTally, LaneTally>::type t;
@@ -882,7 +956,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     Photon ph;
     Flight w;
     float tau = 0.f;
-    uint32_t nev = 0u;  // pass 2: events of pass 1; forward: the photon's last record
+    uint32_t nev = 0u;  // pass 2: events of pass 1
     double acc = 0.0;   // pass 1: W; pass 2: S
     bool fly = false, dry = false;
     uint32_t wbase = 0u, wend = 0u;
@@ -909,7 +983,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
         }
         refill(A, pool_n, fly, dry, wbase, wend, lane, [&](uint32_t j) -> bool {
             uint32_t pid = j;
-            nev = MODE == kFwdVoxel ? kNoEvent : 0u;
+            nev = 0u;
             acc = 0.0;
             if (PASS2) {  // item j of the pass-1 list
                 const ScoreRec r = A.plist[j];
@@ -949,7 +1023,6 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             if (stop) {
                 r = flight_end<TWO>(A, ph, w, tau, b, S, scatters);
                 if (r >= 0) --nstep;  // the halo voxel is no segment of the path
-                if (MODE == kFwdVoxel && r == kCollided) ph.tau = tau;  // kept for the stored event
             }
             segments += nstep;
             // a flight longer than any straight walk through the grid is abandoned
@@ -984,28 +1057,6 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             uint32_t enev = 0u;
             double eacc = 0.0;
             int term = -1;  // -1 idle lane, 0 goes on, > 0 ended
-            unsigned long long ev_slot = 0ull;  // forward storing events: this lane's record slot
-            if (MODE == kFwdVoxel && A.ev_cap) {
-                // the round's slots continue the warp's chunk and spill into a new one
-                unsigned long long nb = 0ull;
-                if (ch_fill + (unsigned)n > kEvChunk) {  // a new chunk, linked to the warp's last one
-                    if (lane == 0u) {
-                        nb = atomicAdd(A.ev_count, (unsigned long long)kEvChunk);
-                        // (a chunk past the buffer is not linked: the call then replays instead)
-                        if (nb + kEvChunk <= A.ev_cap)
-                            A.ch_prev[nb / kEvChunk] = ch_base == ~0ull ? kEndChunk : (uint32_t)(ch_base / kEvChunk);
-                    }
-                    nb = __shfl_sync(kFull, nb, 0);
-                }
-                const unsigned f = ch_fill + lane;
-                ev_slot = f < kEvChunk ? ch_base + f : nb + (f - kEvChunk);
-                if (ch_fill + (unsigned)n > kEvChunk) {
-                    ch_base = nb;
-                    ch_fill = ch_fill + (unsigned)n - kEvChunk;
-                } else {
-                    ch_fill += (unsigned)n;
-                }
-            }
             if constexpr (CLASSIC) {
                 // the classic estimate runs on the whole warp (its shadow rays are spread over all
                 // lanes), between the event's per-lane first half and its second
@@ -1053,7 +1104,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                         term = e.s == enev ? 1 : after_event<TWO>(A, e, t, air, xb);  // stop at pass 1's last event
                     }
                 }
-            } else {  // the voxelised estimate (or the stored w_s), per lane
+            } else {  // the voxelised estimate's replay, per lane
                 if ((int)lane < n) {
                     get(stk, ev_n - 1 - (int)lane, A, e, enev, eacc);
                     e.s += 1u;
@@ -1069,15 +1120,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                     }
                     if (air) air_events.add();
                     const float wgt = (air ? A.albedo_air : A.albedo) * e.I;
-                    if (!REPLAY) {
-                        e.hash = (e.hash ^ (uint32_t)k) * kFnvPrime;
-                        if (MODE == kFwdVoxel && A.ev_cap && ev_slot < A.ev_cap) store_event(A, ev_slot, e, wgt, air, enev);
-                        if (MODE == kFwdVoxel) enev = (uint32_t)ev_slot;
-                        le_voxel(A, e, wgt, k, air);
-                        if constexpr (TWO) xb = unstash_block(stk, slot);
-                        term = after_event<TWO>(A, e, t, air, xb);
-                        if (term) finish_photon(A, e, term);
-                    } else {
+                    {
                         const float we = le_adjoint(A, e, wgt, k, air);
                         if (PASS1) {
                             eacc += (double)we;
@@ -1126,12 +1169,6 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     } else {
         flush_tally(A, t.load(), segments, events, lane);
         air_events.flush(A.stats + MST_ST_AIR_EVENTS, lane);
-        if (MODE == kFwdVoxel && A.ev_cap) {  // the warp's last chunk; its tail holds no event
-            if (lane == 0u) A.warp_tail[gwarp] = ch_base == ~0ull ? kEndChunk : (uint32_t)(ch_base / kEvChunk);
-            if (ch_base != ~0ull)
-                for (unsigned f = ch_fill + lane; f < kEvChunk; f += 32u)
-                    if (ch_base + f < A.ev_cap) A.evrec[2ull * A.ev_cap + ch_base + f].x = kNoPhoton;
-        }
     }
 }
 
@@ -1150,6 +1187,407 @@ __global__ void __launch_bounds__(kTB, min_blocks(MODE))
     extern __shared__ uint32_t smem[];
     for (int s = 0; s < n_scenes; ++s) {
         transport_run<DT, MODE, TWO, TRIP>(scenes[s], smem);
+        __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// The forward render with the voxelised local estimate. A warp owns kSlots photons, each in a slot of
+// shared memory for its whole life; lanes walk flights and hold nothing of a photon but its walk.
+// Every loop trip (1) launches new photons into free slots when the ready queue runs short, (2) hands
+// ready photons to idle lanes, (3) walks every flight by up to TRIP voxels, queueing flights that
+// ended in a collision and putting aside those that left the grid, and (4) takes 32 queued
+// collisions at once through their event: collision point, record, local estimates, albedo,
+// roulette, new direction and the set-up of the next flight, which makes the photon ready again.
+//
+// A flight is set up and ended where all 32 lanes have one in hand; a lane that begins one only
+// loads its walk and stores five words when it ends. (Both used to happen in the walking lanes, ten
+// of 32 at a time: 40 % of the kernel's warp instructions, and with a whole photon held in
+// registers across the walk.)
+
+// words of a slot: direction (3), weight, events so far, position in the call, previous record, then
+// the flight: t (3), free path, padded index, and q (3) while it is ready, the extinction of the
+// collision voxel in the fourth word of the walk when it has ended
+constexpr int kSlotWords = 15;
+constexpr int kSD = 0, kSI = 3, kSs = 4, kSIdx = 5, kSPrev = 6, kST = 7, kSTau = 10, kSLin = 11, kSQ = 12;
+constexpr int kEscSlots = 64;  // flights out of the grid a warp puts aside
+
+// shared words per warp: the tallies (FP64), slots, escapes (weight, padded index), and the queues
+// of slot numbers
+constexpr int kFwdWords = 2 * MST_NSTATS + kSlotWords * kSlots + 2 * kEscSlots + 3 * kSlots / 4;
+static_assert(kFwdWords % 2 == 0, "the tallies are FP64");
+
+// One axis of a flight as flight_axis sets it up, without its branches; q carries the direction's
+// sign. An axis the flight does not move along keeps its offset in q (t = +inf: q is never used there).
+__device__ __forceinline__ void ready_axis(float p0, float d, float h, float& t, float& q) {
+    const float p = fminf(fmaxf(p0, 0.f), h);
+    const float inv = __fdividef(1.f, fabsf(d));
+    const float u = (d > 0.f ? h - p : p) * inv;
+    t = d == 0.f ? CUDART_INF_F : u;
+    q = d == 0.f ? p0 : copysignf(h * inv, d);
+}
+
+// What an event adds to the forward's tallies; rare: one of the last four may be set.
+struct EventTally {
+    float absorbed = 0.f, killed = 0.f, gained = 0.f, forced = 0.f, capped = 0.f;
+    bool rare = false;
+    __device__ __forceinline__ void add_absorbed(float v) { absorbed = v; }
+    __device__ __forceinline__ void add_killed(float v) { killed = v; rare = true; }
+    __device__ __forceinline__ void add_gained(float v) { gained = v; rare = true; }
+    __device__ __forceinline__ void add_forced(float v) { forced = v; rare = true; }
+    __device__ __forceinline__ void add_capped() { capped = 1.f; rare = true; }
+};
+
+template <int DT, bool TWO, int TRIP>
+__device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* smem) {
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    double* tally = reinterpret_cast<double*>(smem + warp * kFwdWords);    // the warp's share of the statistics
+    uint32_t* sl = smem + warp * kFwdWords + 2 * MST_NSTATS;               // word f of slot i at sl[f * kSlots + i]
+    uint32_t* esc = sl + kSlotWords * kSlots;
+    uint8_t* evq = reinterpret_cast<uint8_t*>(esc + 2 * kEscSlots);  // slots of ended flights
+    uint8_t* rdq = evq + kSlots;                                     // of ready photons
+    uint8_t* frq = rdq + kSlots;                                     // of no photon
+    const uint32_t gwarp = blockIdx.x * (kTB / 32) + warp;           // the warp's chunk list
+    for (int i = (int)lane; i < MST_NSTATS; i += 32) tally[i] = 0.0;
+    // adds the lanes' values to a statistic of the warp (nothing when all are 0)
+    auto add_tally = [&](int which, float v) {
+        if (__any_sync(kFull, v != 0.f)) {
+            v = warp_sumf(v);
+            if (lane == 0u) tally[which] += (double)v;
+        }
+    };
+    for (int i = (int)lane; i < kSlots; i += 32) frq[i] = (uint8_t)i;
+    __syncwarp();
+
+    int ev_n = 0, rd_n = 0, fr_n = kSlots, esc_n = 0;  // warp-uniform queue lengths
+    unsigned long long ch_base = ~0ull;                // forward storing events: the warp's current chunk (none yet) ...
+    unsigned ch_fill = kEvChunk;                       // ... and its slots in use
+    uint32_t wbase = 0u, wend = 0u;                    // photons of the warp's ticket batch not launched yet
+    bool dry = false;
+    unsigned segments = 0u, events = 0u, launched = 0u, escaped = 0u;
+    EventCount<TWO> air_events;
+
+    // the lane's flight
+    float tx = 0.f, ty = 0.f, tz = 0.f, qx = 0.f, qy = 0.f, qz = 0.f, tau = 0.f, bn = 0.f;
+    int dx = 0, dy = 0, dz = 0, lin = 0, left = 0;
+    int slot = -1;  // its photon's slot; -1: no flight
+
+    // a photon in slot i is ready for the flight from offset p of voxel (ix, iy, iz) along d
+    auto make_ready = [&](int i, float3 p, float3 d, int ix, int iy, int iz, float free_path) {
+        uint32_t* s = sl + i;
+        float3 tt, qq;
+        ready_axis(p.x, d.x, A.g.hx, tt.x, qq.x);
+        ready_axis(p.y, d.y, A.g.hy, tt.y, qq.y);
+        ready_axis(p.z, d.z, A.g.hz, tt.z, qq.z);
+        s[(kSD + 0) * kSlots] = __float_as_uint(d.x);
+        s[(kSD + 1) * kSlots] = __float_as_uint(d.y);
+        s[(kSD + 2) * kSlots] = __float_as_uint(d.z);
+        s[(kST + 0) * kSlots] = __float_as_uint(tt.x);
+        s[(kST + 1) * kSlots] = __float_as_uint(tt.y);
+        s[(kST + 2) * kSlots] = __float_as_uint(tt.z);
+        s[kSTau * kSlots] = __float_as_uint(free_path);
+        s[kSLin * kSlots] = (uint32_t)pad_index(A.g, ix, iy, iz);
+        s[(kSQ + 0) * kSlots] = __float_as_uint(qq.x);
+        s[(kSQ + 1) * kSlots] = __float_as_uint(qq.y);
+        s[(kSQ + 2) * kSlots] = __float_as_uint(qq.z);
+    };
+    // tallies of up to 32 flights that left the grid, from the end of their queue
+    auto count_escapes = [&](int n) {
+        int face = -1;
+        float I = 0.f;
+        if ((int)lane < n) {
+            const int i = esc_n - 1 - (int)lane;
+            const int at = (int)esc[kEscSlots + i];
+            I = __uint_as_float(esc[i]);
+            face = at < 0 ? kWalkOverflow : halo_face(A.g, at);
+            if (face < kWalkOverflow) ++escaped;
+        }
+#pragma unroll
+        for (int f = 0; f < 6; ++f) add_tally(MST_ST_ESC_XM + f, face == f ? I : 0.f);
+        add_tally(MST_ST_LOST, face == kWalkOverflow ? 1.f : 0.f);
+        esc_n -= n;
+        __syncwarp();
+    };
+    uint32_t fly = 0u;  // lanes with a flight
+
+    for (;;) {
+        const uint32_t idle = ~fly;
+        // (1) launch (a few dozen at a time, so that the launch runs with most lanes)
+        while (rd_n < __popc(idle) && !dry && (fr_n >= kLaunchFrom || (rd_n == 0 && fly == 0u && ev_n == 0))) {
+            if (wbase >= wend) {
+                unsigned t0 = 0u;
+                if (lane == 0u) t0 = atomicAdd(A.ticket, (unsigned)kTicketBatch);
+                t0 = __shfl_sync(kFull, t0, 0);
+                if (t0 >= A.n) {
+                    dry = true;
+                    break;
+                }
+                wbase = t0;
+                wend = min(t0 + (unsigned)kTicketBatch, A.n);
+                fold_slice<kFwdVoxel>(A, t0 / (uint32_t)kTicketBatch, lane);
+            }
+            const int n = min(min(32, fr_n), (int)(wend - wbase));
+            bool in = false;
+            int i = 0;
+            if ((int)lane < n) {
+                const uint32_t j = wbase + lane;
+                if (A.skip && A.skip[A.out_base + j]) {
+                    if (A.hash) A.hash[A.out_base + j] = 0u;
+                } else {
+                    in = true;
+                    i = frq[fr_n - 1 - (int)lane];
+                    Photon ph;
+                    launch_photon(A, ph, j);
+                    make_ready(i, ph.p, ph.d, ph.ix, ph.iy, ph.iz, ph.tau);
+                    uint32_t* s = sl + i;
+                    s[kSI * kSlots] = __float_as_uint(ph.I);
+                    s[kSs * kSlots] = 0u;
+                    s[kSIdx * kSlots] = ph.idx;
+                    s[kSPrev * kSlots] = kNoEvent;
+                    if (A.hash) A.hash[ph.idx] = kFnvOffset;
+                    if (A.point) write_point(A, ph);
+                    ++launched;
+                }
+            }
+            wbase += (uint32_t)n;
+            // skipped photons give their slots back: the launched ones are packed to the top
+            const unsigned im = __ballot_sync(kFull, in);
+            const unsigned sm = __ballot_sync(kFull, (int)lane < n && !in);
+            const int back = (int)lane < n && !in ? frq[fr_n - 1 - (int)lane] : 0;
+            __syncwarp();
+            if (in) rdq[rd_n + __popc(im & lanemask_lt())] = (uint8_t)i;
+            if ((int)lane < n && !in) frq[fr_n - n + __popc(sm & lanemask_lt())] = (uint8_t)back;
+            rd_n += __popc(im);
+            fr_n += __popc(sm) - n;
+            __syncwarp();
+        }
+        // (2) ready photons to idle lanes
+        if (slot < 0) {
+            const int r = rd_n - 1 - __popc(idle & lanemask_lt());
+            if (r >= 0) {
+                slot = rdq[r];
+                const uint32_t* s = sl + slot;
+                tx = __uint_as_float(s[(kST + 0) * kSlots]);
+                ty = __uint_as_float(s[(kST + 1) * kSlots]);
+                tz = __uint_as_float(s[(kST + 2) * kSlots]);
+                const uint32_t ux = s[(kSQ + 0) * kSlots], uy = s[(kSQ + 1) * kSlots], uz = s[(kSQ + 2) * kSlots];
+                qx = fabsf(__uint_as_float(ux));
+                qy = fabsf(__uint_as_float(uy));
+                qz = fabsf(__uint_as_float(uz));
+                tau = __uint_as_float(s[kSTau * kSlots]);
+                lin = (int)s[kSLin * kSlots];
+                // the sign says which way (an axis without motion is never crossed)
+                dx = (int)ux < 0 ? -1 : 1;
+                dy = (int)uy < 0 ? -A.g.p0 : A.g.p0;
+                dz = (int)uz < 0 ? -A.g.p01 : A.g.p01;
+                bn = BetaFetch<DT>::get(A.beta_pad, lin);
+                left = A.g.max_steps;
+            }
+        }
+        const int took = min(rd_n, __popc(idle));
+        rd_n -= took;
+        fly = __ballot_sync(kFull, slot >= 0);
+        if (fly == 0u && ev_n == 0) break;  // (dry: a warp without flights has launched what it could)
+
+        // (3) up to TRIP voxels for every flight (see flight_step)
+        bool hit = false, out = false;
+        float b = 0.f;
+        if (slot >= 0) {
+            int n = 0;
+#pragma unroll 1
+            while (n < TRIP) {
+                ++n;
+                b = bn;
+                const float m = fminf(tx, fminf(ty, tz));
+                const bool px = tx <= m;
+                const bool py = !px && ty <= m;
+                const int next = lin + (px ? dx : (py ? dy : dz));
+                bn = BetaFetch<DT>::get(A.beta_pad, next);
+                const float bs = __fmul_rn(b, m);
+                if (!(tau > bs)) {
+                    hit = true;
+                    break;
+                }
+                tau -= bs;
+                tx = px ? qx : tx - m;
+                ty = py ? qy : ty - m;
+                tz = (px || py) ? tz - m : qz;
+                lin = next;
+            }
+            out = hit && isinf(b);
+            if (out) {
+                hit = false;
+                --n;  // the halo voxel is no segment of the path
+            }
+            segments += n;
+            left -= n;
+            if (!hit && !out && left < 0) {  // longer than any straight walk through the grid
+                out = true;
+                lin = -1;
+            }
+        }
+        const unsigned hm = __ballot_sync(kFull, hit), om = __ballot_sync(kFull, out);
+        if (hit) {
+            uint32_t* s = sl + slot;
+            s[(kST + 0) * kSlots] = __float_as_uint(tx);
+            s[(kST + 1) * kSlots] = __float_as_uint(ty);
+            s[(kST + 2) * kSlots] = __float_as_uint(tz);
+            s[kSTau * kSlots] = __float_as_uint(tau);
+            s[kSLin * kSlots] = (uint32_t)lin;
+            evq[ev_n + __popc(hm & lanemask_lt())] = (uint8_t)slot;
+            slot = -1;
+        }
+        ev_n += __popc(hm);
+        fly &= ~(hm | om);
+        if (om) {
+            if (out) {
+                const int r = __popc(om & lanemask_lt());
+                esc[esc_n + r] = sl[kSI * kSlots + slot];
+                esc[kEscSlots + esc_n + r] = (uint32_t)lin;
+                frq[fr_n + r] = (uint8_t)slot;
+                if (A.hash) finish_hash(A, sl[kSIdx * kSlots + slot], sl[kSs * kSlots + slot], 1);
+                slot = -1;
+            }
+            esc_n += __popc(om);
+            fr_n += __popc(om);
+            __syncwarp();
+            if (esc_n > kEscSlots - 32) count_escapes(32);
+        }
+        __syncwarp();
+
+        const int fly_n = __popc(fly);
+        // (4) events, 32 at a time; while the warp drains, whatever is queued as soon as no photon is ready
+        while (ev_n >= 32 || (ev_n > 0 && dry && rd_n == 0 && fly_n <= kDrain * ev_n)) {
+            const int n = min(32, ev_n);
+            unsigned long long ev_slot = 0ull;  // storing events: this lane's record slot
+            if (A.ev_cap) {
+                // the round's slots continue the warp's chunk and spill into a new one
+                unsigned long long nb = 0ull;
+                if (ch_fill + (unsigned)n > kEvChunk) {  // a new chunk, linked to the warp's last one
+                    if (lane == 0u) {
+                        nb = atomicAdd(A.ev_count, (unsigned long long)kEvChunk);
+                        // (a chunk past the buffer is not linked: the call then replays instead)
+                        if (nb + kEvChunk <= A.ev_cap)
+                            A.ch_prev[nb / kEvChunk] = ch_base == ~0ull ? kEndChunk : (uint32_t)(ch_base / kEvChunk);
+                    }
+                    nb = __shfl_sync(kFull, nb, 0);
+                }
+                const unsigned f = ch_fill + lane;
+                ev_slot = f < kEvChunk ? ch_base + f : nb + (f - kEvChunk);
+                if (ch_fill + (unsigned)n > kEvChunk) {
+                    ch_base = nb;
+                    ch_fill = ch_fill + (unsigned)n - kEvChunk;
+                } else {
+                    ch_fill += (unsigned)n;
+                }
+            }
+            int term = -1;  // -1 idle lane, 0 goes on, > 0 ended
+            int i = 0;
+            EventTally t;
+            if ((int)lane < n) {
+                i = evq[ev_n - 1 - (int)lane];
+                const uint32_t* s = sl + i;
+                Photon e;
+                e.d = make_float3(__uint_as_float(s[(kSD + 0) * kSlots]), __uint_as_float(s[(kSD + 1) * kSlots]),
+                                  __uint_as_float(s[(kSD + 2) * kSlots]));
+                const int at = (int)s[kSLin * kSlots];
+                e.tau = __uint_as_float(s[kSTau * kSlots]);
+                // the collision point (see flight_end)
+                const float l = e.tau / BetaFetch<DT>::get(A.beta_pad, at);
+                e.p = make_float3(flight_offset(__uint_as_float(s[(kST + 0) * kSlots]), e.d.x, A.g.hx,
+                                                fabsf(__uint_as_float(s[(kSQ + 0) * kSlots])), l),
+                                  flight_offset(__uint_as_float(s[(kST + 1) * kSlots]), e.d.y, A.g.hy,
+                                                fabsf(__uint_as_float(s[(kSQ + 1) * kSlots])), l),
+                                  flight_offset(__uint_as_float(s[(kST + 2) * kSlots]), e.d.z, A.g.hz,
+                                                fabsf(__uint_as_float(s[(kSQ + 2) * kSlots])), l));
+                unpad(A.g, at, e.ix, e.iy, e.iz);
+                e.I = __uint_as_float(s[kSI * kSlots]);
+                e.s = s[kSs * kSlots] + 1u;
+                e.idx = s[kSIdx * kSlots];
+                e.id = A.first_id + (e.idx - A.out_base);
+                ++events;
+                const int k = lin_index(A.g, e.ix, e.iy, e.iz);
+                uint4 xb = make_uint4(0u, 0u, 0u, 0u);  // two species: the event's Philox block
+                bool air = false;
+                if constexpr (TWO) {
+                    xb = draw_bits(A.key, e.id, e.s);
+                    air = particle_is_air(A, xb, k);
+                }
+                if (air) air_events.add();
+                const float wgt = (air ? A.albedo_air : A.albedo) * e.I;
+                if (A.hash) A.hash[e.idx] = (A.hash[e.idx] ^ (uint32_t)k) * kFnvPrime;
+                if (A.point) write_point(A, e);
+                if (A.ev_cap && ev_slot < A.ev_cap) store_event(A, ev_slot, e, wgt, air, s[kSPrev * kSlots]);
+                le_voxel(A, e, wgt, k, air);
+                term = after_event<TWO>(A, e, t, air, xb);
+                if (term == 0) {
+                    make_ready(i, e.p, e.d, e.ix, e.iy, e.iz, e.tau);
+                    uint32_t* o = sl + i;
+                    o[kSI * kSlots] = __float_as_uint(e.I);
+                    o[kSs * kSlots] = e.s;
+                    o[kSPrev * kSlots] = (uint32_t)ev_slot;
+                } else if (A.hash) {
+                    finish_hash(A, e.idx, e.s, term);
+                }
+            }
+            ev_n -= n;
+            add_tally(MST_ST_ABSORBED, t.absorbed);
+            if (__any_sync(kFull, t.rare)) {
+                add_tally(MST_ST_RR_KILLED, t.killed);
+                add_tally(MST_ST_RR_GAINED, t.gained);
+                add_tally(MST_ST_FORCED, t.forced);
+                add_tally(MST_ST_CAPPED, t.capped);
+            }
+            const unsigned gm = __ballot_sync(kFull, term == 0), fm = __ballot_sync(kFull, term > 0);
+            if (term == 0) rdq[rd_n + __popc(gm & lanemask_lt())] = (uint8_t)i;
+            if (term > 0) frq[fr_n + __popc(fm & lanemask_lt())] = (uint8_t)i;
+            rd_n += __popc(gm);
+            fr_n += __popc(fm);
+            __syncwarp();
+        }
+    }
+    while (esc_n > 0) count_escapes(min(32, esc_n));
+    {
+        const unsigned long long ev = warp_sumu(events), sg = warp_sumu(segments), la = warp_sumu(launched),
+                                 es = warp_sumu(escaped);
+        if (lane == 0u) {
+            tally[MST_ST_EVENTS] = (double)ev;
+            tally[MST_ST_SEGMENTS] = (double)sg;
+            tally[MST_ST_TRACED] = (double)la;
+            tally[MST_ST_LAUNCHED] = (double)la * (double)A.I0;
+            tally[MST_ST_ESCAPED_N] = (double)es;
+        }
+        __syncwarp();
+        for (int i = (int)lane; i < MST_NSTATS; i += 32)
+            if (tally[i] != 0.0) atomicAdd(A.stats + i, tally[i]);
+        __syncwarp();
+    }
+    air_events.flush(A.stats + MST_ST_AIR_EVENTS, lane);
+    if (A.ev_cap) {  // the warp's last chunk; its tail holds no event
+        if (lane == 0u) A.warp_tail[gwarp] = ch_base == ~0ull ? kEndChunk : (uint32_t)(ch_base / kEvChunk);
+        if (ch_base != ~0ull)
+            for (unsigned f = ch_fill + lane; f < kEvChunk; f += 32u)
+                if (ch_base + f < A.ev_cap) A.evrec[2ull * A.ev_cap + ch_base + f].x = kNoPhoton;
+    }
+}
+
+constexpr size_t forward_smem() {
+    return (size_t)(kTB / 32) * kFwdWords * sizeof(uint32_t);
+}
+
+template <int DT, bool TWO, int TRIP>
+__global__ void __launch_bounds__(kTB, kMinBlocksForward) k_forward(const TransportArgs A) {
+    extern __shared__ uint32_t smem[];
+    forward_run<DT, TWO, TRIP>(A, smem);
+}
+
+// Many scenes in one persistent launch: every warp runs the scenes of the table one after another
+template <int TRIP>
+__global__ void __launch_bounds__(kTB, kMinBlocksForward)
+    k_forward_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
+    extern __shared__ uint32_t smem[];
+    for (int s = 0; s < n_scenes; ++s) {
+        forward_run<0, false, TRIP>(scenes[s], smem);
         __syncwarp();
     }
 }
@@ -1548,12 +1986,12 @@ constexpr size_t score_smem() {
 }
 
 template <typename K>
-int occupancy(K kern, size_t smem) {
+int occupancy(K kern, size_t smem, int blocks = 3) {
     int n = 0;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    {   // shared-memory carveout: enough for three blocks (the register budget allows no more), the
-        // rest of the SM's 256 KB to L1, which caches the extinction grid the walks fetch
-        const size_t need = 3 * (smem + 1024);
+    {   // shared-memory carveout: enough for the blocks of the kernel's register budget, the rest of the
+        // SM's 256 KB to L1, which caches the extinction grid the walks fetch
+        const size_t need = blocks * (smem + 1024);
         const int pct = (int)std::min<size_t>(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     }
@@ -1571,31 +2009,46 @@ cudaError_t launch_mode(const TransportArgs& a, int blocks, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Trip-length variants of the FP32-grid forward and pass-2 kernels, for the autotuner
-// (kForwardTrips / kReplayTrips; the defaults are the un-suffixed kernels).
+// Trip-length variants of the FP32-grid pass-2 kernel, for the autotuner
 template <int MODE, bool TWO>
 cudaError_t launch_trip(const TransportArgs& a, int trip, int blocks, cudaStream_t st) {
-    if constexpr (MODE == kFwdVoxel) {
+    switch (trip) {
+        case 4: return launch_mode<0, MODE, TWO, 4>(a, blocks, st);
+        case 8: return launch_mode<0, MODE, TWO, 8>(a, blocks, st);
+        case 10: return launch_mode<0, MODE, TWO, 10>(a, blocks, st);
+        default: return launch_mode<0, MODE, TWO>(a, blocks, st);
+    }
+}
+
+template <int DT, bool TWO, int TRIP>
+cudaError_t launch_forward_t(const TransportArgs& a, int blocks, cudaStream_t st) {
+    if constexpr (TRIP != kStepsForward) {  // the default's attributes are set by occupancy()
+        static const int once = occupancy(k_forward<DT, TWO, TRIP>, forward_smem(), kMinBlocksForward);
+        (void)once;
+    }
+    k_forward<DT, TWO, TRIP><<<blocks, kTB, forward_smem(), st>>>(a);
+    return cudaGetLastError();
+}
+
+// The forward of the voxel estimator; FP32 grids have the trip-length variants of the autotuner.
+template <int DT, bool TWO>
+cudaError_t launch_forward(const TransportArgs& a, int trip, int blocks, cudaStream_t st) {
+    if constexpr (DT == 0) {
         switch (trip) {
-            case 8: return launch_mode<0, MODE, TWO, 8>(a, blocks, st);
-            case 10: return launch_mode<0, MODE, TWO, 10>(a, blocks, st);
-            case 16: return launch_mode<0, MODE, TWO, 16>(a, blocks, st);
-            default: return launch_mode<0, MODE, TWO>(a, blocks, st);
-        }
-    } else {  // pass 2
-        switch (trip) {
-            case 4: return launch_mode<0, MODE, TWO, 4>(a, blocks, st);
-            case 8: return launch_mode<0, MODE, TWO, 8>(a, blocks, st);
-            case 10: return launch_mode<0, MODE, TWO, 10>(a, blocks, st);
-            default: return launch_mode<0, MODE, TWO>(a, blocks, st);
+            case 8: return launch_forward_t<0, TWO, 8>(a, blocks, st);
+            case 10: return launch_forward_t<0, TWO, 10>(a, blocks, st);
+            case 12: return launch_forward_t<0, TWO, 12>(a, blocks, st);
+            case 16: return launch_forward_t<0, TWO, 16>(a, blocks, st);
+            default: break;
         }
     }
+    return launch_forward_t<DT, TWO, kStepsForward>(a, blocks, st);
 }
 
 template <int DT, bool TWO>
 int occupancy_mode(int mode) {
     switch (mode) {
-        case kFwdVoxel: return occupancy(k_transport<DT, kFwdVoxel, TWO>, smem_bytes<kFwdVoxel>());
+        case kFwdVoxel: return occupancy(k_forward<DT, TWO, kStepsForward>, forward_smem(), kMinBlocksForward);
         case kFwdClassic: return occupancy(k_transport<DT, kFwdClassic, TWO>, smem_bytes<kFwdClassic>());
         case kPass2: return occupancy(k_transport<DT, kPass2, TWO>, smem_bytes<kPass2>());
         case kScore: return occupancy(k_score<DT, TWO, kStepsScore>, score_smem<kStepsScore>());
@@ -1608,11 +2061,10 @@ int occupancy_mode(int mode) {
 template <int DT, bool TWO>
 cudaError_t launch_dt(const TransportArgs& a, int mode, int trip, int blocks, cudaStream_t st) {
     if constexpr (DT == 0) {
-        if (trip > 0 && mode == kFwdVoxel) return launch_trip<kFwdVoxel, TWO>(a, trip, blocks, st);
         if (trip > 0 && mode == kPass2) return launch_trip<kPass2, TWO>(a, trip, blocks, st);
     }
     switch (mode) {
-        case kFwdVoxel: return launch_mode<DT, kFwdVoxel, TWO>(a, blocks, st);
+        case kFwdVoxel: return launch_forward<DT, TWO>(a, trip, blocks, st);
         case kFwdClassic: return launch_mode<DT, kFwdClassic, TWO>(a, blocks, st);
         case kPass2: return launch_mode<DT, kPass2, TWO>(a, blocks, st);
         case kPass1C: return launch_mode<DT, kPass1C, TWO>(a, blocks, st);
@@ -1649,11 +2101,12 @@ cudaError_t launch_transport_batch(const TransportArgs* table, int n, int mode, 
     switch (mode) {
         case kFwdVoxel:
             switch (trip) {
-                case 8: return launch_batch_mode<kFwdVoxel, 8>(table, n, blocks, st);
-                case 10: return launch_batch_mode<kFwdVoxel, 10>(table, n, blocks, st);
-                case 16: return launch_batch_mode<kFwdVoxel, 16>(table, n, blocks, st);
-                default: return launch_batch_mode<kFwdVoxel>(table, n, blocks, st);
+                case 8: k_forward_batch<8><<<blocks, kTB, forward_smem(), st>>>(table, n); break;
+                case 10: k_forward_batch<10><<<blocks, kTB, forward_smem(), st>>>(table, n); break;
+                case 16: k_forward_batch<16><<<blocks, kTB, forward_smem(), st>>>(table, n); break;
+                default: k_forward_batch<kStepsForward><<<blocks, kTB, forward_smem(), st>>>(table, n);
             }
+            return cudaGetLastError();
         case kPass2: return launch_batch_mode<kPass2>(table, n, blocks, st);
         case kPass1: return launch_batch_mode<kPass1>(table, n, blocks, st);
         default: return cudaErrorInvalidValue;
@@ -1664,10 +2117,10 @@ int transport_batch_blocks_per_sm(int mode) {
     static int occ[7] = {0, 0, 0, 0, 0, 0, 0};
     static bool ready = false;
     if (!ready) {  // every instantiation's attributes, once; the default trips give the occupancy
-        occ[kFwdVoxel] = batch_occupancy<kFwdVoxel>();
-        batch_occupancy<kFwdVoxel, 8>();
-        batch_occupancy<kFwdVoxel, 10>();
-        batch_occupancy<kFwdVoxel, 16>();
+        occ[kFwdVoxel] = occupancy(k_forward_batch<kStepsForward>, forward_smem(), kMinBlocksForward);
+        occupancy(k_forward_batch<8>, forward_smem(), kMinBlocksForward);
+        occupancy(k_forward_batch<10>, forward_smem(), kMinBlocksForward);
+        occupancy(k_forward_batch<16>, forward_smem(), kMinBlocksForward);
         occ[kScore] = occupancy(k_score_batch<kStepsScore>, score_smem<kStepsScore>());
         occupancy(k_score_batch<4>, score_smem<4>());
         occupancy(k_score_batch<8>, score_smem<8>());
