@@ -150,6 +150,7 @@ TransportArgs transport_args(mst_grid* g, const mst_params* p) {
     a.adj = g->adj;
     a.gacc = g->gacc;
     a.gbrk = g->gbrk;
+    a.score_tiles = g->score_tiles;
     a.wbuf = g->wbuf;
     a.nevbuf = g->nevbuf;
     a.plist = g->plist;
@@ -163,9 +164,12 @@ TransportArgs transport_args(mst_grid* g, const mst_params* p) {
     return a;
 }
 
-// Rolling-fold slicing of a tile of `bins` bins (see kFoldSweep): slices of a multiple of 32
-// bins, at least 128, such that one sweep takes at most about kFoldSweep photons.
-void set_fold(TransportArgs& a, uint64_t bins) {
+// Rolling-fold slicing of a tile of `bins` bins (see kFoldSweep) for a launch of n photons: slices of
+// a multiple of 32 bins, at least 128, such that one sweep takes at most about kFoldSweep photons.
+// A launch of no more photons than that leaves its tile to the fold that follows it.
+void set_fold(TransportArgs& a, uint64_t bins, uint64_t n) {
+    a.fold_bins = 0;
+    if (n <= kFoldSweep) return;
     const uint64_t batches = kFoldSweep / kTicketBatch;
     uint64_t slice = (bins + batches - 1) / batches;
     slice = std::max<uint64_t>(128, (slice + 31) / 32 * 32);
@@ -176,8 +180,10 @@ void set_fold(TransportArgs& a, uint64_t bins) {
 
 // The score kernel folds one slice of its brick tile per chunk of stored events. A photon makes
 // a few events at most on average; counting one per photon keeps a sweep within kFoldSweep photons.
-void set_score_fold(TransportArgs& a) {
-    const uint64_t bins = (uint64_t)brick_bins(a.g), chunks = kFoldSweep / kEventChunk;
+void set_score_fold(TransportArgs& a, uint64_t n) {
+    a.fold_bins = 0;
+    if (n <= kFoldSweep) return;
+    const uint64_t bins = (uint64_t)brick_bins(a.g) * a.score_tiles, chunks = kFoldSweep / kEventChunk;
     const uint64_t slice = std::max<uint64_t>(32, ((bins + chunks - 1) / chunks + 31) / 32 * 32);
     a.fold_bins = bins;
     a.fold_slice = (uint32_t)slice;
@@ -205,8 +211,8 @@ int run_photons(mst_grid* g, const mst_params* p, bool replay, double* cimg, cud
     const int b_fwd = transport_blocks(g, p->grid_dtype, est);
     const int b_p1 = transport_blocks(g, p->grid_dtype, m_p1);
     const int b_p2 = transport_blocks(g, p->grid_dtype, m_p2);
-    if (replay) set_fold(a, (uint64_t)g->geo.npad);
-    else if (est == MST_EST_VOXEL) set_fold(a, (uint64_t)g->geo.nvox * g->cp);
+    if (replay) set_fold(a, (uint64_t)g->geo.npad, n);
+    else if (est == MST_EST_VOXEL) set_fold(a, (uint64_t)g->geo.nvox * g->cp, n);
     if (store_events) {
         a.evrec = g->evrec;
         a.ev_cap = g->ev_cap;
@@ -280,12 +286,12 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
     auto blocks = [&](int mode) { return transport_blocks(g, p->grid_dtype, mode); };
     {
         Phase ph(g, MST_PH_REPLAY2, st);
-        set_score_fold(a);
+        set_score_fold(a, n);
         a.ticket = g->tickets + 2;  // its warps take the forward warps' lists from it
         MST_CK(launch_score(g, a, p->grid_dtype, blocks(4), st));
         MST_CK(launch_fold_bricks(g, st));
     }
-    set_fold(a, (uint64_t)g->geo.npad);
+    set_fold(a, (uint64_t)g->geo.npad, n);
     a.ticket = g->tickets;
     {
         Phase ph(g, MST_PH_REPLAY, st);  // these return at once when the events fitted
@@ -546,6 +552,7 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     geo.npad = geo.p01 * (d->nz + 2 * kHalo);
     for (int a = 0; a < 3; ++a) g->origin[a] = d->origin[a];
     g->voxel_volume = d->dx * d->dy * d->dz;
+    g->score_tiles = score_tile_copies((uint64_t)brick_bins(geo));
     g->n_cams = n_cams;
     g->cp = (n_cams + 3) / 4 * 4;
     g->n_rays = n_rays;
@@ -612,7 +619,7 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         {(void**)&g->gT, C * geo.npad * 4},
         {(void**)&g->adj, nvox * g->cp * 4},
         {(void**)&g->gacc, (size_t)geo.npad * 4},
-        {(void**)&g->gbrk, (size_t)brick_bins(geo) * 4},
+        {(void**)&g->gbrk, (size_t)brick_bins(geo) * g->score_tiles * 4},
         {(void**)&g->score_cnt, (2 * kScoreBins + 1) * 4},
         {(void**)&g->g64, nvox * 8},
         {(void**)&g->resid, (size_t)off * 8},
@@ -647,7 +654,7 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     if (e == cudaSuccess) e = cudaMemset(g->R, 0xFF, C * geo.npad * 4);  // the halo's mark (k_los writes the rest)
     if (e == cudaSuccess) e = cudaMemset(g->Lacc, 0, nvox * g->cp * 4);
     if (e == cudaSuccess) e = cudaMemset(g->gacc, 0, (size_t)geo.npad * 4);
-    if (e == cudaSuccess) e = cudaMemset(g->gbrk, 0, (size_t)brick_bins(geo) * 4);
+    if (e == cudaSuccess) e = cudaMemset(g->gbrk, 0, (size_t)brick_bins(geo) * g->score_tiles * 4);
     if (e == cudaSuccess) e = cudaMemset(g->stats, 0, MST_NSTATS * 8 + 64);
     if (e != cudaSuccess) {
         free_all(g);
@@ -1333,7 +1340,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         const mst_params* p = &params[i];
         g->beta_in = betas[i];
         TransportArgs f = transport_args(g, p);
-        set_fold(f, (uint64_t)g->geo.nvox * g->cp);
+        set_fold(f, (uint64_t)g->geo.nvox * g->cp, p->n_photons);
         f.evrec = g->evrec;
         f.ev_cap = g->ev_cap;
         f.ev_count = g->ev_count;
@@ -1346,7 +1353,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         f.ticket = g->tickets;
         t[i] = f;
         TransportArgs r = transport_args(g, p);
-        set_score_fold(r);
+        set_score_fold(r, p->n_photons);
         r.evrec = g->evrec;
         r.ev_cap = g->ev_cap;
         r.ev_count = g->ev_count;
@@ -1358,7 +1365,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         r.n = (uint32_t)p->n_photons;
         r.ticket = g->tickets + 2;  // the score kernel's warps take the forward warps' lists from it
         t[n + i] = r;
-        set_fold(r, (uint64_t)g->geo.npad);
+        set_fold(r, (uint64_t)g->geo.npad, p->n_photons);
         r.ticket = g->tickets;      // pass 1 (returns at once when the events fitted)
         t[2 * n + i] = r;
         r.ticket = g->tickets + 1;  // pass 2
@@ -1535,7 +1542,7 @@ int mst_batch_set_wavefront(mst_batch* b, int forward_trip, int forward_blocks, 
         b->err = "forward trip in {0, 8, 10, 12, 16}, pass-2 trip in {0, 4, 6, 8, 10}, blocks per SM in 0..8";
         return MST_ERR_INVALID_ARG;
     }
-    b->trip_fwd = forward_trip == 12 ? 0 : forward_trip;  // 12 and 6 are the kernels' defaults
+    b->trip_fwd = forward_trip == 8 ? 0 : forward_trip;  // 8 and 6 are the kernels' defaults
     b->blocks_fwd = forward_blocks;
     b->trip_p2 = replay_trip == 6 ? 0 : replay_trip;
     b->blocks_p2 = replay_blocks;

@@ -27,7 +27,10 @@ constexpr uint64_t kRecordMaxPhotons = 1ull << 27;
 // path left when the flight entered the event's voxel, the photon's previous record
 constexpr int kEventBytes = 3 * 16;
 constexpr unsigned kEventChunk = 256;  // record slots a warp of the forward reserves at a time
-constexpr int kTransportWarps = 8;     // warps per transport block (256 threads)
+// Warps per forward or score block. Four blocks of seven, 28 warps, fit an SM at 72 registers a thread,
+// which both kernels need: the forward ran 37.1 ms with 24 warps at 80 registers, 34.7 with 28,
+// 35.4 with 32 at 64 registers and their spills (64^3, 1e8 photons).
+constexpr int kTransportWarps = 7;
 constexpr uint32_t kEndChunk = 0xFFFFFFFFu;  // end of a warp's chunk list
 constexpr int kMaxWarpsPerSm = 64;     // warp_tail entries per SM (the forward runs 24)
 constexpr uint64_t kDefaultRecordBytes = 32ull << 30;
@@ -35,6 +38,16 @@ constexpr uint64_t kFoldSweep = 1ull << 21;
 constexpr int kTicketBatch = 64;  // photon ids a warp takes from the global ticket at a time
 constexpr int kMaxTickets = (int)(2 * (kMaxPhotons / kReplayChunk));
 constexpr int kScoreBins = 64;  // replay pass-2 list bins over the pass-1 event count (multiple of 32)
+
+// Copies of the score kernel's gradient tile for a grid of `bins` bins: up to a million bins in all
+// (4 MB, which stay in L2) and 32 copies. Its atomics on one bin queue up: 32^3 voxels at 1e7
+// photons take 3.00 / 2.23 / 1.67 ms with 1 / 4 / 8 copies, 64^3 at 1e8 take 18.8 / 17.8 / 17.6 / 17.8
+// with 1 / 2 / 4 / 8.
+inline uint32_t score_tile_copies(uint64_t bins) {
+    uint32_t c = 1;
+    while (c < 32 && 2 * c * bins <= (1ull << 20)) c *= 2;
+    return c;
+}
 
 // A photon that replay pass 2 must walk: index in the chunk, event count and W of pass 1.
 struct ScoreRec {
@@ -66,7 +79,8 @@ struct TransportArgs {
     const double* cres;        // [total pix] dE/di of the classic images (classic-estimator gradient)
     const float* adj;          // [nvox][cp] a_c(k) = T_c(k) b_c(k) (replay)
     float* gacc;               // [npad] FP32 gradient accumulator on the padded grid (replay)
-    float* gbrk;               // FP32 gradient accumulator in 2 x 2 x 2 bricks (score of the stored events)
+    float* gbrk;               // FP32 gradient accumulator in 2 x 2 x 2 bricks (score of the stored events) ...
+    uint32_t score_tiles;      // ... and its copies
     double* wbuf;              // [photons of the chunk] W per photon (replay pass 1; the score kernel's
                                // running sum of each photon's later w_s)
     uint32_t* nevbuf;          // [photons of the chunk] events per photon (replay pass 1)
@@ -113,7 +127,8 @@ struct mst_grid {
     float* gT = nullptr;          // [C][npad]  W_c^T (L T b)
     float* adj = nullptr;         // [nvox][cp] T_c b_c
     float* gacc = nullptr;        // [npad] gradient tile on the padded grid
-    float* gbrk = nullptr;        // [brick_bins] gradient tile in 2 x 2 x 2 bricks
+    float* gbrk = nullptr;        // [score_tiles][brick_bins] gradient tile in 2 x 2 x 2 bricks
+    uint32_t score_tiles = 1;     // its copies
     double* wbuf = nullptr;       // [replay_cap], allocated by the first full-gradient call
     uint32_t* nevbuf = nullptr;   // [replay_cap]
     mst::ScoreRec* plist = nullptr;     // [replay_cap]

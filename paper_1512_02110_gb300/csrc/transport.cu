@@ -16,6 +16,7 @@ namespace mst {
 namespace {
 
 constexpr int kTB = 256;
+constexpr int kFT = kTransportWarps * 32;  // threads of a forward or score block
 constexpr unsigned kFull = 0xffffffffu;
 constexpr uint32_t kFnvOffset = 2166136261u;
 constexpr uint32_t kFnvPrime = 16777619u;
@@ -684,38 +685,26 @@ constexpr int kScoreTile = 4096;   // photons per block in the list kernels
 // chunks backwards and meet every photon's events from the last to the first. The buffer keeps
 // one chunk per resident warp of headroom for the chunks' unused tails.
 constexpr unsigned kEvChunk = kEventChunk;
-static_assert(kTB / 32 == kTransportWarps, "transport block size");
 constexpr uint32_t kNoPhoton = 0xFFFFFFFFu;  // photon word of a chunk's unused tail slots
 constexpr uint32_t kNoEvent = 0xFFFFFFFFu;   // previous record of a photon's first event
 constexpr int kSlots = 64;
 // Voxels a flying lane advances per loop trip, and minimum resident blocks per SM (register
 // budget), per kernel mode; set from sweeps on the 64^3 cumulus workload.
-#ifndef KSF
-#define KSF 8
-#endif
-constexpr int kStepsForward = KSF;
+constexpr int kStepsForward = 8;
 constexpr int kStepsPass1 = 8;
 constexpr int kStepsPass2 = 6;
-#ifndef MBF
-#define MBF 3
-#endif
-#ifndef KSF
-#define KSF 8
-#endif
-#ifndef KDR
-#define KDR 1
-#endif
-constexpr int kDrain = KDR;
-#ifndef LFR
-#define LFR 16
-#endif
-constexpr int kLaunchFrom = LFR;
-constexpr int kMinBlocksForward = MBF;
+constexpr int kStepsScore = 6;  // list entries a score lane adds per loop trip
+// A draining warp of the forward takes its queued events once they are no fewer than the flights
+// still under way.
+constexpr int kDrain = 1;
+// The forward launches photons when this many slots are free: 1 / 8 / 16 / 24 / 32 ran 37.0 / 36.9 /
+// 37.1 / 39.2 / 42.8 ms at 1e8 photons (64^3): waiting for more leaves lanes idle.
+constexpr int kLaunchFrom = 8;
+constexpr int kMinBlocksForward = 4;
+constexpr int kMinBlocksScore = 4;
 constexpr int kMinBlocksClassic = 3;
 constexpr int kMinBlocksPass1 = 3;
 constexpr int kMinBlocksPass2 = 3;
-constexpr int kMinBlocksScore = 3;
-constexpr int kStepsScore = 6;  // list entries a score lane adds per loop trip
 
 // kernel modes
 // kScore: the score of the stored events (k_score); kPass1C, kPass2C: passes 1 and 2 of the
@@ -1209,6 +1198,7 @@ __global__ void __launch_bounds__(kTB, min_blocks(MODE))
 // the flight: t (3), free path, padded index, and q (3) while it is ready, the extinction of the
 // collision voxel in the fourth word of the walk when it has ended
 constexpr int kSlotWords = 15;
+static_assert(kSlots == 64, "the queues hold slot numbers in bytes");
 constexpr int kSD = 0, kSI = 3, kSs = 4, kSIdx = 5, kSPrev = 6, kST = 7, kSTau = 10, kSLin = 11, kSQ = 12;
 constexpr int kEscSlots = 64;  // flights out of the grid a warp puts aside
 
@@ -1247,7 +1237,7 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
     uint8_t* evq = reinterpret_cast<uint8_t*>(esc + 2 * kEscSlots);  // slots of ended flights
     uint8_t* rdq = evq + kSlots;                                     // of ready photons
     uint8_t* frq = rdq + kSlots;                                     // of no photon
-    const uint32_t gwarp = blockIdx.x * (kTB / 32) + warp;           // the warp's chunk list
+    const uint32_t gwarp = blockIdx.x * kTransportWarps + warp;       // the warp's chunk list
     for (int i = (int)lane; i < MST_NSTATS; i += 32) tally[i] = 0.0;
     // adds the lanes' values to a statistic of the warp (nothing when all are 0)
     auto add_tally = [&](int which, float v) {
@@ -1507,11 +1497,17 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
                 e.id = A.first_id + (e.idx - A.out_base);
                 ++events;
                 const int k = lin_index(A.g, e.ix, e.iy, e.iz);
-                uint4 xb = make_uint4(0u, 0u, 0u, 0u);  // two species: the event's Philox block
                 bool air = false;
                 if constexpr (TWO) {
-                    xb = draw_bits(A.key, e.id, e.s);
-                    air = particle_is_air(A, xb, k);
+                    // the event's Philox block: its scattering step needs it again, and it waits in
+                    // the flight's words meanwhile (volatile, so that no register holds it)
+                    const uint4 x = draw_bits(A.key, e.id, e.s);
+                    air = particle_is_air(A, x, k);
+                    volatile uint32_t* o = sl + i + kST * kSlots;
+                    o[0] = x.x;
+                    o[kSlots] = x.y;
+                    o[2 * kSlots] = x.z;
+                    o[3 * kSlots] = x.w;
                 }
                 if (air) air_events.add();
                 const float wgt = (air ? A.albedo_air : A.albedo) * e.I;
@@ -1519,6 +1515,11 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
                 if (A.point) write_point(A, e);
                 if (A.ev_cap && ev_slot < A.ev_cap) store_event(A, ev_slot, e, wgt, air, s[kSPrev * kSlots]);
                 le_voxel(A, e, wgt, k, air);
+                uint4 xb = make_uint4(0u, 0u, 0u, 0u);
+                if constexpr (TWO) {
+                    const volatile uint32_t* o = sl + i + kST * kSlots;
+                    xb = make_uint4(o[0], o[kSlots], o[2 * kSlots], o[3 * kSlots]);
+                }
                 term = after_event<TWO>(A, e, t, air, xb);
                 if (term == 0) {
                     make_ready(i, e.p, e.d, e.ix, e.iy, e.iz, e.tau);
@@ -1572,18 +1573,18 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
 }
 
 constexpr size_t forward_smem() {
-    return (size_t)(kTB / 32) * kFwdWords * sizeof(uint32_t);
+    return (size_t)kTransportWarps * kFwdWords * sizeof(uint32_t);
 }
 
 template <int DT, bool TWO, int TRIP>
-__global__ void __launch_bounds__(kTB, kMinBlocksForward) k_forward(const TransportArgs A) {
+__global__ void __launch_bounds__(kFT, kMinBlocksForward) k_forward(const TransportArgs A) {
     extern __shared__ uint32_t smem[];
     forward_run<DT, TWO, TRIP>(A, smem);
 }
 
 // Many scenes in one persistent launch: every warp runs the scenes of the table one after another
 template <int TRIP>
-__global__ void __launch_bounds__(kTB, kMinBlocksForward)
+__global__ void __launch_bounds__(kFT, kMinBlocksForward)
     k_forward_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
     extern __shared__ uint32_t smem[];
     for (int s = 0; s < n_scenes; ++s) {
@@ -1609,6 +1610,8 @@ __global__ void __launch_bounds__(kTB, kMinBlocksForward)
 // strip and out transposed, so that one atomic instruction holds consecutive voxels of a few
 // flights. Random FP32 atomics run at 2.0e11 a second on this chip whatever the tile's size, but
 // the words of one 32-byte sector go out together, and the tile keeps 2 x 2 x 2 voxels in a sector.
+// Additions to one bin queue up, so small grids have the tile several times over (score_tiles), a
+// block adding to one of the copies.
 
 constexpr int kFlightWords = 10;  // of a queued flight
 constexpr int kScoreSlots = 64;   // flights a warp queues: fewer than 32 left when a batch adds 32
@@ -1642,6 +1645,7 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
     uint32_t* q = rec + 3 * 4 * 32;                                // queue: word f of slot i at q[f * kScoreSlots + i]
     float2* strip = reinterpret_cast<float2*>(q + kFlightWords * kScoreSlots);
     const unsigned nbins = (unsigned)brick_bins(A.g);
+    float* tile = A.gbrk + (size_t)(blockIdx.x % A.score_tiles) * nbins;  // the block's copy
     const uint32_t by8 = 8u * (unsigned)((A.g.nx + 1) >> 1), bz8 = by8 * (unsigned)((A.g.ny + 1) >> 1);
     unsigned stored = 0u, flights = 0u, entries = 0u, lost = 0u;
 
@@ -1672,12 +1676,12 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
             prev = A.ch_prev[ch];
             base = (int)kEvChunk - 32;
             // one slice of the rolling fold (see kFoldSweep) per chunk
-            const uint32_t i0 = ch % A.fold_nslices * A.fold_slice;
+            const uint32_t i0 = A.fold_bins ? ch % A.fold_nslices * A.fold_slice : 0u;
             const uint32_t i1 = min(i0 + A.fold_slice, (uint32_t)A.fold_bins);
             for (uint32_t i = i0 + lane; i < i1; i += 32) {
                 const float v = atomicExch(A.gbrk + i, 0.f);
                 int k;
-                if (v != 0.f && brick_voxel(A.g, (int)i, k)) atomicAdd(A.g64 + k, (double)v);
+                if (v != 0.f && brick_voxel(A.g, (int)(i % nbins), k)) atomicAdd(A.g64 + k, (double)v);
             }
         }
         const uint4* r = A.evrec + ((unsigned long long)ch * kEvChunk + (unsigned)base + lane);
@@ -1746,7 +1750,7 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
                 const float ib = 1.f / b;
                 float is = ib;  // [aerosol] / beta_aer with two species
                 if constexpr (TWO) is = air ? 0.f : 1.f / __ldg(A.beta_aer + k);
-                atomicAdd(A.gbrk + bin, Sf * (is - __uint_as_float(r2.z) * ib));
+                atomicAdd(tile + bin, Sf * (is - __uint_as_float(r2.z) * ib));
                 ++flights;
                 entries += (unsigned)n + 1u;
             }
@@ -1826,7 +1830,7 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
             const int i = r * 32 + (int)lane, j = i % K, l = i / K;  // entry j of lane l
             const float2 en = strip[j * 32 + ((l ^ (2 * j)) & 31)];
             const uint32_t key = __float_as_uint(en.x);
-            if (key < nbins) atomicAdd(A.gbrk + key, en.y);
+            if (key < nbins) atomicAdd(tile + key, en.y);
         }
         __syncwarp();
     }
@@ -1841,14 +1845,14 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
 }
 
 template <int DT, bool TWO, int K>
-__global__ void __launch_bounds__(kTB, kMinBlocksScore) k_score(const TransportArgs A) {
+__global__ void __launch_bounds__(kFT, kMinBlocksScore) k_score(const TransportArgs A) {
     extern __shared__ uint32_t smem[];
     score_run<DT, TWO, K>(A, smem);
 }
 
 // the batched form: the scenes of a table one after the other
 template <int K>
-__global__ void __launch_bounds__(kTB, kMinBlocksScore)
+__global__ void __launch_bounds__(kFT, kMinBlocksScore)
     k_score_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
     extern __shared__ uint32_t smem[];
     for (int s = 0; s < n_scenes; ++s) {
@@ -1928,17 +1932,33 @@ __global__ void __launch_bounds__(kTB) k_score_scatter(const double* __restrict_
     }
 }
 
-// Folds the FP32 chunk tiles into the FP64 results and clears them.
-__global__ void k_fold_L(float* __restrict__ Lacc, double* __restrict__ L64, int nvox, int C, int cp) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nvox; k += gridDim.x * blockDim.x) {
-        float* row = Lacc + (size_t)k * cp;
-        for (int c = 0; c < C; ++c) {
-            const float v = row[c];
-            if (v != 0.f) {
-                L64[(size_t)c * nvox + k] += (double)v;
-                row[c] = 0.f;
-            }
+// Folds the FP32 L tile [nvox][cp] into the FP64 result [C][nvox] and clears it. A block takes kFoldRows
+// rows through shared memory, so that both sides move whole lines (a thread per row read 32 lines
+// an instruction: 1.1 ms for 80 x 80 x 120 voxels and 36 cameras).
+constexpr int kFoldRows = 32;
+__global__ void __launch_bounds__(kTB) k_fold_L(float* __restrict__ Lacc, double* __restrict__ L64, int nvox, int C,
+                                                int cp) {
+    extern __shared__ float rows[];  // [kFoldRows][cp + 1]
+    for (int k0 = blockIdx.x * kFoldRows; k0 < nvox; k0 += gridDim.x * kFoldRows) {
+        const int n = min(kFoldRows, nvox - k0);
+        float4* from = reinterpret_cast<float4*>(Lacc + (size_t)k0 * cp);
+        for (int i = threadIdx.x; i < n * cp / 4; i += kTB) {
+            const float4 v = from[i];
+            const int row = 4 * i / cp;
+            float* to = rows + row * (cp + 1) + (4 * i - row * cp);
+            to[0] = v.x;
+            to[1] = v.y;
+            to[2] = v.z;
+            to[3] = v.w;
+            if (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f) from[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kFoldRows * C; i += kTB) {
+            const int r = i % kFoldRows, c = i / kFoldRows;
+            const float v = r < n ? rows[r * (cp + 1) + c] : 0.f;
+            if (v != 0.f) L64[(size_t)c * nvox + k0 + r] += (double)v;
+        }
+        __syncthreads();
     }
 }
 
@@ -1956,15 +1976,16 @@ __global__ void k_fold_grad(float* __restrict__ gacc, double* __restrict__ g64, 
 }
 
 // what the score kernel left in its brick tile
-__global__ void k_fold_bricks(float* __restrict__ gbrk, double* __restrict__ g64, const Geo g) {
+__global__ void k_fold_bricks(float* __restrict__ gbrk, double* __restrict__ g64, const Geo g, int tiles) {
     const int nb = brick_bins(g);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
-        const float v = gbrk[i];
-        if (v != 0.f) {
-            int k;
-            if (brick_voxel(g, i, k)) g64[k] += (double)v;
-            gbrk[i] = 0.f;
+        double v = 0.0;
+        for (int t = 0; t < tiles; ++t) {
+            v += (double)gbrk[(size_t)t * nb + i];
+            gbrk[(size_t)t * nb + i] = 0.f;
         }
+        int k;
+        if (v != 0.0 && brick_voxel(g, i, k)) g64[k] += v;
     }
 }
 
@@ -1982,11 +2003,11 @@ constexpr size_t smem_bytes() {
 // the score kernel's: the warps' flight queues and entry strips
 template <int K>
 constexpr size_t score_smem() {
-    return (size_t)(kTB / 32) * score_words<K>() * sizeof(uint32_t);
+    return (size_t)kTransportWarps * score_words<K>() * sizeof(uint32_t);
 }
 
 template <typename K>
-int occupancy(K kern, size_t smem, int blocks = 3) {
+int occupancy(K kern, size_t smem, int blocks = 3, int threads = kTB) {
     int n = 0;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     {   // shared-memory carveout: enough for the blocks of the kernel's register budget, the rest of the
@@ -1995,7 +2016,7 @@ int occupancy(K kern, size_t smem, int blocks = 3) {
         const int pct = (int)std::min<size_t>(100, (need * 100 + 228 * 1024 - 1) / (228 * 1024));
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     }
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kTB, smem) != cudaSuccess || n < 1) n = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess || n < 1) n = 1;
     return n;
 }
 
@@ -2023,10 +2044,10 @@ cudaError_t launch_trip(const TransportArgs& a, int trip, int blocks, cudaStream
 template <int DT, bool TWO, int TRIP>
 cudaError_t launch_forward_t(const TransportArgs& a, int blocks, cudaStream_t st) {
     if constexpr (TRIP != kStepsForward) {  // the default's attributes are set by occupancy()
-        static const int once = occupancy(k_forward<DT, TWO, TRIP>, forward_smem(), kMinBlocksForward);
+        static const int once = occupancy(k_forward<DT, TWO, TRIP>, forward_smem(), kMinBlocksForward, kFT);
         (void)once;
     }
-    k_forward<DT, TWO, TRIP><<<blocks, kTB, forward_smem(), st>>>(a);
+    k_forward<DT, TWO, TRIP><<<blocks, kFT, forward_smem(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -2048,10 +2069,10 @@ cudaError_t launch_forward(const TransportArgs& a, int trip, int blocks, cudaStr
 template <int DT, bool TWO>
 int occupancy_mode(int mode) {
     switch (mode) {
-        case kFwdVoxel: return occupancy(k_forward<DT, TWO, kStepsForward>, forward_smem(), kMinBlocksForward);
+        case kFwdVoxel: return occupancy(k_forward<DT, TWO, kStepsForward>, forward_smem(), kMinBlocksForward, kFT);
         case kFwdClassic: return occupancy(k_transport<DT, kFwdClassic, TWO>, smem_bytes<kFwdClassic>());
         case kPass2: return occupancy(k_transport<DT, kPass2, TWO>, smem_bytes<kPass2>());
-        case kScore: return occupancy(k_score<DT, TWO, kStepsScore>, score_smem<kStepsScore>());
+        case kScore: return occupancy(k_score<DT, TWO, kStepsScore>, score_smem<kStepsScore>(), kMinBlocksScore, kFT);
         case kPass1C: return occupancy(k_transport<DT, kPass1C, TWO>, smem_bytes<kPass1C>());
         case kPass2C: return occupancy(k_transport<DT, kPass2C, TWO>, smem_bytes<kPass2C>());
         default: return occupancy(k_transport<DT, kPass1, TWO>, smem_bytes<kPass1>());
@@ -2101,10 +2122,10 @@ cudaError_t launch_transport_batch(const TransportArgs* table, int n, int mode, 
     switch (mode) {
         case kFwdVoxel:
             switch (trip) {
-                case 8: k_forward_batch<8><<<blocks, kTB, forward_smem(), st>>>(table, n); break;
-                case 10: k_forward_batch<10><<<blocks, kTB, forward_smem(), st>>>(table, n); break;
-                case 16: k_forward_batch<16><<<blocks, kTB, forward_smem(), st>>>(table, n); break;
-                default: k_forward_batch<kStepsForward><<<blocks, kTB, forward_smem(), st>>>(table, n);
+                case 12: k_forward_batch<12><<<blocks, kFT, forward_smem(), st>>>(table, n); break;
+                case 10: k_forward_batch<10><<<blocks, kFT, forward_smem(), st>>>(table, n); break;
+                case 16: k_forward_batch<16><<<blocks, kFT, forward_smem(), st>>>(table, n); break;
+                default: k_forward_batch<kStepsForward><<<blocks, kFT, forward_smem(), st>>>(table, n);
             }
             return cudaGetLastError();
         case kPass2: return launch_batch_mode<kPass2>(table, n, blocks, st);
@@ -2117,14 +2138,14 @@ int transport_batch_blocks_per_sm(int mode) {
     static int occ[7] = {0, 0, 0, 0, 0, 0, 0};
     static bool ready = false;
     if (!ready) {  // every instantiation's attributes, once; the default trips give the occupancy
-        occ[kFwdVoxel] = occupancy(k_forward_batch<kStepsForward>, forward_smem(), kMinBlocksForward);
-        occupancy(k_forward_batch<8>, forward_smem(), kMinBlocksForward);
-        occupancy(k_forward_batch<10>, forward_smem(), kMinBlocksForward);
-        occupancy(k_forward_batch<16>, forward_smem(), kMinBlocksForward);
-        occ[kScore] = occupancy(k_score_batch<kStepsScore>, score_smem<kStepsScore>());
-        occupancy(k_score_batch<4>, score_smem<4>());
-        occupancy(k_score_batch<8>, score_smem<8>());
-        occupancy(k_score_batch<10>, score_smem<10>());
+        occ[kFwdVoxel] = occupancy(k_forward_batch<kStepsForward>, forward_smem(), kMinBlocksForward, kFT);
+        occupancy(k_forward_batch<12>, forward_smem(), kMinBlocksForward, kFT);
+        occupancy(k_forward_batch<10>, forward_smem(), kMinBlocksForward, kFT);
+        occupancy(k_forward_batch<16>, forward_smem(), kMinBlocksForward, kFT);
+        occ[kScore] = occupancy(k_score_batch<kStepsScore>, score_smem<kStepsScore>(), kMinBlocksScore, kFT);
+        occupancy(k_score_batch<4>, score_smem<4>(), kMinBlocksScore, kFT);
+        occupancy(k_score_batch<8>, score_smem<8>(), kMinBlocksScore, kFT);
+        occupancy(k_score_batch<10>, score_smem<10>(), kMinBlocksScore, kFT);
         occ[kPass2] = batch_occupancy<kPass2>();
         occ[kPass1] = batch_occupancy<kPass1>();
         ready = true;
@@ -2134,10 +2155,10 @@ int transport_batch_blocks_per_sm(int mode) {
 
 cudaError_t launch_score_batch(const TransportArgs* table, int n, int trip, int blocks, cudaStream_t st) {
     switch (trip) {
-        case 4: k_score_batch<4><<<blocks, kTB, score_smem<4>(), st>>>(table, n); break;
-        case 8: k_score_batch<8><<<blocks, kTB, score_smem<8>(), st>>>(table, n); break;
-        case 10: k_score_batch<10><<<blocks, kTB, score_smem<10>(), st>>>(table, n); break;
-        default: k_score_batch<kStepsScore><<<blocks, kTB, score_smem<kStepsScore>(), st>>>(table, n);
+        case 4: k_score_batch<4><<<blocks, kFT, score_smem<4>(), st>>>(table, n); break;
+        case 8: k_score_batch<8><<<blocks, kFT, score_smem<8>(), st>>>(table, n); break;
+        case 10: k_score_batch<10><<<blocks, kFT, score_smem<10>(), st>>>(table, n); break;
+        default: k_score_batch<kStepsScore><<<blocks, kFT, score_smem<kStepsScore>(), st>>>(table, n);
     }
     return cudaGetLastError();
 }
@@ -2179,10 +2200,10 @@ namespace {
 template <int DT, bool TWO, int K>
 cudaError_t launch_score_k(const TransportArgs& a, int blocks, cudaStream_t st) {
     if constexpr (K != kStepsScore) {  // the default's attributes are set by occupancy()
-        static const int once = occupancy(k_score<DT, TWO, K>, score_smem<K>());
+        static const int once = occupancy(k_score<DT, TWO, K>, score_smem<K>(), kMinBlocksScore, kFT);
         (void)once;
     }
-    k_score<DT, TWO, K><<<blocks, kTB, score_smem<K>(), st>>>(a);
+    k_score<DT, TWO, K><<<blocks, kFT, score_smem<K>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -2208,13 +2229,14 @@ cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, i
 
 cudaError_t launch_fold_bricks(const mst_grid* g, cudaStream_t st) {
     const int nb = (brick_bins(g->geo) + 255) / 256;
-    k_fold_bricks<<<nb < 4096 ? nb : 4096, 256, 0, st>>>(g->gbrk, g->g64, g->geo);
+    k_fold_bricks<<<nb < 4096 ? nb : 4096, 256, 0, st>>>(g->gbrk, g->g64, g->geo, (int)g->score_tiles);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fold_L(const mst_grid* g, cudaStream_t st) {
-    const int nb = (g->geo.nvox + 255) / 256;
-    k_fold_L<<<nb < 4096 ? nb : 4096, 256, 0, st>>>(g->Lacc, g->L64, g->geo.nvox, g->n_cams, g->cp);
+    const int nb = (g->geo.nvox + kFoldRows - 1) / kFoldRows;
+    const size_t smem = sizeof(float) * kFoldRows * (g->cp + 1);
+    k_fold_L<<<nb < 4096 ? nb : 4096, kTB, smem, st>>>(g->Lacc, g->L64, g->geo.nvox, g->n_cams, g->cp);
     return cudaGetLastError();
 }
 
