@@ -126,7 +126,6 @@ TransportArgs transport_args(mst_grid* g, const mst_params* p) {
     a.hg.opg = (float)(1.0 + gg);
     a.hg.tg = (float)(2.0 * gg);
     a.hg.iso = std::fabs(gg) < 1e-6;
-    a.beta = g->ext;
     a.beta_pad = g->ext_pad;
     a.beta_air = g->air;  // two species (Sec. 2): the particle of each event is drawn
     a.beta_aer = g->air ? g->beta_in : nullptr;
@@ -164,12 +163,9 @@ TransportArgs transport_args(mst_grid* g, const mst_params* p) {
     return a;
 }
 
-// Rolling-fold slicing of a tile of `bins` bins (see kFoldSweep) for a launch of n photons: slices of
-// a multiple of 32 bins, at least 128, such that one sweep takes at most about kFoldSweep photons.
-// A launch of no more photons than that leaves its tile to the fold that follows it.
-void set_fold(TransportArgs& a, uint64_t bins, uint64_t n) {
-    a.fold_bins = 0;
-    if (n <= kFoldSweep) return;
+// Rolling-fold slicing of a tile of `bins` bins (see kFoldSweep): slices of a multiple of 32
+// bins, at least 128, such that one sweep takes at most about kFoldSweep photons.
+void set_fold(TransportArgs& a, uint64_t bins) {
     const uint64_t batches = kFoldSweep / kTicketBatch;
     uint64_t slice = (bins + batches - 1) / batches;
     slice = std::max<uint64_t>(128, (slice + 31) / 32 * 32);
@@ -180,9 +176,7 @@ void set_fold(TransportArgs& a, uint64_t bins, uint64_t n) {
 
 // The score kernel folds one slice of its brick tile per chunk of stored events. A photon makes
 // a few events at most on average; counting one per photon keeps a sweep within kFoldSweep photons.
-void set_score_fold(TransportArgs& a, uint64_t n) {
-    a.fold_bins = 0;
-    if (n <= kFoldSweep) return;
+void set_score_fold(TransportArgs& a) {
     const uint64_t bins = (uint64_t)brick_bins(a.g) * a.score_tiles, chunks = kFoldSweep / kEventChunk;
     const uint64_t slice = std::max<uint64_t>(32, ((bins + chunks - 1) / chunks + 31) / 32 * 32);
     a.fold_bins = bins;
@@ -211,8 +205,8 @@ int run_photons(mst_grid* g, const mst_params* p, bool replay, double* cimg, cud
     const int b_fwd = transport_blocks(g, p->grid_dtype, est);
     const int b_p1 = transport_blocks(g, p->grid_dtype, m_p1);
     const int b_p2 = transport_blocks(g, p->grid_dtype, m_p2);
-    if (replay) set_fold(a, (uint64_t)g->geo.npad, n);
-    else if (est == MST_EST_VOXEL) set_fold(a, (uint64_t)g->geo.nvox * g->cp, n);
+    if (replay) set_fold(a, (uint64_t)g->geo.npad);
+    else if (est == MST_EST_VOXEL) set_fold(a, (uint64_t)g->geo.nvox * g->cp);
     if (store_events) {
         a.evrec = g->evrec;
         a.ev_cap = g->ev_cap;
@@ -286,12 +280,12 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
     auto blocks = [&](int mode) { return transport_blocks(g, p->grid_dtype, mode); };
     {
         Phase ph(g, MST_PH_REPLAY2, st);
-        set_score_fold(a, n);
+        set_score_fold(a);
         a.ticket = g->tickets + 2;  // its warps take the forward warps' lists from it
         MST_CK(launch_score(g, a, p->grid_dtype, blocks(4), st));
         MST_CK(launch_fold_bricks(g, st));
     }
-    set_fold(a, (uint64_t)g->geo.npad, n);
+    set_fold(a, (uint64_t)g->geo.npad);
     a.ticket = g->tickets;
     {
         Phase ph(g, MST_PH_REPLAY, st);  // these return at once when the events fitted
@@ -609,7 +603,6 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         void** p;
         size_t bytes;
     } allocs[] = {
-        {&g->ext, nvox * 4},
         {&g->ext_pad, (size_t)geo.npad * 4},
         {(void**)&g->Lacc, nvox * g->cp * 4},
         {(void**)&g->L64, C * nvox * 8},
@@ -1340,7 +1333,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         const mst_params* p = &params[i];
         g->beta_in = betas[i];
         TransportArgs f = transport_args(g, p);
-        set_fold(f, (uint64_t)g->geo.nvox * g->cp, p->n_photons);
+        set_fold(f, (uint64_t)g->geo.nvox * g->cp);
         f.evrec = g->evrec;
         f.ev_cap = g->ev_cap;
         f.ev_count = g->ev_count;
@@ -1353,7 +1346,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         f.ticket = g->tickets;
         t[i] = f;
         TransportArgs r = transport_args(g, p);
-        set_score_fold(r, p->n_photons);
+        set_score_fold(r);
         r.evrec = g->evrec;
         r.ev_cap = g->ev_cap;
         r.ev_count = g->ev_count;
@@ -1365,7 +1358,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         r.n = (uint32_t)p->n_photons;
         r.ticket = g->tickets + 2;  // the score kernel's warps take the forward warps' lists from it
         t[n + i] = r;
-        set_fold(r, (uint64_t)g->geo.npad, p->n_photons);
+        set_fold(r, (uint64_t)g->geo.npad);
         r.ticket = g->tickets;      // pass 1 (returns at once when the events fitted)
         t[2 * n + i] = r;
         r.ticket = g->tickets + 1;  // pass 2

@@ -60,8 +60,7 @@ struct TransportArgs {
     Geo g;
     CamSet cams;
     HG hg;
-    const void* beta;          // staged extinction [nvox] in the compute dtype (camera and shadow rays)
-    const void* beta_pad;      // the same on the padded grid of the flights (halo +inf)
+    const void* beta_pad;      // staged extinction in the compute dtype on the padded grid (halo +inf)
     const float* beta_air;     // two species: air extinction [nvox] (NULL: one species)
     const float* beta_aer;     // two species: aerosol extinction [nvox], the unknown
     float3 sun;                // photon direction at launch
@@ -117,7 +116,7 @@ struct mst_grid {
     double voxel_volume = 0;
 
     // device buffers owned by the handle
-    void* ext = nullptr;          // staged extinction [nvox], up to 4 bytes per voxel
+    void* ext = nullptr;          // staged extinction [nvox] of a call without a handle (mst_transmittance_noalloc)
     void* ext_pad = nullptr;      // staged extinction on the padded grid [npad] (photon flights)
     float* Lacc = nullptr;        // [nvox][cp]
     double* L64 = nullptr;        // [C][nvox]

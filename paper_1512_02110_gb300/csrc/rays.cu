@@ -19,24 +19,18 @@ constexpr int kRayBlock = 256;  // threads of a pixel-ray block (n_rays <= 64 di
 // threads of a block that hold a ray: the largest multiple of n_rays within kRayBlock
 __host__ __device__ __forceinline__ int pixel_rays_block(int n_rays) { return kRayBlock / n_rays * n_rays; }
 
-// The extinction grid in the compute dtype, in the linear voxel order of the input.
-template <int DT>
-__global__ void k_stage(const float* __restrict__ beta, const float* __restrict__ air, void* __restrict__ ext,
-                        float* __restrict__ tot, int nvox) {
-    typedef typename BetaFetch<DT>::T T;
-    T* out = static_cast<T*>(ext);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nvox; k += gridDim.x * blockDim.x) {
-        const float b = air ? beta[k] + air[k] : beta[k];  // Sec. 2: beta = beta_aerosol + beta_air
-        out[k] = BetaFetch<DT>::make(b);
-        if (tot) tot[k] = b;  // two species: the FP32 total for the surrogate's j = L / beta
-    }
+// The extinction in FP32 in the linear voxel order of the input, for the call without a handle.
+__global__ void k_stage(const float* __restrict__ beta, float* __restrict__ ext, int nvox) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nvox; k += gridDim.x * blockDim.x) ext[k] = beta[k];
 }
 
-// The grid of the photon flights: the same values on [nz + 4][ny + 4][nx + 4] with a halo of
-// +inf extinction, where a flight stops (a free path never outlasts infinite optical depth).
+// The grid that every ray and flight walks: the extinction in the compute dtype on
+// [nz + 4][ny + 4][nx + 4] with a halo of +inf, where a walk stops (a free path never outlasts
+// infinite optical depth). Two species (Sec. 2): beta = beta_aerosol + beta_air, and the FP32 total
+// for the surrogate's j = L / beta.
 template <int DT>
 __global__ void k_stage_pad(const float* __restrict__ beta, const float* __restrict__ air, void* __restrict__ ext,
-                            const Geo g) {
+                            float* __restrict__ tot, const Geo g) {
     typedef typename BetaFetch<DT>::T T;
     T* out = static_cast<T*>(ext);
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.npad; q += gridDim.x * blockDim.x) {
@@ -45,6 +39,7 @@ __global__ void k_stage_pad(const float* __restrict__ beta, const float* __restr
         if (ix >= 0 && ix < g.nx && iy >= 0 && iy < g.ny && iz >= 0 && iz < g.nz) {
             const int k = lin_index(g, ix, iy, iz);
             b = air ? beta[k] + air[k] : beta[k];
+            if (tot) tot[k] = b;
         }
         out[q] = BetaFetch<DT>::make(b);
     }
@@ -66,64 +61,6 @@ __device__ __forceinline__ void block_count(double* stats, int slot, unsigned n)
     if ((threadIdx.x & 31u) == 0u && n) atomicAdd(&total, n);
     __syncthreads();
     if (threadIdx.x == 0 && total) atomicAdd(stats + slot, (double)total);
-}
-
-// A sum of FP32 terms held as an unevaluated pair hi + lo: each addition's rounding error is
-// recovered exactly (Knuth's TwoSum, six additions) and summed beside it, so n terms keep about
-// 48 - log2(n) bits. This chip's FP64 pipe takes 2.6e11 conversions with their additions a second
-// against 3.2e13 FP32 operations, and the ray kernels add one term per voxel segment: k_los took
-// 0.93 ms for 1.8e8 segments with FP64 sums, 0.32 ms with this and the walk below.
-struct PairSum {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(hi, x);
-        const float t = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
-        hi = s;
-    }
-    // an infinite or NaN sum has no error term
-    __device__ __forceinline__ double value() const { return isfinite(lo) ? (double)hi + (double)lo : (double)hi; }
-};
-
-// A camera ray or line of sight on the padded grid (its halo tells the walk that it has left): per
-// axis the distance to the next face (t), between faces (q) and the padded index's change at a
-// crossing, and the current padded index. The distances are those of axis_init with the rounded
-// division, and a step moves them as walk_step does; the voxel indices, the three bounds tests and
-// the exit face of that walk are gone.
-struct PadWalk {
-    float tx, ty, tz, qx, qy, qz;
-    int dx, dy, dz, lin;
-
-    static __device__ __forceinline__ void axis(float p, float d, float h, int stride, float& t, float& q, int& dl) {
-        float a;
-        int s;
-        axis_init<false>(p, d, h, t, q, a, s);
-        dl = s * stride;
-    }
-    // from offset p of voxel `at` of a grid with the strides 1, sy, sz
-    __device__ __forceinline__ PadWalk(const Geo& g, float3 p, float3 d, int at, int sy, int sz) : lin(at) {
-        axis(fminf(fmaxf(p.x, 0.f), g.hx), d.x, g.hx, 1, tx, qx, dx);
-        axis(fminf(fmaxf(p.y, 0.f), g.hy), d.y, g.hy, sy, ty, qy, dy);
-        axis(fminf(fmaxf(p.z, 0.f), g.hz), d.z, g.hz, sz, tz, qz, dz);
-    }
-    // distance to the next face, the axis it belongs to (ties to x, then y, then z), the voxel behind it
-    __device__ __forceinline__ float face(bool& px, bool& py, int& next) const {
-        const float m = fminf(tx, fminf(ty, tz));
-        px = tx <= m;
-        py = !px && ty <= m;
-        next = lin + (px ? dx : (py ? dy : dz));
-        return m;
-    }
-    __device__ __forceinline__ void cross(float m, bool px, bool py, int next) {
-        tx = px ? qx : tx - m;
-        ty = py ? qy : ty - m;
-        tz = (px || py) ? tz - m : qz;
-        lin = next;
-    }
-};
-
-__device__ __forceinline__ PadWalk pad_walk(const Geo& g, float3 p, float3 d, int ix, int iy, int iz) {
-    return PadWalk(g, p, d, pad_index(g, ix, iy, iz), g.p0, g.p01);
 }
 
 // R is stored on the padded grid with this bit pattern in its halo, which no arithmetic produces
@@ -182,32 +119,29 @@ __global__ void __launch_bounds__(kTB) k_los(const Geo g, const CamSet cs, const
             const int goal = !cm.inside ? -1 : (PAD ? pad_index(g, cm.ix, cm.iy, cm.iz) : lin_index(g, cm.ix, cm.iy, cm.iz));
             PadWalk w(g, p, d, PAD ? pad_index(g, ix, iy, iz) : k, PAD ? g.p0 : g.nx, PAD ? g.p01 : g.nx * g.ny);
             int lx = d.x > 0.f ? g.nx - 1 - ix : ix, ly = d.y > 0.f ? g.ny - 1 - iy : iy, lz = d.z > 0.f ? g.nz - 1 - iz : iz;
-            float bn = PAD ? BetaFetch<DT>::get(ext, w.lin) : 0.f;
-            for (;;) {
-                const float b = PAD ? bn : BetaFetch<DT>::get(ext, w.lin);
-                if (PAD && isinf(b)) {  // the halo, unless the field itself is infinite here
-                    int q;
-                    if (!interior_lin(g, w.lin, q)) break;
-                }
-                ++nseg;
-                bool px, py;
-                int next;
-                const float m = w.face(px, py, next);
+            float b, m, bn = BetaFetch<DT>::get(ext, w.lin);
+            bool px, py;
+            int next;
+            for (;;) {  // one exit, whatever ends the walk: the loop is bound by its instructions
+                b = bn;
+                m = w.face(px, py, next);
                 if (PAD) bn = BetaFetch<DT>::get(ext, next);  // the walk stands inside: next is at most in the halo
-                if (w.lin == goal) {
-                    const float len = camera_leg(g, cm, w, d, p);
-                    tau.add(__fmul_rn(b, fminf(fmaxf(len, 0.f), rem)));
-                    break;
-                }
-                if (m >= rem) {
-                    tau.add(__fmul_rn(b, rem));
-                    break;
-                }
+                if ((PAD && isinf(b)) || w.lin == goal || m >= rem || nseg >= (unsigned)g.max_steps) break;
+                ++nseg;
                 tau.add(__fmul_rn(b, m));
                 rem -= m;
-                if (nseg > (unsigned)g.max_steps) break;
-                if (!PAD && (px ? lx-- : (py ? ly-- : lz--)) == 0) break;
+                if (!PAD && (px ? lx-- : (py ? ly-- : lz--)) == 0) {  // out of the grid
+                    m = -1.f;
+                    break;
+                }
                 w.cross(m, px, py, next);
+                if (!PAD) bn = BetaFetch<DT>::get(ext, w.lin);
+            }
+            int q;
+            if (m >= 0.f && (!PAD || !isinf(b) || interior_lin(g, w.lin, q))) {  // not in the halo: the last voxel
+                ++nseg;
+                if (w.lin == goal) m = fmaxf(camera_leg(g, cm, w, d, p), 0.f);
+                tau.add(__fmul_rn(b, fminf(m, rem)));
             }
         }
         const float T = (float)exp(-tau.value());
@@ -369,21 +303,24 @@ __global__ void __launch_bounds__(kTB) k_los_adjoint(const Geo g, const CamSet c
         if (s != 0.f && los_dir(g, cm, ix, iy, iz, p, d, rem)) {
             const int goal = camera_lin(g, cm);
             PadWalk w = pad_walk(g, p, d, ix, iy, iz);
-            float rn = __ldg(Rc + w.lin);
-            while (__float_as_int(rn) != kOutside) {
-                ++nseg;
-                bool px, py;
-                int next;
-                const float m = w.face(px, py, next);
+            float m, r, rn = __ldg(Rc + w.lin);
+            bool px, py;
+            int next;
+            for (;;) {
+                r = rn;
+                m = w.face(px, py, next);
                 rn = __ldg(Rc + next);
-                float len = m;
-                const bool at_camera = w.lin == goal;
-                if (at_camera) len = fminf(fmaxf(camera_leg(g, cm, w, d, p), 0.f), rem);
-                else if (m >= rem) len = rem;
-                if (len > 0.f) atomicAdd(gc + w.lin, s * len);
-                if (at_camera || m >= rem || nseg > (unsigned)g.max_steps) break;
+                if (__float_as_int(r) == kOutside || w.lin == goal || m >= rem || nseg >= (unsigned)g.max_steps) break;
+                ++nseg;
+                if (m > 0.f) atomicAdd(gc + w.lin, s * m);
                 rem -= m;
                 w.cross(m, px, py, next);
+            }
+            if (__float_as_int(r) != kOutside) {  // the last voxel
+                ++nseg;
+                if (w.lin == goal) m = fmaxf(camera_leg(g, cm, w, d, p), 0.f);
+                m = fminf(m, rem);
+                if (m > 0.f) atomicAdd(gc + w.lin, s * m);
             }
         }
     }
@@ -524,18 +461,16 @@ inline int nblocks(long long n, int tb = kTB, int cap = 1 << 20) {
 }  // namespace
 
 cudaError_t launch_stage(const mst_grid* g, const float* beta, const float* air, int dtype, cudaStream_t st) {
-    const int nvox = g->geo.nvox;
-    const int nb = nblocks(nvox, kTB, 8192);
-    float* tot = air ? g->btot : nullptr;
-    if (dtype == 0) k_stage<0><<<nb, kTB, 0, st>>>(beta, air, g->ext, tot, nvox);
-    else if (dtype == 1) k_stage<1><<<nb, kTB, 0, st>>>(beta, air, g->ext, tot, nvox);
-    else k_stage<2><<<nb, kTB, 0, st>>>(beta, air, g->ext, tot, nvox);
-    if (g->ext_pad) {
-        const int np = nblocks(g->geo.npad, kTB, 4096);
-        if (dtype == 0) k_stage_pad<0><<<np, kTB, 0, st>>>(beta, air, g->ext_pad, g->geo);
-        else if (dtype == 1) k_stage_pad<1><<<np, kTB, 0, st>>>(beta, air, g->ext_pad, g->geo);
-        else k_stage_pad<2><<<np, kTB, 0, st>>>(beta, air, g->ext_pad, g->geo);
+    if (!g->ext_pad) {  // mst_transmittance_noalloc: FP32, one species
+        if (dtype != 0 || air) return cudaErrorInvalidValue;
+        k_stage<<<nblocks(g->geo.nvox, kTB, 8192), kTB, 0, st>>>(beta, static_cast<float*>(g->ext), g->geo.nvox);
+        return cudaGetLastError();
     }
+    float* tot = air ? g->btot : nullptr;
+    const int np = nblocks(g->geo.npad, kTB, 4096);
+    if (dtype == 0) k_stage_pad<0><<<np, kTB, 0, st>>>(beta, air, g->ext_pad, tot, g->geo);
+    else if (dtype == 1) k_stage_pad<1><<<np, kTB, 0, st>>>(beta, air, g->ext_pad, tot, g->geo);
+    else k_stage_pad<2><<<np, kTB, 0, st>>>(beta, air, g->ext_pad, tot, g->geo);
     return cudaGetLastError();
 }
 

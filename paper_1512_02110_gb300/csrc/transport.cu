@@ -1676,7 +1676,7 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
             prev = A.ch_prev[ch];
             base = (int)kEvChunk - 32;
             // one slice of the rolling fold (see kFoldSweep) per chunk
-            const uint32_t i0 = A.fold_bins ? ch % A.fold_nslices * A.fold_slice : 0u;
+            const uint32_t i0 = ch % A.fold_nslices * A.fold_slice;
             const uint32_t i1 = min(i0 + A.fold_slice, (uint32_t)A.fold_bins);
             for (uint32_t i = i0 + lane; i < i1; i += 32) {
                 const float v = atomicExch(A.gbrk + i, 0.f);
