@@ -283,7 +283,6 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
         set_score_fold(a);
         a.ticket = g->tickets + 2;  // its warps take the forward warps' lists from it
         MST_CK(launch_score(g, a, p->grid_dtype, blocks(4), st));
-        MST_CK(launch_fold_bricks(g, st));
     }
     set_fold(a, (uint64_t)g->geo.npad);
     a.ticket = g->tickets;
@@ -294,9 +293,7 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
         a.ticket = g->tickets + 1;
         MST_CK(launch_transport(g, a, p->grid_dtype, 2, blocks(2), st));
     }
-    Phase ph(g, MST_PH_FOLD, st);
-    MST_CK(launch_fold_grad(g, st));
-    return MST_OK;
+    return MST_OK;  // what is left in the tiles is folded by launch_combine_full
 }
 
 // Per-photon buffers of the replay for n photons (at least kReplayChunk), allocated by the
@@ -783,7 +780,7 @@ int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const 
         if (rc) return rc;
         {
             Phase ph(g, MST_PH_COMBINE, st);
-            MST_CK(launch_combine_full(g, nullptr, g->g64, grad, st));
+            MST_CK(launch_combine_full(g, nullptr, g->g64, false, grad, st));
         }
         if (p->reg_eta != 0.0) {
             Phase ph(g, MST_PH_COMBINE, st);
@@ -847,7 +844,7 @@ int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const 
         if (rc) return rc;
         {
             Phase ph(g, MST_PH_COMBINE, st);
-            MST_CK(launch_combine_full(g, g->gT, g->g64, grad, st));
+            MST_CK(launch_combine_full(g, g->gT, g->g64, stored, grad, st));
         }
     }
     if (p->reg_eta != 0.0) {
@@ -1457,9 +1454,7 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
     for (int i = 0; i < n; ++i) {
         g = b->grids[i];
         cudaStream_t st = b->branch[i];
-        MST_CK(launch_fold_bricks(g, st));
-        MST_CK(launch_fold_grad(g, st));
-        MST_CK(launch_combine_full(g, g->gT, g->g64, grads[i], st));
+        MST_CK(launch_combine_full(g, g->gT, g->g64, true, grads[i], st));
         if (params[i].reg_eta != 0.0)
             MST_CK(launch_regularizer(g, betas[i], params[i].reg_eta, g->lap, g->stats + MST_NSTATS + 1, losses + i,
                                       grads[i], st));

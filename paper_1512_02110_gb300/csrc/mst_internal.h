@@ -202,10 +202,8 @@ cudaError_t launch_fold_L(const mst_grid* g, cudaStream_t st);
 cudaError_t launch_fold_grad(const mst_grid* g, cudaStream_t st);
 // the pass-2 list; with `stored` its kernels return at once when the stored events fitted
 cudaError_t launch_score_list(const mst_grid* g, uint32_t n, bool stored, cudaStream_t st);
-// the score gradient from the stored events (returns at once when they did not fit), and what it
-// left in the brick tile
+// the score gradient from the stored events (returns at once when they did not fit)
 cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, int blocks, cudaStream_t st);
-cudaError_t launch_fold_bricks(const mst_grid* g, cudaStream_t st);
 // backward MC images (Eq. ble): n paths per pixel, sums into sum / sum2, then sum <- means and
 // var <- variances of the means (var may be NULL)
 cudaError_t launch_bmc(const mst_grid* g, const mst_params* p, uint32_t n, double* sum, double* sum2, double* var,
@@ -221,7 +219,10 @@ cudaError_t launch_adjoint_tiles(const mst_grid* g, const float* T, const float*
 cudaError_t launch_combine_surrogate(const mst_grid* g, const double* Lsrc, const double* jfix, const float* beta_ref,
                                      const float* beta, const float* T, const float* bacc, const float* gT,
                                      const float* Qw, double* grad, cudaStream_t st);
-cudaError_t launch_combine_full(const mst_grid* g, const float* gT, const double* gL, double* grad, cudaStream_t st);
+// grad = gL - sum_c gT_c; with `tiles`, gL is first given what the score kernel and pass 2 left in
+// their tiles, which are cleared
+cudaError_t launch_combine_full(const mst_grid* g, const float* gT, const double* gL, bool tiles, double* grad,
+                                cudaStream_t st);
 cudaError_t launch_classic_residual(const mst_grid* g, const double* img, const double* meas, const uint8_t* mask,
                                     double* resid, double* loss, cudaStream_t st);
 cudaError_t launch_regularizer(const mst_grid* g, const float* beta, double eta, double* lap, double* psi,

@@ -251,6 +251,7 @@ __global__ void k_images(const Geo g, const CamSet cs, const Halton hs, float in
 // terms up before the atomic took 0.27 ms and was not kept: the bins next to a camera sum so
 // many terms in FP32 that grouped additions move them by 1e-4.
 constexpr int kPixelStride = 4;
+constexpr int kRaysApart = 1 << 15;  // pixels below which the rays of a pixel go to threads of their own
 __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet cs, const Halton hs, float inv_nv,
                                                      const double* __restrict__ resid, const float* __restrict__ R,
                                                      float* __restrict__ bacc, int total_pix, double* stats) {
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet c
         const int c = cam_of_pixel(cs, gp);
         const float* Rc = R + (size_t)c * g.npad;
         float* bc = bacc + (size_t)c * g.npad;
-        for (int rho = 0; rho < hs.n; ++rho) {
+        for (int rho = blockIdx.y; rho < hs.n; rho += gridDim.y) {
             float3 p, d;
             int ix, iy, iz;
             if (!pixel_ray_start(g, cs.c[c], hs, gp, rho, p, d, ix, iy, iz)) continue;
@@ -389,15 +390,34 @@ __global__ void k_combine_surrogate(const Geo g, const double* __restrict__ Lsrc
     }
 }
 
-// full: grad(m) = gL(m) - sum_c gT_c(m)
+// full: grad(m) = gL(m) - sum_c gT_c(m). With the tiles of a stored-event replay (gbrk not NULL), gL
+// lacks what the score kernel left in the copies of its brick tile and pass 2 in its padded tile:
+// both are added here and cleared (one launch instead of three).
 __global__ void k_combine_full(const Geo g, const float* __restrict__ gT, const double* __restrict__ gL,
+                               float* __restrict__ gbrk, int copies, float* __restrict__ gacc,
                                double* __restrict__ grad, int C) {
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < g.nvox; k += gridDim.x * blockDim.x) {
+        const int ix = k % g.nx, iy = (k / g.nx) % g.ny, iz = k / (g.nx * g.ny);
+        const int at = pad_index(g, ix, iy, iz);
         double acc = gL[k];
-        if (gT) {  // voxel estimator: the LOS term; the classic estimator has none
-            const int at = pad_of(g, k);
-            for (int c = 0; c < C; ++c) acc -= (double)gT[(size_t)c * g.npad + at];
+        if (gbrk) {
+            const size_t nb = (size_t)brick_bins(g);
+            float* x = gbrk + brick_bin(g, (unsigned)ix, (unsigned)iy, (unsigned)iz);
+            for (int t = 0; t < copies; ++t) {
+                const float v = x[t * nb];
+                if (v != 0.f) {
+                    acc += (double)v;
+                    x[t * nb] = 0.f;
+                }
+            }
+            const float v = gacc[at];
+            if (v != 0.f) {
+                acc += (double)v;
+                gacc[at] = 0.f;
+            }
         }
+        if (gT)  // voxel estimator: the LOS term; the classic estimator has none
+            for (int c = 0; c < C; ++c) acc -= (double)gT[(size_t)c * g.npad + at];
         grad[k] = acc;
     }
 }
@@ -516,7 +536,10 @@ cudaError_t launch_backproject(const mst_grid* g, const double* resid, float* ba
     const float inv_nv = (float)(1.0 / (g->n_rays * g->voxel_volume));
     const int group = 32 * kPixelStride;  // pixels of kPixelStride warps
     const int warps = (g->total_pix + group - 1) / group * kPixelStride;
-    k_backproject<<<(warps + kTB / 32 - 1) / (kTB / 32), kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, g->R, bacc,
+    // few pixels leave the chip to single threads' chains of rays: a thread per ray then (5 cameras of
+    // 32^2 pixels in 16^3 voxels: 48 us against 36)
+    const dim3 nb((warps + kTB / 32 - 1) / (kTB / 32), g->total_pix < kRaysApart ? g->n_rays : 1);
+    k_backproject<<<nb, kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, g->R, bacc,
                                                                        g->total_pix, g->stats);
     return cudaGetLastError();
 }
@@ -549,8 +572,10 @@ cudaError_t launch_combine_surrogate(const mst_grid* g, const double* Lsrc, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_combine_full(const mst_grid* g, const float* gT, const double* gL, double* grad, cudaStream_t st) {
-    k_combine_full<<<nblocks(g->geo.nvox, kTB, 4096), kTB, 0, st>>>(g->geo, gT, gL, grad, g->n_cams);
+cudaError_t launch_combine_full(const mst_grid* g, const float* gT, const double* gL, bool tiles, double* grad,
+                                cudaStream_t st) {
+    k_combine_full<<<nblocks(g->geo.nvox, kTB, 4096), kTB, 0, st>>>(g->geo, gT, gL, tiles ? g->gbrk : nullptr,
+                                                                    (int)g->score_tiles, g->gacc, grad, g->n_cams);
     return cudaGetLastError();
 }
 

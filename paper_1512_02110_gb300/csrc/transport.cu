@@ -1446,7 +1446,7 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
         __syncwarp();
 
         const int fly_n = __popc(fly);
-        // (4) events, 32 at a time; while the warp drains, whatever is queued as soon as no photon is ready
+        // (4) events, 32 at a time; while the warp drains, whatever is queued once no photon is ready
         while (ev_n >= 32 || (ev_n > 0 && dry && rd_n == 0 && fly_n <= kDrain * ev_n)) {
             const int n = min(32, ev_n);
             unsigned long long ev_slot = 0ull;  // storing events: this lane's record slot
@@ -1975,20 +1975,6 @@ __global__ void k_fold_grad(float* __restrict__ gacc, double* __restrict__ g64, 
     }
 }
 
-// what the score kernel left in its brick tile
-__global__ void k_fold_bricks(float* __restrict__ gbrk, double* __restrict__ g64, const Geo g, int tiles) {
-    const int nb = brick_bins(g);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += gridDim.x * blockDim.x) {
-        double v = 0.0;
-        for (int t = 0; t < tiles; ++t) {
-            v += (double)gbrk[(size_t)t * nb + i];
-            gbrk[(size_t)t * nb + i] = 0.f;
-        }
-        int k;
-        if (v != 0.0 && brick_voxel(g, i, k)) g64[k] += v;
-    }
-}
-
 // dynamic shared memory of a transport block: the warps' photon stacks, the forward's tallies
 // and the classic estimate's scratch
 template <int MODE>
@@ -2225,12 +2211,6 @@ cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, i
     const int trip = g->wf_trip[kScore];
     return a.beta_air ? launch_score_dt<true>(a, dtype, trip, blocks, st)
                       : launch_score_dt<false>(a, dtype, trip, blocks, st);
-}
-
-cudaError_t launch_fold_bricks(const mst_grid* g, cudaStream_t st) {
-    const int nb = (brick_bins(g->geo) + 255) / 256;
-    k_fold_bricks<<<nb < 4096 ? nb : 4096, 256, 0, st>>>(g->gbrk, g->g64, g->geo, (int)g->score_tiles);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_fold_L(const mst_grid* g, cudaStream_t st) {
