@@ -67,12 +67,13 @@ enum {
     MST_ST_REPLAY_SCATTERS = 22,
     MST_ST_LOST = 23, /* walks abandoned (non-finite direction), or replay flights that missed their stored
                          event's voxel; 0 in valid use */
-    MST_ST_EVENTS_STORED = 24, /* full gradient: events the forward stored for the adjoint (0: replayed instead) */
+    MST_ST_EVENTS_STORED = 24, /* full gradient of the voxelised estimator: stored events the score read (0:
+                                  replayed instead) */
     MST_ST_BMC_PATHS = 25, MST_ST_BMC_EVENTS = 26, MST_ST_BMC_SEGMENTS = 27, /* mst_render_bmc: flight + sun-ray voxels */
     MST_ST_AIR_EVENTS = 28, /* two-species medium (mst_set_air): forward events whose particle was air */
     MST_ST_SHADOW_RAYS = 29, MST_ST_SHADOW_SEGMENTS = 30 /* classic estimator (Eq. fle): shadow rays walked by the
                                                             call's transport passes, and their voxel segments (the
-                                                            scatter walk of replay pass 2 counted again) */
+                                                            gradient's scatter walk counted again) */
 };
 
 /* phases timed by the profiler (mst_get_phase_times) */
@@ -80,9 +81,10 @@ enum {
     MST_PH_STAGE = 0, MST_PH_TRANSPORT = 1, MST_PH_FOLD = 2, MST_PH_LOS = 3, MST_PH_IMAGES = 4,
     MST_PH_BACKPROJECT = 5, MST_PH_LOS_ADJOINT = 6, MST_PH_REPLAY = 7, MST_PH_COMBINE = 8, MST_PH_REPLAY2 = 9,
     MST_PH_REPLAY_LIST = 10, MST_PH_EVENT_ADJOINT = 11, MST_PH_BMC = 12,
-    MST_NPHASES = 13 /* MST_PH_REPLAY: replay pass 1 (W per photon); MST_PH_EVENT_ADJOINT: W per photon from
-                        the events the forward stored (instead of pass 1); MST_PH_REPLAY_LIST: the list of
-                        photons with W != 0 that pass 2 walks; MST_PH_REPLAY2: pass 2 (scatter) */
+    MST_NPHASES = 13 /* MST_PH_REPLAY2: the score gradient, from the stored events or by replay pass 2;
+                        MST_PH_REPLAY: replay pass 1 (W per photon; after a score from stored events: the
+                        launches that only work when they did not fit); MST_PH_REPLAY_LIST: the list of
+                        photons with W != 0 that pass 2 walks; MST_PH_EVENT_ADJOINT: unused */
 };
 
 typedef struct mst_grid mst_grid; /* opaque; owned by the library */
@@ -166,13 +168,12 @@ int mst_render(mst_grid *g, const float *beta_dev, const mst_params *p, double *
  * Eq. Jaco1, Eq. TcofJaco1, Eq. DivTc) and conditioning Q_c.
  * MST_GRAD_FULL: the full gradient of Eq. DirectJacob applied to the residual, where
  * dL/dbeta is estimated by the score of the free-flight density (Eq. beer-lambert,
- * Eq. MCextinct) over paths replayed from their Philox keys. W = sum_s w_s per photon and the
- * w_s come from the events the forward render stored (44 B per event, within the handle's
- * budget, see mst_set_replay_memory), or, when they do not fit, from a first replay of every
- * path; a last replay scatters the score. Results agree either way. With MST_EST_CLASSIC the
+ * Eq. MCextinct) along every path, from the events the forward render stored (48 B per event,
+ * within the handle's budget, see mst_set_replay_memory), or, when they do not fit, by two replays
+ * of the paths from their Philox keys. Results agree either way. With MST_EST_CLASSIC the
  * images are Eq. fle's, w_s weights each camera's classic contribution by its pixel's dE/di,
- * and each contribution's shadow ray adds its own term (no events are stored). The surrogate
- * gradient needs the voxel estimator. */
+ * and each contribution's shadow ray adds its own term. The surrogate gradient needs the voxel
+ * estimator. */
 int mst_render_grad(mst_grid *g, const float *beta_dev, const mst_params *p, const double *images_meas_dev,
                     const uint8_t *mask_dev, double *images_dev, double *grad_dev, double *loss_dev, void *stream);
 
@@ -293,12 +294,13 @@ int mst_render_grad_channels(mst_grid *g, const float *beta_aer_dev, int n_chann
 
 /* Wavefront shape of the persistent transport kernels on this handle: the voxels a flying lane
  * advances per loop trip, and the resident blocks per SM, for the forward render (voxel
- * estimator) and for replay pass 2. 0 keeps the built-in default (12 and 6 voxels; the
- * register budget's occupancy, 3 blocks). The trip is a compile-time constant of the kernels:
- * forward trips 8, 10, 12, 16 and pass-2 trips 4, 6, 8, 10 are built, for the FP32 grid (the
- * FP16 / BF16 grids use the defaults). Results do not depend on the shape beyond the order of
- * floating-point additions: each photon's path is fixed by its Philox key. Blocks per SM in
- * 0..8 (more than the occupancy runs at the occupancy); other trips return MST_ERR_INVALID_ARG. */
+ * estimator) and for the score of the stored events (replay pass 2 when there are none). 0 keeps
+ * the built-in default (8 and 6 voxels; the register budget's occupancy, 4 blocks of 7 warps). The
+ * trip is a compile-time constant of the kernels: forward trips 8, 10, 12, 16 and score trips 4,
+ * 6, 8, 10 are built, for the FP32 grid (the FP16 / BF16 grids use the defaults). Results do not
+ * depend on the shape beyond the order of floating-point additions: each photon's path is fixed by
+ * its Philox key. Blocks per SM in 0..8 (more than the occupancy runs at the occupancy); other trips
+ * return MST_ERR_INVALID_ARG. */
 int mst_set_wavefront(mst_grid *g, int forward_trip, int forward_blocks_per_sm, int replay_trip,
                       int replay_blocks_per_sm);
 
@@ -314,9 +316,8 @@ int mst_autotune(mst_grid *g, const float *beta_dev, const mst_params *p, uint64
                  void *stream);
 
 /* Device memory the handle may hold for the events a full-gradient forward render stores
- * (60 B per scattering event: voxel, position, incoming direction, weight, photon index, event
- * number, the free path left on entering the voxel, and the event's step for replay pass 2:
- * w_s, voxel, free path), for
+ * (48 B per scattering event: voxel, position, incoming direction, weight, photon index, event
+ * number, the free path left on entering the voxel, and the photon's previous record), for
  * calls of at most 2^27 photons. Default 32 GiB; 0 stores nothing (W by replay). The buffer
  * is allocated at the first full-gradient call that needs it and grown, within the budget,
  * when a call stored more events than it held, and never so large that less than a sixteenth of
@@ -405,7 +406,7 @@ const char *mst_batch_last_error(mst_batch *b);
  * MST_BATCH_BRANCHES (the default): one graph branch per scene holding that scene's
  * mst_render_grad sequence; the branches overlap on the GPU.
  * MST_BATCH_PERSISTENT: the photon transport of all scenes runs as single
- * persistent launches (forward, stored-event adjoint, replay passes 1 and 2), every warp taking
+ * persistent launches (forward, score, replay passes 1 and 2), every warp taking
  * the scenes one after the other from a device table, with each scene's small kernels (staging,
  * LOS, images, back-projection, folds) on a graph branch of its own between them. It applies
  * when every scene renders the voxel estimator's full gradient on an FP32 grid with one species
@@ -418,7 +419,7 @@ int mst_batch_set_form(mst_batch *b, int form);
 int mst_batch_get_form(mst_batch *b);
 
 /* Wavefront of the persistent form's launches, as mst_set_wavefront sets it for one handle:
- * forward voxels per trip in {0, 8, 10, 12, 16} (0 or 12: default), pass-2 voxels per trip in
+ * forward voxels per trip in {0, 8, 10, 12, 16} (0 or 8: default), score voxels per trip in
  * {0, 4, 6, 8, 10} (0 or 6: default), blocks per SM (0: the register budget's occupancy). */
 int mst_batch_set_wavefront(mst_batch *b, int forward_trip, int forward_blocks, int replay_trip, int replay_blocks);
 

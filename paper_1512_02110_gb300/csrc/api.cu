@@ -191,7 +191,7 @@ void set_score_fold(TransportArgs& a) {
 // replay runs pass 1, the pass-2 list and pass 2 per kReplayChunk photons (the size of its
 // per-photon buffers). The launches fold their FP32 tiles while they run; a last fold after each
 // launch takes what is left. store_events (forward of a full gradient, one launch): the forward
-// also stores its events and each photon's event count for the stored-event adjoint.
+// also stores its events for the score kernel.
 int run_photons(mst_grid* g, const mst_params* p, bool replay, double* cimg, cudaStream_t st,
                 bool store_events = false) {
     TransportArgs a = transport_args(g, p);

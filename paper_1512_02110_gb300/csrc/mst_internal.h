@@ -194,7 +194,8 @@ cudaError_t launch_add_air(const mst_grid* g, const float* beta, const float* ai
 cudaError_t launch_channel_beta(const mst_grid* g, const float* ref, double sigma, float* out, cudaStream_t st);
 cudaError_t launch_channel_add(const mst_grid* g, double* grad, double sigma, const double* gmu, double* loss,
                                const double* loss_mu, cudaStream_t st);
-// transport kernel modes: 0 forward voxel LE, 1 forward classic LE, 3 replay pass 1, 2 replay pass 2,
+// transport kernel modes: 0 / 1 forward with the voxelised / classic estimate (k_forward), 3 / 2 replay
+// passes 1 / 2 of the voxelised estimate,
 // 5 / 6 passes 1 / 2 of the classic-estimator gradient (4, the score of the stored events, is
 // launch_score)
 cudaError_t launch_transport(const mst_grid* g, const TransportArgs& a, int dtype, int mode, int blocks,

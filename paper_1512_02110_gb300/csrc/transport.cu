@@ -1,12 +1,11 @@
 // Photon transport on the GPU: the forward MC life cycle (Sec. 2.1.2, steps i-vi) with the
-// voxelised local estimate of Eq. Lcupdate (or the classic one of Eq. fle), and the replay
-// adjoint that re-walks every photon from its Philox key to scatter the score-function
-// gradient of L (no path is stored).
+// voxelised local estimate of Eq. Lcupdate or the classic one of Eq. fle (k_forward), and the
+// score-function gradient of the estimate: from the events the forward stored (k_score), or, when
+// they are not held, by two passes that walk the photons again from their Philox keys
+// (k_transport).
 //
-// Work distribution: a persistent grid sized to the SM count. Each lane owns one photon at a
-// time and advances it one free flight plus one event per loop trip; lanes whose photon has
-// ended take a new photon id from a warp-local pool that lane 0 refills from a global ticket,
-// so the warp stays full until the chunk runs dry.
+// Work distribution: persistent grids sized to the SM count; warps take photons in batches from a
+// global ticket (the score kernel: a forward warp's list of records) until none are left.
 #include <algorithm>
 #include <type_traits>
 
@@ -673,8 +672,8 @@ constexpr int kMinBlocksPass1 = 3;
 constexpr int kMinBlocksPass2 = 3;
 
 // kernel modes
-// kScore: the score of the stored events (k_score); kPass1C, kPass2C: passes 1 and 2 of the
-// classic-estimator gradient
+// kFwdVoxel, kFwdClassic: k_forward; kScore: k_score; kPass1, kPass2 and kPass1C, kPass2C: the replay
+// passes of the voxelised and the classic estimate (k_transport)
 constexpr int kFwdVoxel = 0, kFwdClassic = 1, kPass2 = 2, kPass1 = 3, kScore = 4, kPass1C = 5, kPass2C = 6;
 
 template <int NW>
@@ -817,14 +816,14 @@ __device__ __forceinline__ void refill(const TransportArgs& A, uint32_t n, bool&
 }
 
 // ------------------------------------------------------------------------------------------
-// The transport kernel. MODE 0: forward with the voxelised local estimate; 1: forward with the
-// classic local estimate; 3 and 2: the two passes of the replay adjoint. Every loop trip (1) fills empty lanes from the
-// ready stack, then from the id pool, (2) advances every flying photon by one voxel, pushing
-// collisions onto the event stack, and (3) whenever 32 events are queued (or the chunk is
-// draining), processes 32 events at once: local estimate, albedo, roulette, new direction;
-// photons that go on are pushed onto the ready stack.
+// The replay kernel: the two passes of the adjoint of a call whose events are not held. Every loop
+// trip (1) fills empty lanes from the ready stack, then from the id pool, (2) advances every flying
+// photon by up to TRIP voxels, pushing collisions onto the event stack, and (3) whenever 32 events
+// are queued (or the chunk is draining), processes 32 events at once: w_s, albedo, roulette, new
+// direction; photons that go on are pushed onto the ready stack. (The forward took the same form
+// once; see k_forward for what it gained.)
 //
-// Replay adjoint, two launches per chunk. Pass 1 (MODE 3) walks every photon and stores
+// Two launches per chunk. Pass 1 (MODE 3) walks every photon and stores
 // W = sum_s w_s, w_s = sum_c a_c(k_s) albedo I_s P_c(s), and its event count per photon; the
 // photons with W != 0 are then gathered into a list, longest first. Pass 2 (MODE 2) walks the
 // listed photons again, with S_j = W - sum_{s<j} w_s (FP64), and
@@ -832,12 +831,9 @@ __device__ __forceinline__ void refill(const TransportArgs& A, uint32_t n, bool&
 // Both passes run the same flight and event arithmetic, so they see the same path.
 // TWO: two-species medium (the launch has an air field); one-species kernels carry none of its
 // code. TRIP: voxels a flying lane advances per loop trip (0: the mode's default), a compile-time
-// constant (a run-time bound cost the forward 2 %); the autotuner picks among the instantiated ones.
+// constant.
 constexpr int min_blocks(int mode) {
-    return mode == kPass2
-               ? kMinBlocksPass2
-               : (mode == kPass1 ? kMinBlocksPass1
-                                 : kMinBlocksClassic);
+    return mode == kPass2 ? kMinBlocksPass2 : (mode == kPass1 ? kMinBlocksPass1 : kMinBlocksClassic);
 }
 
 // One scene's photons, run by every warp of the launch until the scene's pool is dry and the
@@ -1086,8 +1082,7 @@ __global__ void __launch_bounds__(kTB, min_blocks(MODE))
 // registers across the walk.)
 
 // words of a slot: direction (3), weight, events so far, position in the call, previous record, then
-// the flight: t (3), free path, padded index, and q (3) while it is ready, the extinction of the
-// collision voxel in the fourth word of the walk when it has ended
+// the flight: t (3), free path, padded index, and q (3)
 constexpr int kSlotWords = 15;
 static_assert(kSlots == 64, "the queues hold slot numbers in bytes");
 constexpr int kSD = 0, kSI = 3, kSs = 4, kSIdx = 5, kSPrev = 6, kST = 7, kSTau = 10, kSLin = 11, kSQ = 12;
@@ -1479,7 +1474,7 @@ constexpr size_t forward_smem() {
     return (size_t)kTransportWarps * (kFwdWords + (CL ? kClassicWords : 0)) * sizeof(uint32_t);
 }
 
-// (the classic estimate needs 96 registers: three blocks an SM)
+// (the classic estimate has its shadow rays' state beside the walk: three blocks an SM)
 template <int DT, bool TWO, int TRIP, bool CL = false>
 __global__ void __launch_bounds__(kFT, CL ? kMinBlocksClassic : kMinBlocksForward) k_forward(const TransportArgs A) {
     extern __shared__ uint32_t smem[];
