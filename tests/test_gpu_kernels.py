@@ -1,0 +1,119 @@
+"""The forward, score and ray kernels at the sizes where their tiles, queues and batches have edges:
+single photons and batches that never fill, grids of odd and single-voxel extents (half-empty bricks
+of the score's tile), camera counts around the groups of two, four and eight, a sun straight down
+(flights along one axis only), sub-pixel ray counts that do not divide a block."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests.gpu_util import dev, f32_scene, gpu_hashes, max_rel, need_gpu, record, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def m():
+    return need_gpu()
+
+
+def _scene(shape, cams, seed, n_rays=10, px=(8, 6), outside=False):
+    rng = np.random.default_rng(seed)
+    h = (50.0, 40.0, 60.0)
+    beta = rng.uniform(1.0, 15.0, int(np.prod(shape))) * synth.KM
+    ext = np.array(shape) * np.array(h)
+    pos = np.column_stack([ext[0] * rng.uniform(0.2, 0.8, cams), ext[1] * rng.uniform(0.2, 0.8, cams),
+                           np.full(cams, -25.0 if outside else 1.0)])
+    c = synth.make_cameras(pos, px[0], px[1], 70.0)
+    return f32_scene(synth.make_scene(shape, h, beta, c, n_rays=n_rays))
+
+
+# (grid, cameras, photons, sun zenith): a launch of one photon; one batch of 32 and one more; rounds
+# that drain with fewer than 32 events; several chunks of records per warp
+CASES = [((1, 1, 1), 1, 33, 0.6), ((2, 3, 1), 4, 1, 0.0), ((5, 7, 9), 5, 33, 0.0), ((5, 7, 9), 13, 5000, 0.7),
+         ((33, 17, 12), 17, 70_001, 0.3), ((16, 16, 16), 9, 400_000, 0.0)]
+
+
+def _full_gradient(shape, cams, photons, zenith, estimator):
+    sc = _scene(shape, cams, 7)
+    p = synth.Params(albedo=0.95, g=0.7, sun_zenith=zenith, sun_azimuth=0.4, n_photons=photons, seed=11)
+    return sc, p, dict(grad_mode="full", estimator=estimator), np.linspace(0.0, 0.1, sc.n_pix)
+
+
+@pytest.mark.parametrize("shape,cams,photons,zenith", CASES)
+def test_score_of_stored_events_matches_the_replay(m, shape, cams, photons, zenith):
+    """The gradient from the stored events (k_forward, k_score) against the one of the replay passes,
+    which walk every photon again from its Philox key in a kernel of their own: the same terms in
+    another order, so the two agree to the rounding of FP32 sums (1e-5, the bound of the
+    repository's other comparison of the two forms)."""
+    sc, p, opt, meas = _full_gradient(shape, cams, photons, zenith, "voxel")
+    a_grid, b_grid = m.Grid.from_scene(sc), m.Grid.from_scene(sc)
+    b_grid.set_replay_memory(0)
+    a, b = (g.render_grad(dev(sc.beta, np.float32), m.make_params(p, **opt), dev(meas, np.float64)) for g in (a_grid, b_grid))
+    sa, sb = a_grid.stats(), b_grid.stats()
+    for k in ("events", "segments", "escaped_n", "traced"):
+        assert sa[k] == sb[k], (k, sa[k], sb[k])
+    assert sa["lost"] == 0 and sa["traced"] == photons
+    assert sa["events_stored"] == sa["events"] and sb["events_stored"] == 0
+    ga, gb = a["grad"].cpu().numpy(), b["grad"].cpu().numpy()
+    assert np.isfinite(ga).all()
+    eg = rel_l2(ga, gb) if np.any(gb) else float(np.abs(ga).max())
+    record(f"score_vs_replay[{shape},{cams},{photons}]", grad_rel_l2=eg, events=sa["events"])
+    assert eg < 1e-5, eg
+
+
+@pytest.mark.parametrize("budget", ["stored", "replay"])
+@pytest.mark.parametrize("shape,cams,photons,zenith", CASES)
+def test_classic_gradient_matches_the_oracle(m, shape, cams, photons, zenith, budget):
+    """The classic estimate's gradient, from the stored events and by the replay passes, against the
+    FP64 oracle on the photons whose paths agree. (Not one against the other as above: next to a
+    camera in the cloud the terms are large and nearly cancel, and the replay's one FP32 tile
+    repeats itself to 3e-5 only, the stored events' to 2e-6.) 1e-3: the bound of the repository's
+    other gradients against the oracle."""
+    sc, p, opt, meas = _full_gradient(shape, cams, photons, zenith, "classic")
+    beta, grid = dev(sc.beta, np.float32), m.Grid.from_scene(sc)
+    if budget == "replay":
+        grid.set_replay_memory(0)
+    ref_hash = oracle.render(sc, p, want_L=False, hashes=True)["hash"]
+    skip = (gpu_hashes(m, grid, beta, m.make_params(p), photons) != ref_hash).astype(np.uint8)
+    assert skip.mean() < 2e-3
+    skip_dev = dev(skip, np.uint8)
+    grid.set_debug(None, skip_dev)
+    out = grid.render_grad(beta, m.make_params(p, **opt), dev(meas, np.float64))
+    grid.set_debug(None, None)
+    ref = oracle.full_grad(sc, p, meas, skip=skip, classic=True)
+    assert grid.stats()["lost"] == 0
+    eg = rel_l2(out["grad"].cpu().numpy(), ref["grad"])
+    el = abs(out["loss"].item() - ref["loss"]) / ref["loss"]
+    record(f"classic_gradient[{shape},{cams},{photons},{budget}]", grad_rel_l2=eg, loss=el)
+    assert eg < 1e-3 and el < 1e-3, (eg, el)
+
+
+@pytest.mark.parametrize("shape,cams,n_rays,px,outside", [((1, 1, 1), 1, 1, (1, 1), False), ((5, 7, 9), 3, 7, (5, 3), False),
+                                                          ((9, 5, 4), 2, 64, (9, 4), True), ((33, 17, 12), 5, 10, (33, 9), True)])
+def test_rays_match_the_oracle(m, shape, cams, n_rays, px, outside):
+    """Transmittance, images of a given field, and the fixed-field loss and gradient against the FP64
+    oracle: FP32 chords leave 1e-6 of a segment, the bounds of the repository's other ray tests
+    (2e-6 + 2e-5 max(tau, 1), 1e-4 of an image, 1e-3 of the gradient) hold here too."""
+    sc = _scene(shape, cams, 3, n_rays=n_rays, px=px, outside=outside)
+    rng = np.random.default_rng(5)
+    L = rng.uniform(0.5, 2.0, (cams, sc.nvox)) * sc.beta
+    meas = rng.uniform(0.0, 1e-4, sc.n_pix)
+    now = (sc.beta * rng.uniform(0.8, 1.2, sc.nvox)).astype(np.float32).astype(np.float64)
+    grid, beta = m.Grid.from_scene(sc), dev(sc.beta, np.float32)
+    tau, T_ref = oracle.transmittance(sc)
+    eT = []
+    for T in (grid.transmittance(beta),  # the handle's haloed copy of beta, and the linear one without a handle
+              m.transmittance_noalloc(sc.shape, sc.h, sc.origin, sc.cam_pos, sc.cam_rot, sc.cam_w, sc.cam_h, sc.cam_fov, beta)):
+        err = np.abs(T.cpu().numpy() - T_ref) / T_ref
+        eT.append(float(np.max(err / (2e-5 * np.maximum(tau, 1.0) + 2e-6))))
+    img = grid.form_images(beta, dev(L, np.float64).view(cams, -1)).cpu().numpy()
+    img_ref = oracle.images(sc, L, T_ref)
+    ei = max_rel(img, img_ref, 1e-3 * np.abs(img_ref).max())
+    out = grid.surrogate_grad(dev(now, np.float32), dev(L, np.float64).view(cams, -1), beta, m.make_params(synth.Params()),
+                              dev(meas, np.float64))
+    ref = oracle.surrogate_grad(sc.with_beta(now), L, sc.beta, meas)
+    el = abs(out["loss"].item() - ref["loss"]) / ref["loss"]
+    eg = rel_l2(out["grad"].cpu().numpy(), ref["grad"])
+    record(f"rays[{shape},{n_rays},{px}]", T=eT[0], T_noalloc=eT[1], images=ei, loss=el, grad=eg)
+    assert max(eT) <= 1.0 and ei < 1e-4 and el < 1e-4 and eg < 1e-3, (eT, ei, el, eg)
