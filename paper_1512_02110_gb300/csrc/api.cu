@@ -176,13 +176,15 @@ void set_fold(TransportArgs& a, uint64_t bins) {
 
 // The score kernel folds one slice of its brick tile per chunk of stored events. A photon makes
 // a few events at most on average; counting one per photon keeps a sweep within kFoldSweep photons.
-// The classic estimate's shadow rays add far more to a bin, so its slices are at least 128 bins.
-void set_score_fold(TransportArgs& a, bool classic) {
+void set_score_fold(TransportArgs& a) {
     const uint64_t bins = (uint64_t)brick_bins(a.g) * a.score_tiles, chunks = kFoldSweep / kEventChunk;
-    const uint64_t slice = std::max<uint64_t>(classic ? 128 : 32, ((bins + chunks - 1) / chunks + 31) / 32 * 32);
+    const uint64_t slice = std::max<uint64_t>(32, ((bins + chunks - 1) / chunks + 31) / 32 * 32);
     a.fold_bins = bins;
     a.fold_slice = (uint32_t)slice;
     a.fold_nslices = (uint32_t)((bins + slice - 1) / slice);
+    // the classic score's other tile, at least 128 bins per chunk (about as many photons as a ticket batch)
+    a.pad_slice = (uint32_t)std::max<uint64_t>(128, (((uint64_t)a.g.npad + chunks - 1) / chunks + 31) / 32 * 32);
+    a.pad_nslices = ((uint32_t)a.g.npad + a.pad_slice - 1) / a.pad_slice;
 }
 
 // Runs the photon transport. The forward render is one launch per kLaunchPhotons photons; the
@@ -284,7 +286,7 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
     if (classic) a.cres = g->resid;
     {
         Phase ph(g, MST_PH_REPLAY2, st);
-        set_score_fold(a, classic);
+        set_score_fold(a);
         a.ticket = g->tickets + 2;  // its warps take the forward warps' lists from it
         // (the classic kernel's blocks are those of its forward: both take three an SM)
         MST_CK(launch_score(g, a, p->grid_dtype, classic, blocks(classic ? 1 : 4), st));
@@ -1351,7 +1353,7 @@ int persistent_tables(mst_batch* b, const float* const* betas, const mst_params*
         f.ticket = g->tickets;
         t[i] = f;
         TransportArgs r = transport_args(g, p);
-        set_score_fold(r, false);
+        set_score_fold(r);
         r.evrec = g->evrec;
         r.ev_cap = g->ev_cap;
         r.ev_count = g->ev_count;

@@ -96,6 +96,7 @@ struct TransportArgs {
     uint64_t fold_bins;        // bins of the tile this launch folds while it runs (0: none)
     uint32_t fold_slice;       // bins per slice (one slice per ticket batch)
     uint32_t fold_nslices;     // slices per sweep
+    uint32_t pad_slice, pad_nslices;  // the same for the padded tile (classic score)
     double* stats;             // [MST_NSTATS]
     uint32_t* hash;            // per-photon checksum or NULL
     float4* point;             // per-photon last event point (offset, packed voxel) or NULL

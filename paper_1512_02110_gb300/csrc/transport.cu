@@ -444,87 +444,6 @@ __device__ __forceinline__ void shadow_scatter(const TransportArgs& A, int ix, i
     }
 }
 
-// Shared-memory strip of (bin, term) entries, K per lane: written lane by lane, read transposed
-// (entry j of a lane lies at [j][lane ^ 2j]: neither meets in a bank), so that one atomic
-// instruction adds consecutive voxels of a few rays.
-constexpr uint32_t kNoEntry = 0xFFFFFFFFu;
-
-__device__ __forceinline__ void strip_put(float2* strip, unsigned lane, int j, uint32_t key, float v) {
-    strip[j * 32 + ((lane ^ (2 * j)) & 31)] = make_float2(__uint_as_float(key), v);
-}
-
-template <int K>
-__device__ __forceinline__ void strip_add(float2* strip, unsigned lane, float* tile, unsigned nbins) {
-    __syncwarp();
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-        const int i = r * 32 + (int)lane, j = i % K, l = i / K;  // entry j of lane l
-        const float2 en = strip[j * 32 + ((l ^ (2 * j)) & 31)];
-        const uint32_t key = __float_as_uint(en.x);
-        if (key < nbins) atomicAdd(tile + key, en.y);
-    }
-    __syncwarp();
-}
-
-// A walk's steps through the brick bins: the stride of the bricks along each axis, signed, with the
-// axis' bit of the voxel inside its brick. `at` is the bin with the bits of the axes the walk
-// descends mirrored (`flip`): a crossing toggles the axis' bit and enters the next brick when it was set.
-struct BrickSteps {
-    uint32_t sx, sy, sz;
-    __device__ __forceinline__ void set(const Geo& g, uint32_t flip) {
-        const uint32_t by8 = 8u * (unsigned)((g.nx + 1) >> 1), bz8 = by8 * (unsigned)((g.ny + 1) >> 1);
-        sx = (flip & 1u ? 0u - 8u : 8u) | 1u;
-        sy = (flip & 2u ? 0u - by8 : by8) | 2u;
-        sz = (flip & 4u ? 0u - bz8 : bz8) | 4u;
-    }
-    __device__ __forceinline__ void cross(uint32_t& at, bool px, bool py) const {
-        const uint32_t s = px ? sx : (py ? sy : sz);
-        const bool over = (at & s & 7u) != 0u;
-        at ^= s & 7u;
-        if (over) at += s & ~7u;
-    }
-};
-
-// shadow_scatter for the warp's 32 rays at once (nvox 0: the lane has none), into the tile in
-// bricks, K voxels per trip through the strip. Bound by the atomics: one per voxel and lane into the
-// padded tile, the score of 1e7 photons (64^3, 9 cameras, 1.3e10 shadow voxels) took 150 ms; 94 so,
-// 47 of them for the first walk of the rays.
-template <int K>
-__device__ __forceinline__ void shadow_scatter_warp(const TransportArgs& A, float* tile, unsigned nbins, float2* strip,
-                                                    unsigned lane, int ix, int iy, int iz, float3 p, const Cam& cm,
-                                                    float sw, unsigned nvox) {
-    Shadow r{};
-    BrickSteps st{};
-    uint32_t at = 0u, flip = 0u;
-    if (nvox != 0u) {
-        r = shadow_init(A.g, ix, iy, iz, p, cm);
-        flip = (r.dx < 0 ? 1u : 0u) | (r.dy < 0 ? 2u : 0u) | (r.dz < 0 ? 4u : 0u);
-        at = brick_bin(A.g, (unsigned)ix, (unsigned)iy, (unsigned)iz) ^ flip;
-        st.set(A.g, flip);
-    }
-    while (__any_sync(kFull, nvox != 0u)) {
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            uint32_t key = kNoEntry;
-            const float m = fminf(r.tx, fminf(r.ty, r.tz));
-            const float len = r.rem > m ? m : r.rem;
-            if (nvox != 0u) {
-                key = at ^ flip;
-                const bool px = r.tx <= m;
-                const bool py = !px && r.ty <= m;
-                st.cross(at, px, py);
-                r.rem -= m;
-                r.tx = px ? r.qx : r.tx - m;
-                r.ty = py ? r.qy : r.ty - m;
-                r.tz = (px || py) ? r.tz - m : r.qz;
-                --nvox;
-            }
-            strip_put(strip, lane, j, key, sw * len);
-        }
-        strip_add<K>(strip, lane, tile, nbins);
-    }
-}
-
 // Where an event lands in camera cm (Eq. fle): false when the camera does not see it (behind
 // the camera, outside the image, on the centre, or, with a residual, a pixel of zero residual);
 // else the pixel gp and f0 = albedo I_s P(mu) / (|X_c - X_s|^2 Omega_p), times the pixel's
@@ -597,12 +516,10 @@ __device__ __forceinline__ void flush_classic(const TransportArgs& A, const Clas
 // stay busy however few cameras see each event. OP 0 adds each f = f0 exp(-t) to its pixel of
 // the classic image; OP 1 returns w_s = sum_c cres[p] f (the event's share of <dE/di, i>, for the
 // classic-estimator gradient), summed over the cameras in their order; OP 2 also scatters the
-// shadow-ray terms -cres[p] f * (length in voxel m) into the padded gradient tile; OP 3 into `tile`,
-// the one in bricks, K voxels at a time through `strip`.
-template <int DT, int OP, int K = 1>
+// shadow-ray terms -cres[p] f * (length in voxel m) into the gradient tile.
+template <int DT, int OP>
 __device__ __forceinline__ float le_classic(const TransportArgs& A, const Photon& e, float w, bool air, bool act,
-                                            const ClassicScratch& cs, float* tile = nullptr, unsigned nbins = 0u,
-                                            float2* strip = nullptr) {
+                                            const ClassicScratch& cs) {
     const unsigned lane = threadIdx.x & 31u;
     const uint32_t vox = (uint32_t)e.ix | ((uint32_t)e.iy << 11) | ((uint32_t)e.iz << 22);
     float acc = 0.f;
@@ -628,22 +545,20 @@ __device__ __forceinline__ float le_classic(const TransportArgs& A, const Photon
             const uint32_t v = __shfl_sync(kFull, vox, el);
             const float3 p = make_float3(__shfl_sync(kFull, e.p.x, el), __shfl_sync(kFull, e.p.y, el),
                                          __shfl_sync(kFull, e.p.z, el));
-            const Cam& cm = A.cams.c[c0 + cl];
-            const int ix = (int)(v & 0x7FFu), iy = (int)((v >> 11) & 0x7FFu), iz = (int)(v >> 22);
-            unsigned nv = 0u;
-            float f = 0.f;
             if (j < qn) {
+                const Cam& cm = A.cams.c[c0 + cl];
+                const int ix = (int)(v & 0x7FFu), iy = (int)((v >> 11) & 0x7FFu), iz = (int)(v >> 22);
                 const int r = cl * 32 + el;
-                f = cs.res[r] * expf(-shadow_tau<DT>(A, ix, iy, iz, p, cm, nv));
+                unsigned nv = 0u;
+                const float f = cs.res[r] * expf(-shadow_tau<DT>(A, ix, iy, iz, p, cm, nv));
                 if (OP == 0) {
                     atomicAdd(A.cimg + cs.pix[r], (double)f);
                 } else {
                     cs.res[r] = f;
                     if (OP == 2) shadow_scatter(A, ix, iy, iz, p, cm, -f, nv);
                 }
-                cs.seg[lane] += OP >= 2 ? 2u * nv : nv;
+                cs.seg[lane] += OP == 2 ? 2u * nv : nv;
             }
-            if constexpr (OP == 3) shadow_scatter_warp<K>(A, tile, nbins, strip, lane, ix, iy, iz, p, cm, -f, nv);
         }
         __syncwarp();
         if (OP > 0)
@@ -1599,6 +1514,7 @@ __global__ void __launch_bounds__(kFT, kMinBlocksForward)
 
 constexpr int kFlightWords = 10;  // of a queued flight
 constexpr int kScoreSlots = 64;   // flights a warp queues: fewer than 32 left when a batch adds 32
+constexpr uint32_t kNoEntry = 0xFFFFFFFFu;
 
 template <int K, bool CL>
 constexpr int score_words() {  // shared words per warp: a batch of records, the queue, the strip, the classic scratch
@@ -1621,7 +1537,7 @@ __device__ __forceinline__ void copy16_async(uint32_t* dst, const uint4* src) {
 }
 
 // CL: w_s of the classic estimate, whose shadow rays are walked for it and walked again to scatter
-// their own terms (le_classic).
+// their own terms (le_classic) into the padded tile.
 template <int DT, bool TWO, int K, bool CL>
 __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem) {
     if (*A.ev_count > A.ev_cap) return;  // the events did not fit: the replay passes run instead
@@ -1633,12 +1549,15 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
     if constexpr (CL) cls = classic_scratch(q + kFlightWords * kScoreSlots + 2 * 32 * K, lane);
     const unsigned nbins = (unsigned)brick_bins(A.g);
     float* tile = A.gbrk + (size_t)(blockIdx.x % A.score_tiles) * nbins;  // the block's copy
+    const uint32_t by8 = 8u * (unsigned)((A.g.nx + 1) >> 1), bz8 = by8 * (unsigned)((A.g.ny + 1) >> 1);
     unsigned stored = 0u, flights = 0u, entries = 0u, lost = 0u;
 
-    // The flight in hand: t and q as in Flight, and where it is (see BrickSteps).
+    // The flight in hand: t and q as in Flight, and per axis the step of its bin (the stride of the
+    // bricks, signed, with the axis' bit of the voxel inside the brick). `at` is the bin with the
+    // bits of the axes the flight descends mirrored (`flip`): a crossing toggles the axis' bit and
+    // enters the next brick when it was set.
     float tx = 0.f, ty = 0.f, tz = 0.f, qx = 0.f, qy = 0.f, qz = 0.f, nS = 0.f;
-    BrickSteps st{};
-    uint32_t at = 0u, flip = 0u, goal = 0u;
+    uint32_t sx = 0u, sy = 0u, sz = 0u, at = 0u, flip = 0u, goal = 0u;
     int left = 0;  // faces still to cross; 0: no flight
 
     // the next batch: its records are being copied (pending), or the lists are used up
@@ -1666,6 +1585,14 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
                 const float v = atomicExch(A.gbrk + i, 0.f);
                 int k;
                 if (v != 0.f && brick_voxel(A.g, (int)(i % nbins), k)) atomicAdd(A.g64 + k, (double)v);
+            }
+            if constexpr (CL) {  // and one of the padded tile that the shadow rays add to
+                const uint32_t p0 = ch % A.pad_nslices * A.pad_slice, p1 = min(p0 + A.pad_slice, (uint32_t)A.g.npad);
+                for (uint32_t i = p0 + lane; i < p1; i += 32) {
+                    const float v = atomicExch(A.gacc + i, 0.f);
+                    int k;
+                    if (v != 0.f && interior_lin(A.g, (int)i, k)) atomicAdd(A.g64 + k, (double)v);
+                }
             }
         }
         const uint4* r = A.evrec + ((unsigned long long)ch * kEvChunk + (unsigned)base + lane);
@@ -1704,7 +1631,7 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
             }
             fetch();
             float w = 0.f;
-            if constexpr (CL) w = le_classic<DT, 3, K>(A, e, __uint_as_float(r1.w), air, on, cls, tile, nbins, strip);
+            if constexpr (CL) w = le_classic<DT, 2>(A, e, __uint_as_float(r1.w), air, on, cls);
             else if (on) w = le_adjoint(A, e, __uint_as_float(r1.w), k, air);
             // S: later events first. A batch may hold two events of a photon (rounds of fewer than
             // 32 while the forward's warp drained): they take turns, the later record first.
@@ -1783,11 +1710,14 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
                 const uint32_t nf = s[9 * kScoreSlots];
                 left = (int)(nf & 0xFFFFu);
                 flip = nf >> 16;
-                st.set(A.g, flip);
+                sx = (flip & 1u ? 0u - 8u : 8u) | 1u;
+                sy = (flip & 2u ? 0u - by8 : by8) | 2u;
+                sz = (flip & 4u ? 0u - bz8 : bz8) | 4u;
             }
         }
         qn = max(0, qn - want);
-        // K voxels per lane into the strip
+        // K voxels per lane into the strip (entry j of a lane at [j][lane ^ 2j]: neither the writes
+        // nor the transposed reads meet in a bank)
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             uint32_t key = kNoEntry;
@@ -1796,15 +1726,26 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
                 key = at ^ flip;
                 const bool px = tx <= m;
                 const bool py = !px && ty <= m;
-                st.cross(at, px, py);
+                const uint32_t s = px ? sx : (py ? sy : sz);
+                const bool over = (at & s & 7u) != 0u;
+                at ^= s & 7u;
+                if (over) at += s & ~7u;
                 tx = px ? qx : tx - m;
                 ty = py ? qy : ty - m;
                 tz = (px || py) ? tz - m : qz;
                 --left;
             }
-            strip_put(strip, lane, j, key, nS * m);
+            strip[j * 32 + ((lane ^ (2 * j)) & 31)] = make_float2(__uint_as_float(key), nS * m);
         }
-        strip_add<K>(strip, lane, tile, nbins);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const int i = r * 32 + (int)lane, j = i % K, l = i / K;  // entry j of lane l
+            const float2 en = strip[j * 32 + ((l ^ (2 * j)) & 31)];
+            const uint32_t key = __float_as_uint(en.x);
+            if (key < nbins) atomicAdd(tile + key, en.y);
+        }
+        __syncwarp();
     }
     if constexpr (CL) flush_classic(A, cls, lane);
     const unsigned long long se = warp_sumu(stored), sf = warp_sumu(flights), sn = warp_sumu(entries), sl = warp_sumu(lost);
