@@ -182,9 +182,6 @@ void set_score_fold(TransportArgs& a) {
     a.fold_bins = bins;
     a.fold_slice = (uint32_t)slice;
     a.fold_nslices = (uint32_t)((bins + slice - 1) / slice);
-    // the classic score's other tile, at least 128 bins per chunk (about as many photons as a ticket batch)
-    a.pad_slice = (uint32_t)std::max<uint64_t>(128, (((uint64_t)a.g.npad + chunks - 1) / chunks + 31) / 32 * 32);
-    a.pad_nslices = ((uint32_t)a.g.npad + a.pad_slice - 1) / a.pad_slice;
 }
 
 // Runs the photon transport. The forward render is one launch per kLaunchPhotons photons; the
@@ -281,24 +278,20 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
     MST_CK(cudaMemsetAsync(g->tickets, 0, sizeof(unsigned int) * 3, st));
     MST_CK(cudaMemsetAsync(g->wbuf, 0, sizeof(double) * n, st));
     auto blocks = [&](int mode) { return transport_blocks(g, p->grid_dtype, mode); };
-    const bool classic = p->estimator == MST_EST_CLASSIC;
-    const int m_p1 = classic ? 5 : 3, m_p2 = classic ? 6 : 2;  // as in run_photons
-    if (classic) a.cres = g->resid;
     {
         Phase ph(g, MST_PH_REPLAY2, st);
         set_score_fold(a);
         a.ticket = g->tickets + 2;  // its warps take the forward warps' lists from it
-        // (the classic kernel's blocks are those of its forward: both take three an SM)
-        MST_CK(launch_score(g, a, p->grid_dtype, classic, blocks(classic ? 1 : 4), st));
+        MST_CK(launch_score(g, a, p->grid_dtype, blocks(4), st));
     }
     set_fold(a, (uint64_t)g->geo.npad);
     a.ticket = g->tickets;
     {
         Phase ph(g, MST_PH_REPLAY, st);  // these return at once when the events fitted
-        MST_CK(launch_transport(g, a, p->grid_dtype, m_p1, blocks(m_p1), st));
+        MST_CK(launch_transport(g, a, p->grid_dtype, 3, blocks(3), st));
         MST_CK(launch_score_list(g, a.n, true, st));
         a.ticket = g->tickets + 1;
-        MST_CK(launch_transport(g, a, p->grid_dtype, m_p2, blocks(m_p2), st));
+        MST_CK(launch_transport(g, a, p->grid_dtype, 2, blocks(2), st));
     }
     return MST_OK;  // what is left in the tiles is folded by launch_combine_full
 }
@@ -772,7 +765,34 @@ int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const 
         MST_CK(launch_stage(g, beta, g->air, p->grid_dtype, st));
     }
     MST_CK(cudaMemsetAsync(g->stats, 0, MST_NSTATS * 8, st));
-    // full gradient: the forward stores its events when they can be held (the replay then reads them)
+    if (p->estimator == MST_EST_CLASSIC) {  // Eq. fle images, their loss, and the score replay
+        MST_CK(cudaMemsetAsync(g->cimg, 0, sizeof(double) * g->total_pix, st));
+        rc = run_photons(g, p, false, g->cimg, st);
+        if (rc) return rc;
+        MST_CK(cudaMemsetAsync(lossp, 0, sizeof(double), st));
+        {
+            Phase ph(g, MST_PH_IMAGES, st);
+            MST_CK(launch_classic_residual(g, g->cimg, meas, mask, g->resid, lossp, st));
+        }
+        if (images)
+            MST_CK(cudaMemcpyAsync(images, g->cimg, sizeof(double) * g->total_pix, cudaMemcpyDeviceToDevice, st));
+        rc = ensure_replay(g, kReplayChunk);
+        if (rc) return rc;
+        MST_CK(cudaMemsetAsync(g->g64, 0, sizeof(double) * g->geo.nvox, st));
+        rc = run_photons(g, p, true, nullptr, st);
+        if (rc) return rc;
+        {
+            Phase ph(g, MST_PH_COMBINE, st);
+            MST_CK(launch_combine_full(g, nullptr, g->g64, false, grad, st));
+        }
+        if (p->reg_eta != 0.0) {
+            Phase ph(g, MST_PH_COMBINE, st);
+            MST_CK(launch_regularizer(g, beta, p->reg_eta, g->lap, g->stats + MST_NSTATS + 1, lossp, grad, st));
+        }
+        return MST_OK;
+    }
+    MST_CK(cudaMemsetAsync(g->L64, 0, sizeof(double) * nL, st));
+    // full gradient: the forward stores its events when they can be held (W without pass 1)
     bool stored = false;
     if (p->grad_mode == MST_GRAD_FULL) {
         if (g->capturing) {  // a batch graph: the buffers were sized before the capture
@@ -785,33 +805,6 @@ int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const 
             }
         }
     }
-    if (p->estimator == MST_EST_CLASSIC) {  // Eq. fle images, their loss, and the score replay
-        MST_CK(cudaMemsetAsync(g->cimg, 0, sizeof(double) * g->total_pix, st));
-        rc = run_photons(g, p, false, g->cimg, st, stored);
-        if (rc) return rc;
-        MST_CK(cudaMemsetAsync(lossp, 0, sizeof(double), st));
-        {
-            Phase ph(g, MST_PH_IMAGES, st);
-            MST_CK(launch_classic_residual(g, g->cimg, meas, mask, g->resid, lossp, st));
-        }
-        if (images)
-            MST_CK(cudaMemcpyAsync(images, g->cimg, sizeof(double) * g->total_pix, cudaMemcpyDeviceToDevice, st));
-        rc = ensure_replay(g, stored ? p->n_photons : kReplayChunk);
-        if (rc) return rc;
-        MST_CK(cudaMemsetAsync(g->g64, 0, sizeof(double) * g->geo.nvox, st));
-        rc = stored ? run_replay_stored(g, p, st) : run_photons(g, p, true, nullptr, st);
-        if (rc) return rc;
-        {
-            Phase ph(g, MST_PH_COMBINE, st);
-            MST_CK(launch_combine_full(g, nullptr, g->g64, stored, grad, st));
-        }
-        if (p->reg_eta != 0.0) {
-            Phase ph(g, MST_PH_COMBINE, st);
-            MST_CK(launch_regularizer(g, beta, p->reg_eta, g->lap, g->stats + MST_NSTATS + 1, lossp, grad, st));
-        }
-        return MST_OK;
-    }
-    MST_CK(cudaMemsetAsync(g->L64, 0, sizeof(double) * nL, st));
     rc = run_photons(g, p, false, nullptr, st, stored);
     if (rc) return rc;
     {

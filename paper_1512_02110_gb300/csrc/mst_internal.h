@@ -96,7 +96,6 @@ struct TransportArgs {
     uint64_t fold_bins;        // bins of the tile this launch folds while it runs (0: none)
     uint32_t fold_slice;       // bins per slice (one slice per ticket batch)
     uint32_t fold_nslices;     // slices per sweep
-    uint32_t pad_slice, pad_nslices;  // the same for the padded tile (classic score)
     double* stats;             // [MST_NSTATS]
     uint32_t* hash;            // per-photon checksum or NULL
     float4* point;             // per-photon last event point (offset, packed voxel) or NULL
@@ -206,10 +205,7 @@ cudaError_t launch_fold_grad(const mst_grid* g, cudaStream_t st);
 // the pass-2 list; with `stored` its kernels return at once when the stored events fitted
 cudaError_t launch_score_list(const mst_grid* g, uint32_t n, bool stored, cudaStream_t st);
 // the score gradient from the stored events (returns at once when they did not fit)
-// (classic: with the classic estimate's w_s and shadow-ray terms; transport_blocks_per_sm of mode 1 sets
-// its kernel's attributes)
-cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, bool classic, int blocks,
-                         cudaStream_t st);
+cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, int blocks, cudaStream_t st);
 // backward MC images (Eq. ble): n paths per pixel, sums into sum / sum2, then sum <- means and
 // var <- variances of the means (var may be NULL)
 cudaError_t launch_bmc(const mst_grid* g, const mst_params* p, uint32_t n, double* sum, double* sum2, double* var,

@@ -1,8 +1,8 @@
 // Photon transport on the GPU: the forward MC life cycle (Sec. 2.1.2, steps i-vi) with the
-// voxelised local estimate of Eq. Lcupdate or the classic one of Eq. fle (k_forward), and the
-// score-function gradient of the estimate: from the events the forward stored (k_score), or, when
-// they are not held, by two passes that walk the photons again from their Philox keys
-// (k_transport).
+// voxelised local estimate of Eq. Lcupdate (k_forward) or the classic one of Eq. fle
+// (k_transport), and the score-function gradient of the estimate: from the events the forward
+// stored (k_score), or, for the classic estimate and when the events are not held, by two passes
+// that walk the photons again from their Philox keys (k_transport).
 //
 // Work distribution: persistent grids sized to the SM count; warps take photons in batches from a
 // global ticket (the score kernel: a forward warp's list of records) until none are left.
@@ -30,6 +30,56 @@ struct Photon {
     uint32_t idx;    // call-relative index (hash / skip arrays)
 };
 
+// Photon tallies of the forward render: per-thread totals, reduced over the warp at the end.
+struct Tally {
+    float esc[6];
+    float absorbed, killed, gained, forced, launched;
+    unsigned capped, escaped, traced, lost;
+};
+
+// The forward render keeps its tallies in shared memory, one slot per thread (stride kTB
+// words, so a warp's lanes touch consecutive words): no atomics and no registers held across
+// the voxel loop. The replay passes keep none: their NoTally compiles every update away.
+struct LaneTally {
+    float* f;  // 11 float fields at f[q * kTB]
+    unsigned* u;  // 4 counters at u[q * kTB]
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int q = 0; q < 11; ++q) f[q * kTB] = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) u[q * kTB] = 0u;
+    }
+    __device__ __forceinline__ void add_absorbed(float v) { f[6 * kTB] += v; }
+    __device__ __forceinline__ void add_killed(float v) { f[7 * kTB] += v; }
+    __device__ __forceinline__ void add_gained(float v) { f[8 * kTB] += v; }
+    __device__ __forceinline__ void add_forced(float v) { f[9 * kTB] += v; }
+    __device__ __forceinline__ void add_capped() { u[0] += 1u; }
+    __device__ __forceinline__ void add_launch(float i0) {
+        f[10 * kTB] += i0;
+        u[2 * kTB] += 1u;
+    }
+    __device__ __forceinline__ void add_escape(int face, float v) {
+        if (face < 6) f[face * kTB] += v;
+        if (face == kWalkOverflow) u[3 * kTB] += 1u;
+        else u[1 * kTB] += 1u;
+    }
+    __device__ __forceinline__ Tally load() const {
+        Tally t;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) t.esc[q] = f[q * kTB];
+        t.absorbed = f[6 * kTB];
+        t.killed = f[7 * kTB];
+        t.gained = f[8 * kTB];
+        t.forced = f[9 * kTB];
+        t.launched = f[10 * kTB];
+        t.capped = u[0];
+        t.escaped = u[1 * kTB];
+        t.traced = u[2 * kTB];
+        t.lost = u[3 * kTB];
+        return t;
+    }
+};
+
 // A per-thread event counter that exists only when ON (the one-species kernels carry none).
 template <bool ON>
 struct EventCount {
@@ -46,13 +96,15 @@ struct EventCount<false> {
     __device__ __forceinline__ void flush(double*, unsigned) const {}
 };
 
-// the replay passes keep no tallies
 struct NoTally {
+    __device__ __forceinline__ void zero() {}
     __device__ __forceinline__ void add_absorbed(float) {}
     __device__ __forceinline__ void add_forced(float) {}
     __device__ __forceinline__ void add_gained(float) {}
     __device__ __forceinline__ void add_killed(float) {}
     __device__ __forceinline__ void add_capped() {}
+    __device__ __forceinline__ void add_launch(float) {}
+    __device__ __forceinline__ void add_escape(int, float) {}
 };
 
 // Voxel and offset of u * n voxels, u = (2m + 1) / 2^24 from a Philox word: (2m + 1) n / 2^24 is
@@ -486,29 +538,6 @@ struct ClassicScratch {
     unsigned* rays;  // [1]
 };
 
-// The warp's scratch at `words`, counters cleared; and its counts into the statistics.
-__device__ __forceinline__ ClassicScratch classic_scratch(uint32_t* words, unsigned lane) {
-    ClassicScratch c;
-    c.res = reinterpret_cast<float*>(words);
-    c.pix = reinterpret_cast<int*>(words + kClassicGroup * 32);
-    c.job = reinterpret_cast<uint8_t*>(words + 2 * kClassicGroup * 32);
-    c.seg = words + 2 * kClassicGroup * 32 + kClassicGroup * 8;
-    c.rays = c.seg + 32;
-    c.seg[lane] = 0u;
-    if (lane == 0u) *c.rays = 0u;
-    __syncwarp();
-    return c;
-}
-
-__device__ __forceinline__ void flush_classic(const TransportArgs& A, const ClassicScratch& c, unsigned lane) {
-    const unsigned long long ss = warp_sumu(c.seg[lane]);
-    if (lane == 0u) {
-        atomicAdd(A.stats + MST_ST_SHADOW_RAYS, (double)*c.rays);
-        atomicAdd(A.stats + MST_ST_SHADOW_SEGMENTS, (double)ss);
-    }
-    __syncwarp();
-}
-
 // Eq. fle for the warp's round of events (lane i < n holds event i; act says whether this lane
 // holds one), shadow rays issued warp-coherently: the lanes first find, camera by camera, which
 // cameras see their event and compact those (event, camera) pairs into a list; then every lane
@@ -614,6 +643,11 @@ __device__ __forceinline__ void write_point(const TransportArgs& A, const Photon
                                   __uint_as_float((uint32_t)ph.ix | ((uint32_t)ph.iy << 11) | ((uint32_t)ph.iz << 22)));
 }
 
+__device__ __forceinline__ void finish_photon(const TransportArgs& A, const Photon& ph, int term) {
+    if (A.hash) A.hash[ph.idx] = end_hash(ph.hash, ph.s, term);
+    if (A.point) write_point(A, ph);
+}
+
 // the forward keeps the running checksum in the output itself
 __device__ __forceinline__ void finish_hash(const TransportArgs& A, uint32_t idx, uint32_t s, int term) {
     A.hash[idx] = end_hash(A.hash[idx], s, term);
@@ -672,8 +706,8 @@ constexpr int kMinBlocksPass1 = 3;
 constexpr int kMinBlocksPass2 = 3;
 
 // kernel modes
-// kFwdVoxel, kFwdClassic: k_forward; kScore: k_score; kPass1, kPass2 and kPass1C, kPass2C: the replay
-// passes of the voxelised and the classic estimate (k_transport)
+// kFwdVoxel: k_forward; kScore: k_score; kFwdClassic, kPass1, kPass2 and kPass1C, kPass2C: the classic
+// forward and the replay passes of the voxelised and the classic estimate (k_transport)
 constexpr int kFwdVoxel = 0, kFwdClassic = 1, kPass2 = 2, kPass1 = 3, kScore = 4, kPass1C = 5, kPass2C = 6;
 
 template <int NW>
@@ -685,7 +719,7 @@ struct Stack {
 // words of a stack slot: the photon, and a replay's event count and sum
 template <int MODE>
 struct Rec {
-    static constexpr int NW = 15;
+    static constexpr int NW = MODE >= kPass2 ? 15 : 12;
 };
 
 template <int NW>
@@ -815,8 +849,40 @@ __device__ __forceinline__ void refill(const TransportArgs& A, uint32_t n, bool&
     }
 }
 
+__device__ __forceinline__ void flush_tally(const TransportArgs& A, const Tally& t, unsigned segments,
+                                            unsigned events, unsigned lane) {
+    double v[11];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v[q] = warp_sum((double)t.esc[q]);
+    v[6] = warp_sum((double)t.absorbed);
+    v[7] = warp_sum((double)t.killed);
+    v[8] = warp_sum((double)t.gained);
+    v[9] = warp_sum((double)t.forced);
+    v[10] = warp_sum((double)t.launched);
+    const unsigned long long ev = warp_sumu(events), sg = warp_sumu(segments);
+    const unsigned long long cap = warp_sumu(t.capped), esc = warp_sumu(t.escaped), tr = warp_sumu(t.traced);
+    const unsigned long long lost = warp_sumu(t.lost);
+    if (lane == 0u) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q)
+            if (v[q] != 0.0) atomicAdd(A.stats + MST_ST_ESC_XM + q, v[q]);
+        atomicAdd(A.stats + MST_ST_ABSORBED, v[6]);
+        atomicAdd(A.stats + MST_ST_RR_KILLED, v[7]);
+        atomicAdd(A.stats + MST_ST_RR_GAINED, v[8]);
+        atomicAdd(A.stats + MST_ST_FORCED, v[9]);
+        atomicAdd(A.stats + MST_ST_LAUNCHED, v[10]);
+        atomicAdd(A.stats + MST_ST_EVENTS, (double)ev);
+        atomicAdd(A.stats + MST_ST_SEGMENTS, (double)sg);
+        atomicAdd(A.stats + MST_ST_CAPPED, (double)cap);
+        atomicAdd(A.stats + MST_ST_ESCAPED_N, (double)esc);
+        atomicAdd(A.stats + MST_ST_TRACED, (double)tr);
+        if (lost) atomicAdd(A.stats + MST_ST_LOST, (double)lost);
+    }
+}
+
 // ------------------------------------------------------------------------------------------
-// The replay kernel: the two passes of the adjoint of a call whose events are not held. Every loop
+// The classic forward and the replays: the two passes of the adjoint of a classic call, or of one
+// whose events are not held. Every loop
 // trip (1) fills empty lanes from the ready stack, then from the id pool, (2) advances every flying
 // photon by up to TRIP voxels, pushing collisions onto the event stack, and (3) whenever 32 events
 // are queued (or the chunk is draining), processes 32 events at once: w_s, albedo, roulette, new
@@ -842,18 +908,35 @@ template <int DT, int MODE, bool TWO, int TRIP>
 __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* smem) {
     constexpr bool PASS1 = MODE == kPass1 || MODE == kPass1C;
     constexpr bool PASS2 = MODE == kPass2 || MODE == kPass2C;
-    constexpr bool CLASSIC = MODE == kPass1C || MODE == kPass2C;
-    static_assert(PASS1 || PASS2, "the forward is k_forward");
-    constexpr int kStepsPerTrip = TRIP > 0 ? TRIP : (PASS2 ? kStepsPass2 : kStepsPass1);
+    constexpr bool CLASSIC = MODE == kFwdClassic || MODE == kPass1C || MODE == kPass2C;
+    constexpr bool REPLAY = PASS1 || PASS2;
+    constexpr int kStepsPerTrip = TRIP > 0 ? TRIP : (PASS2 ? kStepsPass2 : (PASS1 ? kStepsPass1 : kStepsForward));
     constexpr int NW = Rec<MODE>::NW;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned warp = threadIdx.x >> 5;
     const Stack<NW> stk{smem + warp * NW * kSlots, kSlots};  // events at slot i, ready photons at kSlots-1-i
     int ev_n = 0, rd_n = 0;  // warp-uniform stack heights
 
-    NoTally t;
-    ClassicScratch cls{};  // the classic estimate's per-warp scratch, after the stacks
-    if constexpr (CLASSIC) cls = classic_scratch(smem + (kTB / 32) * NW * kSlots + warp * kClassicWords, lane);
+    // photon tallies: forward render only, one shared-memory slot per thread after the stacks
+    typename std::conditional<REPLAY, NoTally, LaneTally>::type t;
+    if constexpr (!REPLAY) {
+        float* tb = reinterpret_cast<float*>(smem + (kTB / 32) * NW * kSlots);
+        t.f = tb + threadIdx.x;
+        t.u = reinterpret_cast<unsigned*>(tb + 11 * kTB) + threadIdx.x;
+    }
+    t.zero();
+    ClassicScratch cls{};  // the classic estimate's per-warp scratch, after the stacks and tallies
+    if constexpr (CLASSIC) {
+        uint32_t* cb = smem + (kTB / 32) * NW * kSlots + (REPLAY ? 0 : kTB * 15) + warp * kClassicWords;
+        cls.res = reinterpret_cast<float*>(cb);
+        cls.pix = reinterpret_cast<int*>(cb + kClassicGroup * 32);
+        cls.job = reinterpret_cast<uint8_t*>(cb + 2 * kClassicGroup * 32);
+        cls.seg = cb + 2 * kClassicGroup * 32 + kClassicGroup * 8;
+        cls.rays = cls.seg + 32;
+        cls.seg[lane] = 0u;
+        if (lane == 0u) *cls.rays = 0u;
+        __syncwarp();
+    }
 
     Photon ph;
     Flight w;
@@ -863,9 +946,10 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     bool fly = false, dry = false;
     uint32_t wbase = 0u, wend = 0u;
     unsigned segments = 0u, scatters = 0u, events = 0u;
+    EventCount<TWO && !REPLAY> air_events;  // two species: forward events on air
     const uint32_t pool_n = PASS2 ? *A.plist_n : A.n;  // pass 2 walks the list built from pass 1
     // a call whose forward stored its events: the score kernel did the replay unless they did not fit
-    if (A.ev_cap && *A.ev_count <= A.ev_cap) return;
+    if ((PASS1 || MODE == kPass2) && A.ev_cap && *A.ev_count <= A.ev_cap) return;
 
     for (;;) {
         // (1) fill: ready photons first, new photons only when the ready stack is empty
@@ -892,6 +976,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                 nev = r.nev;
                 acc = r.W;
             } else if (A.skip && A.skip[A.out_base + j]) {
+                if (A.hash) A.hash[A.out_base + j] = 0u;
                 if (PASS1) A.wbuf[j] = 0.0;
                 if (PASS1) A.nevbuf[j] = 0u;
                 return false;
@@ -899,6 +984,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             launch_photon(A, ph, pid);
             flight_init<DT>(w, A, ph);
             tau = ph.tau;
+            t.add_launch(A.I0);
             return true;
         }, [&](uint32_t t0) { fold_slice<MODE>(A, t0 / (uint32_t)kTicketBatch, lane); });
         const bool any_fly = __any_sync(kFull, fly);
@@ -934,11 +1020,17 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             put(stk, ev_n + __popc(cmask & lanemask_lt()), ph, nev, acc);
             fly = false;
         } else if (fly && r >= 0) {
-            if (PASS1) {
-                A.wbuf[ph.idx - A.out_base] = acc;
-                A.nevbuf[ph.idx - A.out_base] = ph.s;
+            if (REPLAY) {
+                if (PASS1) {
+                    A.wbuf[ph.idx - A.out_base] = acc;
+                    A.nevbuf[ph.idx - A.out_base] = ph.s;
+                }
+                fly = false;
+            } else {
+                t.add_escape(r, ph.I);
+                finish_photon(A, ph, 1);
+                fly = false;
             }
-            fly = false;
         }
         ev_n += __popc(cmask);
         __syncwarp();
@@ -967,13 +1059,18 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                         air = particle_is_air(A, x, k);
                         stash_block(stk, slot, x);
                     }
+                    if (air) air_events.add();
                     wgt = (air ? A.albedo_air : A.albedo) * e.I;
+                    if (!REPLAY) e.hash = (e.hash ^ (uint32_t)k) * kFnvPrime;
                 }
-                const float we = le_classic<DT, PASS2 ? 2 : 1>(A, e, wgt, air, act, cls);
+                const float we = le_classic<DT, REPLAY ? (PASS2 ? 2 : 1) : 0>(A, e, wgt, air, act, cls);
                 if (act) {
                     uint4 xb = make_uint4(0u, 0u, 0u, 0u);
                     if constexpr (TWO) xb = unstash_block(stk, slot);
-                    if (PASS1) {
+                    if (!REPLAY) {
+                        term = after_event<TWO>(A, e, t, air, xb);
+                        if (term) finish_photon(A, e, term);
+                    } else if (PASS1) {
                         eacc += (double)we;
                         term = after_event<TWO>(A, e, t, air, xb);
                         if (term) {
@@ -1006,6 +1103,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
                         air = particle_is_air(A, x, k);
                         stash_block(stk, slot, x);
                     }
+                    if (air) air_events.add();
                     const float wgt = (air ? A.albedo_air : A.albedo) * e.I;
                     {
                         const float we = le_adjoint(A, e, wgt, k, air);
@@ -1039,12 +1137,23 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
             __syncwarp();
         }
     }
-    if constexpr (CLASSIC) flush_classic(A, cls, lane);
-    const unsigned long long ev = warp_sumu(events), sg = warp_sumu(segments), sc = warp_sumu(scatters);
-    if (lane == 0u) {
-        atomicAdd(A.stats + MST_ST_REPLAY_EVENTS, (double)ev);
-        atomicAdd(A.stats + MST_ST_REPLAY_SEGMENTS, (double)sg);
-        atomicAdd(A.stats + MST_ST_REPLAY_SCATTERS, (double)sc);
+    if constexpr (CLASSIC) {
+        const unsigned long long ss = warp_sumu(cls.seg[lane]);
+        if (lane == 0u) {
+            atomicAdd(A.stats + MST_ST_SHADOW_RAYS, (double)*cls.rays);
+            atomicAdd(A.stats + MST_ST_SHADOW_SEGMENTS, (double)ss);
+        }
+    }
+    if constexpr (REPLAY) {
+        const unsigned long long ev = warp_sumu(events), sg = warp_sumu(segments), sc = warp_sumu(scatters);
+        if (lane == 0u) {
+            atomicAdd(A.stats + MST_ST_REPLAY_EVENTS, (double)ev);
+            atomicAdd(A.stats + MST_ST_REPLAY_SEGMENTS, (double)sg);
+            atomicAdd(A.stats + MST_ST_REPLAY_SCATTERS, (double)sc);
+        }
+    } else {
+        flush_tally(A, t.load(), segments, events, lane);
+        air_events.flush(A.stats + MST_ST_AIR_EVENTS, lane);
     }
 }
 
@@ -1114,15 +1223,11 @@ struct EventTally {
     __device__ __forceinline__ void add_capped() { capped = 1.f; rare = true; }
 };
 
-// CL: the classic estimate (Eq. fle) into A.cimg instead of the voxelised one.
-template <int DT, bool TWO, int TRIP, bool CL>
+template <int DT, bool TWO, int TRIP>
 __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* smem) {
-    constexpr int kWords = kFwdWords + (CL ? kClassicWords : 0);
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    double* tally = reinterpret_cast<double*>(smem + warp * kWords);  // the warp's share of the statistics
-    uint32_t* sl = smem + warp * kWords + 2 * MST_NSTATS;             // word f of slot i at sl[f * kSlots + i]
-    ClassicScratch cls{};
-    if constexpr (CL) cls = classic_scratch(smem + warp * kWords + kFwdWords, lane);
+    double* tally = reinterpret_cast<double*>(smem + warp * kFwdWords);    // the warp's share of the statistics
+    uint32_t* sl = smem + warp * kFwdWords + 2 * MST_NSTATS;               // word f of slot i at sl[f * kSlots + i]
     uint32_t* esc = sl + kSlotWords * kSlots;
     uint8_t* evq = reinterpret_cast<uint8_t*>(esc + 2 * kEscSlots);  // slots of ended flights
     uint8_t* rdq = evq + kSlots;                                     // of ready photons
@@ -1364,13 +1469,10 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
             int term = -1;  // -1 idle lane, 0 goes on, > 0 ended
             int i = 0;
             EventTally t;
-            Photon e;
-            bool air = false;
-            float wgt = 0.f;
-            const bool act = (int)lane < n;
-            if (act) {
+            if ((int)lane < n) {
                 i = evq[ev_n - 1 - (int)lane];
                 const uint32_t* s = sl + i;
+                Photon e;
                 e.d = make_float3(__uint_as_float(s[(kSD + 0) * kSlots]), __uint_as_float(s[(kSD + 1) * kSlots]),
                                   __uint_as_float(s[(kSD + 2) * kSlots]));
                 const int at = (int)s[kSLin * kSlots];
@@ -1390,6 +1492,7 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
                 e.id = A.first_id + (e.idx - A.out_base);
                 ++events;
                 const int k = lin_index(A.g, e.ix, e.iy, e.iz);
+                bool air = false;
                 if constexpr (TWO) {
                     // the event's Philox block: its scattering step needs it again, and it waits in
                     // the flight's words meanwhile (volatile, so that no register holds it)
@@ -1402,15 +1505,11 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
                     o[3 * kSlots] = x.w;
                 }
                 if (air) air_events.add();
-                wgt = (air ? A.albedo_air : A.albedo) * e.I;
+                const float wgt = (air ? A.albedo_air : A.albedo) * e.I;
                 if (A.hash) A.hash[e.idx] = (A.hash[e.idx] ^ (uint32_t)k) * kFnvPrime;
                 if (A.point) write_point(A, e);
                 if (A.ev_cap && ev_slot < A.ev_cap) store_event(A, ev_slot, e, wgt, air, s[kSPrev * kSlots]);
-                if constexpr (!CL) le_voxel(A, e, wgt, k, air);
-            }
-            // the classic estimate runs on the whole warp: its shadow rays are spread over all lanes
-            if constexpr (CL) le_classic<DT, 0>(A, e, wgt, air, act, cls);
-            if (act) {
+                le_voxel(A, e, wgt, k, air);
                 uint4 xb = make_uint4(0u, 0u, 0u, 0u);
                 if constexpr (TWO) {
                     const volatile uint32_t* o = sl + i + kST * kSlots;
@@ -1444,7 +1543,6 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
         }
     }
     while (esc_n > 0) count_escapes(min(32, esc_n));
-    if constexpr (CL) flush_classic(A, cls, lane);
     {
         const unsigned long long ev = warp_sumu(events), sg = warp_sumu(segments), la = warp_sumu(launched),
                                  es = warp_sumu(escaped);
@@ -1469,16 +1567,14 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
     }
 }
 
-template <bool CL = false>
 constexpr size_t forward_smem() {
-    return (size_t)kTransportWarps * (kFwdWords + (CL ? kClassicWords : 0)) * sizeof(uint32_t);
+    return (size_t)kTransportWarps * kFwdWords * sizeof(uint32_t);
 }
 
-// (the classic estimate has its shadow rays' state beside the walk: three blocks an SM)
-template <int DT, bool TWO, int TRIP, bool CL = false>
-__global__ void __launch_bounds__(kFT, CL ? kMinBlocksClassic : kMinBlocksForward) k_forward(const TransportArgs A) {
+template <int DT, bool TWO, int TRIP>
+__global__ void __launch_bounds__(kFT, kMinBlocksForward) k_forward(const TransportArgs A) {
     extern __shared__ uint32_t smem[];
-    forward_run<DT, TWO, TRIP, CL>(A, smem);
+    forward_run<DT, TWO, TRIP>(A, smem);
 }
 
 // Many scenes in one persistent launch: every warp runs the scenes of the table one after another
@@ -1487,7 +1583,7 @@ __global__ void __launch_bounds__(kFT, kMinBlocksForward)
     k_forward_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
     extern __shared__ uint32_t smem[];
     for (int s = 0; s < n_scenes; ++s) {
-        forward_run<0, false, TRIP, false>(scenes[s], smem);
+        forward_run<0, false, TRIP>(scenes[s], smem);
         __syncwarp();
     }
 }
@@ -1516,9 +1612,9 @@ constexpr int kFlightWords = 10;  // of a queued flight
 constexpr int kScoreSlots = 64;   // flights a warp queues: fewer than 32 left when a batch adds 32
 constexpr uint32_t kNoEntry = 0xFFFFFFFFu;
 
-template <int K, bool CL>
-constexpr int score_words() {  // shared words per warp: a batch of records, the queue, the strip, the classic scratch
-    return 3 * 4 * 32 + kFlightWords * kScoreSlots + 2 * 32 * K + (CL ? kClassicWords : 0);
+template <int K>
+constexpr int score_words() {  // shared words per warp: a batch of records, the queue, the strip
+    return 3 * 4 * 32 + kFlightWords * kScoreSlots + 2 * 32 * K;
 }
 
 // One axis of a score flight: the distance to the next face and between faces, as flight_axis
@@ -1536,17 +1632,13 @@ __device__ __forceinline__ void copy16_async(uint32_t* dst, const uint4* src) {
                  : "memory");
 }
 
-// CL: w_s of the classic estimate, whose shadow rays are walked for it and walked again to scatter
-// their own terms (le_classic) into the padded tile.
-template <int DT, bool TWO, int K, bool CL>
+template <int DT, bool TWO, int K>
 __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem) {
     if (*A.ev_count > A.ev_cap) return;  // the events did not fit: the replay passes run instead
     const unsigned lane = threadIdx.x & 31u;
-    uint32_t* rec = smem + (threadIdx.x >> 5) * score_words<K, CL>();  // the lane's record words f at rec[(f * 32 + lane) * 4]
+    uint32_t* rec = smem + (threadIdx.x >> 5) * score_words<K>();  // the lane's record words f at rec[(f * 32 + lane) * 4]
     uint32_t* q = rec + 3 * 4 * 32;                                // queue: word f of slot i at q[f * kScoreSlots + i]
     float2* strip = reinterpret_cast<float2*>(q + kFlightWords * kScoreSlots);
-    ClassicScratch cls{};
-    if constexpr (CL) cls = classic_scratch(q + kFlightWords * kScoreSlots + 2 * 32 * K, lane);
     const unsigned nbins = (unsigned)brick_bins(A.g);
     float* tile = A.gbrk + (size_t)(blockIdx.x % A.score_tiles) * nbins;  // the block's copy
     const uint32_t by8 = 8u * (unsigned)((A.g.nx + 1) >> 1), bz8 = by8 * (unsigned)((A.g.ny + 1) >> 1);
@@ -1586,14 +1678,6 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
                 int k;
                 if (v != 0.f && brick_voxel(A.g, (int)(i % nbins), k)) atomicAdd(A.g64 + k, (double)v);
             }
-            if constexpr (CL) {  // and one of the padded tile that the shadow rays add to
-                const uint32_t p0 = ch % A.pad_nslices * A.pad_slice, p1 = min(p0 + A.pad_slice, (uint32_t)A.g.npad);
-                for (uint32_t i = p0 + lane; i < p1; i += 32) {
-                    const float v = atomicExch(A.gacc + i, 0.f);
-                    int k;
-                    if (v != 0.f && interior_lin(A.g, (int)i, k)) atomicAdd(A.g64 + k, (double)v);
-                }
-            }
         }
         const uint4* r = A.evrec + ((unsigned long long)ch * kEvChunk + (unsigned)base + lane);
 #pragma unroll
@@ -1630,9 +1714,7 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
                 b = BetaFetch<DT>::get(A.beta_pad, pad_index(A.g, e.ix, e.iy, e.iz));
             }
             fetch();
-            float w = 0.f;
-            if constexpr (CL) w = le_classic<DT, 2>(A, e, __uint_as_float(r1.w), air, on, cls);
-            else if (on) w = le_adjoint(A, e, __uint_as_float(r1.w), k, air);
+            const float w = on ? le_adjoint(A, e, __uint_as_float(r1.w), k, air) : 0.f;
             // S: later events first. A batch may hold two events of a photon (rounds of fewer than
             // 32 while the forward's warp drained): they take turns, the later record first.
             const unsigned same = __match_any_sync(kFull, r2.x);
@@ -1747,10 +1829,9 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
         }
         __syncwarp();
     }
-    if constexpr (CL) flush_classic(A, cls, lane);
     const unsigned long long se = warp_sumu(stored), sf = warp_sumu(flights), sn = warp_sumu(entries), sl = warp_sumu(lost);
     if (lane == 0u) {
-        if (!CL && se) atomicAdd(A.stats + MST_ST_EVENTS_STORED, (double)se);  // (counts the voxelised estimate's)
+        if (se) atomicAdd(A.stats + MST_ST_EVENTS_STORED, (double)se);
         atomicAdd(A.stats + MST_ST_REPLAY_EVENTS, (double)sf);
         atomicAdd(A.stats + MST_ST_REPLAY_SEGMENTS, (double)sn);
         atomicAdd(A.stats + MST_ST_REPLAY_SCATTERS, (double)sn);
@@ -1758,10 +1839,10 @@ __device__ __forceinline__ void score_run(const TransportArgs& A, uint32_t* smem
     }
 }
 
-template <int DT, bool TWO, int K, bool CL = false>
-__global__ void __launch_bounds__(kFT, CL ? kMinBlocksClassic : kMinBlocksScore) k_score(const TransportArgs A) {
+template <int DT, bool TWO, int K>
+__global__ void __launch_bounds__(kFT, kMinBlocksScore) k_score(const TransportArgs A) {
     extern __shared__ uint32_t smem[];
-    score_run<DT, TWO, K, CL>(A, smem);
+    score_run<DT, TWO, K>(A, smem);
 }
 
 // the batched form: the scenes of a table one after the other
@@ -1770,7 +1851,7 @@ __global__ void __launch_bounds__(kFT, kMinBlocksScore)
     k_score_batch(const TransportArgs* __restrict__ scenes, int n_scenes) {
     extern __shared__ uint32_t smem[];
     for (int s = 0; s < n_scenes; ++s) {
-        score_run<0, false, K, false>(scenes[s], smem);
+        score_run<0, false, K>(scenes[s], smem);
         __syncwarp();
     }
 }
@@ -1889,17 +1970,21 @@ __global__ void k_fold_grad(float* __restrict__ gacc, double* __restrict__ g64, 
     }
 }
 
-// dynamic shared memory of a replay block: the warps' photon stacks and the classic estimate's scratch
+// dynamic shared memory of a transport block: the warps' photon stacks, the forward's tallies
+// and the classic estimate's scratch
 template <int MODE>
 constexpr size_t smem_bytes() {
-    constexpr bool CLASSIC = MODE == kPass1C || MODE == kPass2C;
-    return (size_t)(kTB / 32) * (Rec<MODE>::NW * kSlots + (CLASSIC ? kClassicWords : 0)) * sizeof(uint32_t);
+    constexpr bool REPLAY = MODE >= 2;
+    constexpr bool CLASSIC = MODE == kFwdClassic || MODE == kPass1C || MODE == kPass2C;
+    return (size_t)(kTB / 32) * Rec<MODE>::NW * kSlots * sizeof(uint32_t) +
+           (REPLAY ? 0 : (size_t)kTB * 15 * sizeof(uint32_t)) +
+           (CLASSIC ? (size_t)(kTB / 32) * kClassicWords * sizeof(uint32_t) : 0);
 }
 
 // the score kernel's: the warps' flight queues and entry strips
-template <int K, bool CL = false>
+template <int K>
 constexpr size_t score_smem() {
-    return (size_t)kTransportWarps * score_words<K, CL>() * sizeof(uint32_t);
+    return (size_t)kTransportWarps * score_words<K>() * sizeof(uint32_t);
 }
 
 template <typename K>
@@ -1966,9 +2051,7 @@ template <int DT, bool TWO>
 int occupancy_mode(int mode) {
     switch (mode) {
         case kFwdVoxel: return occupancy(k_forward<DT, TWO, kStepsForward>, forward_smem(), kMinBlocksForward, kFT);
-        case kFwdClassic:
-            occupancy(k_score<DT, TWO, kStepsScore, true>, score_smem<kStepsScore, true>(), kMinBlocksClassic, kFT);
-            return occupancy(k_forward<DT, TWO, kStepsForward, true>, forward_smem<true>(), kMinBlocksClassic, kFT);
+        case kFwdClassic: return occupancy(k_transport<DT, kFwdClassic, TWO>, smem_bytes<kFwdClassic>());
         case kPass2: return occupancy(k_transport<DT, kPass2, TWO>, smem_bytes<kPass2>());
         case kScore: return occupancy(k_score<DT, TWO, kStepsScore>, score_smem<kStepsScore>(), kMinBlocksScore, kFT);
         case kPass1C: return occupancy(k_transport<DT, kPass1C, TWO>, smem_bytes<kPass1C>());
@@ -1984,9 +2067,7 @@ cudaError_t launch_dt(const TransportArgs& a, int mode, int trip, int blocks, cu
     }
     switch (mode) {
         case kFwdVoxel: return launch_forward<DT, TWO>(a, trip, blocks, st);
-        case kFwdClassic:
-            k_forward<DT, TWO, kStepsForward, true><<<blocks, kFT, forward_smem<true>(), st>>>(a);
-            return cudaGetLastError();
+        case kFwdClassic: return launch_mode<DT, kFwdClassic, TWO>(a, blocks, st);
         case kPass2: return launch_mode<DT, kPass2, TWO>(a, blocks, st);
         case kPass1C: return launch_mode<DT, kPass1C, TWO>(a, blocks, st);
         case kPass2C: return launch_mode<DT, kPass2C, TWO>(a, blocks, st);
@@ -2121,23 +2202,7 @@ cudaError_t launch_score_dt(const TransportArgs& a, int dtype, int trip, int blo
 
 }  // namespace
 
-namespace {
-
-template <bool TWO>
-cudaError_t launch_score_classic(const TransportArgs& a, int dtype, int blocks, cudaStream_t st) {
-    constexpr int K = kStepsScore;
-    if (dtype == 0) k_score<0, TWO, K, true><<<blocks, kFT, score_smem<K, true>(), st>>>(a);
-    else if (dtype == 1) k_score<1, TWO, K, true><<<blocks, kFT, score_smem<K, true>(), st>>>(a);
-    else k_score<2, TWO, K, true><<<blocks, kFT, score_smem<K, true>(), st>>>(a);
-    return cudaGetLastError();
-}
-
-}  // namespace
-
-cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, bool classic, int blocks,
-                         cudaStream_t st) {
-    if (classic) return a.beta_air ? launch_score_classic<true>(a, dtype, blocks, st)
-                                   : launch_score_classic<false>(a, dtype, blocks, st);
+cudaError_t launch_score(const mst_grid* g, const TransportArgs& a, int dtype, int blocks, cudaStream_t st) {
     const int trip = g->wf_trip[kScore];
     return a.beta_air ? launch_score_dt<true>(a, dtype, trip, blocks, st)
                       : launch_score_dt<false>(a, dtype, trip, blocks, st);
