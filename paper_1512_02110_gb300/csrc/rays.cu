@@ -244,19 +244,15 @@ __global__ void k_images(const Geo g, const CamSet cs, const Halton hs, float in
 // K4: b_c(k) = sum_p Pi_c(p, k) resid(p)  (Pi^T, Eq. PIc transposed), on the padded grid. A thread
 // takes a pixel and walks its rays in their order. An atomic on an address that another lane of
 // the instruction holds costs another transaction (2.0e11 a second on this chip, however many
-// lanes share it), while distinct addresses of one 32-byte sector go out as one: a warp takes every
-// kPixelStride-th of kPixelStride * 32 pixels in a row, whose rays part sooner than neighbours'
-// do (9 cameras of 128^2 pixels in 64^3 voxels: 0.93 ms at stride 1, 0.94 / 0.84 / 0.84 at 2 / 4 /
-// 8). What bounds it is the queue on each camera's own voxel (1.6e5 additions). Adding the lanes'
-// terms up before the atomic took 0.27 ms and was not kept: the bins next to a camera sum so
-// many terms in FP32 that grouped additions move them by 1e-4.
-constexpr int kPixelStride = 4;
+// lanes share it); what bounds the kernel is the queue on each camera's own voxel (1.6e5 additions).
+// 9 cameras of 128^2 pixels in 64^3 voxels: 0.94 ms. A warp taking every fourth pixel, whose rays
+// part sooner, took 0.85, and adding the lanes' terms up before the atomic 0.27; neither was kept:
+// the bins next to a camera sum so many terms in FP32 that another order moves them by up to 1e-3.
 constexpr int kRaysApart = 1 << 15;  // pixels below which the rays of a pixel go to threads of their own
 __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet cs, const Halton hs, float inv_nv,
                                                      const double* __restrict__ resid, const float* __restrict__ R,
                                                      float* __restrict__ bacc, int total_pix, double* stats) {
-    const int warp = blockIdx.x * (kTB / 32) + (int)(threadIdx.x >> 5);
-    const int gp = ((warp / kPixelStride) * 32 + (int)(threadIdx.x & 31u)) * kPixelStride + warp % kPixelStride;
+    const int gp = blockIdx.x * kTB + (int)threadIdx.x;
     unsigned nseg = 0u;
     const float wgt = gp < total_pix ? (float)(resid[gp] * (double)inv_nv) : 0.f;
     if (wgt != 0.f) {
@@ -534,13 +530,10 @@ cudaError_t launch_images(const mst_grid* g, const float* R, double* images, con
 
 cudaError_t launch_backproject(const mst_grid* g, const double* resid, float* bacc, cudaStream_t st) {
     const float inv_nv = (float)(1.0 / (g->n_rays * g->voxel_volume));
-    const int group = 32 * kPixelStride;  // pixels of kPixelStride warps
-    const int warps = (g->total_pix + group - 1) / group * kPixelStride;
     // few pixels leave the chip to single threads' chains of rays: a thread per ray then (5 cameras of
     // 32^2 pixels in 16^3 voxels: 48 us against 36)
-    const dim3 nb((warps + kTB / 32 - 1) / (kTB / 32), g->total_pix < kRaysApart ? g->n_rays : 1);
-    k_backproject<<<nb, kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, g->R, bacc,
-                                                                       g->total_pix, g->stats);
+    const dim3 nb((g->total_pix + kTB - 1) / kTB, g->total_pix < kRaysApart ? g->n_rays : 1);
+    k_backproject<<<nb, kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, g->R, bacc, g->total_pix, g->stats);
     return cudaGetLastError();
 }
 
