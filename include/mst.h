@@ -170,9 +170,9 @@ int mst_render(mst_grid *g, const float *beta_dev, const mst_params *p, double *
  * dL/dbeta is estimated by the score of the free-flight density (Eq. beer-lambert,
  * Eq. MCextinct) along every path, from the events the forward render stored (48 B per event,
  * within the handle's budget, see mst_set_replay_memory), or, when they do not fit, by two replays
- * of the paths from their Philox keys. Results agree either way. With MST_EST_CLASSIC the
- * images are Eq. fle's, w_s weights each camera's classic contribution by its pixel's dE/di,
- * and each contribution's shadow ray adds its own term. The surrogate gradient needs the voxel
+ * of the paths from their Philox keys. Results agree either way. With MST_EST_CLASSIC (always by
+ * replay) the images are Eq. fle's, w_s weights each camera's classic contribution by its pixel's
+ * dE/di, and each contribution's shadow ray adds its own term. The surrogate gradient needs the voxel
  * estimator. */
 int mst_render_grad(mst_grid *g, const float *beta_dev, const mst_params *p, const double *images_meas_dev,
                     const uint8_t *mask_dev, double *images_dev, double *grad_dev, double *loss_dev, void *stream);

@@ -62,18 +62,12 @@ def test_score_of_stored_events_matches_the_replay(m, shape, cams, photons, zeni
     assert eg < 1e-5, eg
 
 
-@pytest.mark.parametrize("budget", ["stored", "replay"])
 @pytest.mark.parametrize("shape,cams,photons,zenith", CASES)
-def test_classic_gradient_matches_the_oracle(m, shape, cams, photons, zenith, budget):
-    """The classic estimate's gradient, from the stored events and by the replay passes, against the
-    FP64 oracle on the photons whose paths agree. (Not one against the other as above: next to a
-    camera in the cloud the terms are large and nearly cancel, and the replay's one FP32 tile
-    repeats itself to 3e-5 only, the stored events' to 2e-6.) 1e-3: the bound of the repository's
-    other gradients against the oracle."""
+def test_classic_gradient_matches_the_oracle(m, shape, cams, photons, zenith):
+    """The classic estimate's gradient against the FP64 oracle on the photons whose paths agree.
+    1e-3: the bound of the repository's other gradients against the oracle."""
     sc, p, opt, meas = _full_gradient(shape, cams, photons, zenith, "classic")
     beta, grid = dev(sc.beta, np.float32), m.Grid.from_scene(sc)
-    if budget == "replay":
-        grid.set_replay_memory(0)
     ref_hash = oracle.render(sc, p, want_L=False, hashes=True)["hash"]
     skip = (gpu_hashes(m, grid, beta, m.make_params(p), photons) != ref_hash).astype(np.uint8)
     assert skip.mean() < 2e-3
@@ -85,7 +79,7 @@ def test_classic_gradient_matches_the_oracle(m, shape, cams, photons, zenith, bu
     assert grid.stats()["lost"] == 0
     eg = rel_l2(out["grad"].cpu().numpy(), ref["grad"])
     el = abs(out["loss"].item() - ref["loss"]) / ref["loss"]
-    record(f"classic_gradient[{shape},{cams},{photons},{budget}]", grad_rel_l2=eg, loss=el)
+    record(f"classic_gradient[{shape},{cams},{photons}]", grad_rel_l2=eg, loss=el)
     assert eg < 1e-3 and el < 1e-3, (eg, el)
 
 
