@@ -429,11 +429,13 @@ double radical_inverse(int base, int i) {
 }
 
 void free_all(mst_grid* g) {
-    void* ptrs[] = {g->arena, g->Qw, g->wbuf, g->nevbuf, g->plist};
+    void* ptrs[] = {g->ext, g->ext_pad, g->Lacc, g->L64, g->T, g->R, g->bacc, g->gT, g->adj, g->gacc, g->g64,
+                    g->resid, g->cimg, g->lap, g->omega, g->Qw, g->stats, g->tickets, g->wbuf, g->nevbuf, g->plist, g->score_cnt};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     drop_records(g);
     cudaFree(g->warp_tail);
+    cudaFree(g->gbrk);
     cudaFree(g->reg_wz);
     cudaFree(g->ch_beta);
     cudaFree(g->ch_grad);
@@ -594,44 +596,36 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     }
 
     const size_t nvox = (size_t)geo.nvox, C = (size_t)n_cams;
-    // One allocation for the handle's arrays, those that start at zero first: an allocation and a
-    // memset cost several microseconds each (creation of a 16^3 handle with five cameras 328 -> 299 us).
     struct A {
         void** p;
         size_t bytes;
-    } arrays[] = {
-        {(void**)&g->Lacc, nvox * g->cp * 4},
-        {(void**)&g->gacc, (size_t)geo.npad * 4},
-        {(void**)&g->gbrk, (size_t)brick_bins(geo) * g->score_tiles * 4},
-        {(void**)&g->stats, MST_NSTATS * 8 + 64},
-        {(void**)&g->R, C * geo.npad * 4},  // the first that does not
+    } allocs[] = {
         {&g->ext_pad, (size_t)geo.npad * 4},
+        {(void**)&g->Lacc, nvox * g->cp * 4},
         {(void**)&g->L64, C * nvox * 8},
         {(void**)&g->T, C * nvox * 4},
+        {(void**)&g->R, C * geo.npad * 4},
         {(void**)&g->bacc, C * geo.npad * 4},
         {(void**)&g->gT, C * geo.npad * 4},
         {(void**)&g->adj, nvox * g->cp * 4},
+        {(void**)&g->gacc, (size_t)geo.npad * 4},
+        {(void**)&g->gbrk, (size_t)brick_bins(geo) * g->score_tiles * 4},
         {(void**)&g->score_cnt, (2 * kScoreBins + 1) * 4},
         {(void**)&g->g64, nvox * 8},
         {(void**)&g->resid, (size_t)off * 8},
         {(void**)&g->cimg, (size_t)off * 8},
         {(void**)&g->lap, nvox * 8},
         {(void**)&g->omega, (size_t)off * 4},
+        {(void**)&g->stats, MST_NSTATS * 8 + 64},
         {(void**)&g->tickets, (size_t)kMaxTickets * 4},
     };
-    auto rounded = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
-    size_t total = 0;
-    for (const A& a : arrays) total += rounded(a.bytes);
-    if (cudaMalloc(&g->arena, total) != cudaSuccess) {
-        cudaGetLastError();
-        free_all(g);
-        delete g;
-        return MST_ERR_OOM;
-    }
-    char* at = (char*)g->arena;
-    for (const A& a : arrays) {
-        *a.p = at;
-        at += rounded(a.bytes);
+    for (auto& a : allocs) {
+        if (cudaMalloc(a.p, a.bytes) != cudaSuccess) {
+            cudaGetLastError();
+            free_all(g);
+            delete g;
+            return MST_ERR_OOM;
+        }
     }
     // pixel solid angles for the classic estimator (exact rectangle formula, FP64 on the host)
     float* om = new float[off];
@@ -647,8 +641,11 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     }
     cudaError_t e = cudaMemcpy(g->omega, om, sizeof(float) * off, cudaMemcpyHostToDevice);
     delete[] om;
-    if (e == cudaSuccess) e = cudaMemset(g->arena, 0, (size_t)((char*)g->R - (char*)g->arena));
     if (e == cudaSuccess) e = cudaMemset(g->R, 0xFF, C * geo.npad * 4);  // the halo's mark (k_los writes the rest)
+    if (e == cudaSuccess) e = cudaMemset(g->Lacc, 0, nvox * g->cp * 4);
+    if (e == cudaSuccess) e = cudaMemset(g->gacc, 0, (size_t)geo.npad * 4);
+    if (e == cudaSuccess) e = cudaMemset(g->gbrk, 0, (size_t)brick_bins(geo) * g->score_tiles * 4);
+    if (e == cudaSuccess) e = cudaMemset(g->stats, 0, MST_NSTATS * 8 + 64);
     if (e != cudaSuccess) {
         free_all(g);
         delete g;

@@ -115,8 +115,7 @@ struct mst_grid {
     double origin[3] = {0, 0, 0};
     double voxel_volume = 0;
 
-    // device buffers owned by the handle; those that every call uses lie in one allocation
-    void* arena = nullptr;
+    // device buffers owned by the handle
     void* ext = nullptr;          // staged extinction [nvox] of a call without a handle (mst_transmittance_noalloc)
     void* ext_pad = nullptr;      // staged extinction on the padded grid [npad] (photon flights)
     float* Lacc = nullptr;        // [nvox][cp]
