@@ -245,7 +245,7 @@ __global__ void k_images(const Geo g, const CamSet cs, const Halton hs, float in
 // takes a pixel and walks its rays in their order. An atomic on an address that another lane of
 // the instruction holds costs another transaction (2.0e11 a second on this chip, however many
 // lanes share it); what bounds the kernel is the queue on each camera's own voxel (1.6e5 additions).
-// 9 cameras of 128^2 pixels in 64^3 voxels: 0.94 ms. A warp taking every fourth pixel, whose rays
+// 9 cameras of 128^2 pixels in 64^3 voxels: 0.94-0.99 ms. A warp taking every fourth pixel, whose rays
 // part sooner, took 0.85, and adding the lanes' terms up before the atomic 0.27; neither was kept:
 // the bins next to a camera sum so many terms in FP32 that another order moves them by up to 1e-3.
 constexpr int kRaysApart = 1 << 15;  // pixels below which the rays of a pixel go to threads of their own
