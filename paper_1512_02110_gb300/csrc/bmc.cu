@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kTB, kBmcBlocks) k_bmc(const BmcArgs A) {
                 const float m = w.face(px, py, next);
                 bn = BetaFetch<DT>::get(A.beta, next);  // at most the second halo layer
                 const float bs = __fmul_rn(b, m);
-                if (sun ? isinf(b) : tau <= bs) {
+                if (ray_ends(!sun, tau, b, bs)) {
                     end = true;
                     break;
                 }
@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kTB, kBmcBlocks) k_bmc(const BmcArgs A) {
             }
         }
         if (ray != kIdle && left < 0) {
+            if (!end) atomicAdd(A.stats + MST_ST_LOST, 1.0);  // abandoned
             if (ray == kFlight) {
                 finish();
             } else {  // on from the event

@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <math_constants.h>
 #include <stdint.h>
 
@@ -177,7 +178,7 @@ __device__ __forceinline__ float3 rotate_dir(float3 d, float ct, float st, float
 __device__ __forceinline__ int lin_index(const Geo& g, int ix, int iy, int iz) { return ix + g.nx * (iy + g.ny * iz); }
 
 // index of voxel (ix, iy, iz) in the padded grid (each index may lie in the halo, -kHalo .. n + kHalo - 1)
-__device__ __forceinline__ int pad_index(const Geo& g, int ix, int iy, int iz) {
+__host__ __device__ __forceinline__ int pad_index(const Geo& g, int ix, int iy, int iz) {
     return (ix + kHalo) + g.p0 * (iy + kHalo) + g.p01 * (iz + kHalo);
 }
 
@@ -374,27 +375,38 @@ struct PadWalk {
     int dx, dy, dz, lin;
 
     PadWalk() = default;
-    static __device__ __forceinline__ void axis(float p, float d, float h, int stride, float& t, float& q, int& dl) {
-        float a;
-        int s;
-        axis_init<false>(p, d, h, t, q, a, s);
-        dl = s * stride;
+    static __host__ __device__ __forceinline__ void axis(float p, float d, float h, int stride, float& t, float& q, int& dl) {
+        if (d > 0.f) {
+            const float inv = 1.f / d;
+            t = (h - p) * inv;
+            q = h * inv;
+            dl = stride;
+        } else if (d < 0.f) {
+            const float inv = 1.f / -d;
+            t = p * inv;
+            q = h * inv;
+            dl = -stride;
+        } else {
+            t = INFINITY;
+            q = INFINITY;
+            dl = 0;
+        }
     }
     // from offset p of voxel `at` of a grid with the strides 1, sy, sz
-    __device__ __forceinline__ PadWalk(const Geo& g, float3 p, float3 d, int at, int sy, int sz) : lin(at) {
+    __host__ __device__ __forceinline__ PadWalk(const Geo& g, float3 p, float3 d, int at, int sy, int sz) : lin(at) {
         axis(fminf(fmaxf(p.x, 0.f), g.hx), d.x, g.hx, 1, tx, qx, dx);
         axis(fminf(fmaxf(p.y, 0.f), g.hy), d.y, g.hy, sy, ty, qy, dy);
         axis(fminf(fmaxf(p.z, 0.f), g.hz), d.z, g.hz, sz, tz, qz, dz);
     }
     // distance to the next face, the axis it belongs to (ties to x, then y, then z), the voxel behind it
-    __device__ __forceinline__ float face(bool& px, bool& py, int& next) const {
+    __host__ __device__ __forceinline__ float face(bool& px, bool& py, int& next) const {
         const float m = fminf(tx, fminf(ty, tz));
         px = tx <= m;
         py = !px && ty <= m;
         next = lin + (px ? dx : (py ? dy : dz));
         return m;
     }
-    __device__ __forceinline__ void cross(float m, bool px, bool py, int next) {
+    __host__ __device__ __forceinline__ void cross(float m, bool px, bool py, int next) {
         tx = px ? qx : tx - m;
         ty = py ? qy : ty - m;
         tz = (px || py) ? tz - m : qz;
@@ -402,8 +414,16 @@ struct PadWalk {
     }
 };
 
-__device__ __forceinline__ PadWalk pad_walk(const Geo& g, float3 p, float3 d, int ix, int iy, int iz) {
+__host__ __device__ __forceinline__ PadWalk pad_walk(const Geo& g, float3 p, float3 d, int ix, int iy, int iz) {
     return PadWalk(g, p, d, pad_index(g, ix, iy, iz), g.p0, g.p01);
+}
+
+// Whether a ray on the padded grid ends in a voxel of extinction b and optical depth bs = b * (distance to
+// the next face): every ray in the halo (b = +inf), a flight also where its free path tau runs out. The
+// halo is told by b alone: a ray that leaves the grid exactly on a voxel's edge crosses its first
+// halo voxel over no distance, where bs is inf * 0 = NaN and no comparison with it ends the walk.
+__host__ __device__ __forceinline__ bool ray_ends(bool flight, float tau, float b, float bs) {
+    return isinf(b) || (flight && tau <= bs);
 }
 
 // offset inside the current voxel of the point a distance l past the current point

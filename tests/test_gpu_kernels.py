@@ -111,3 +111,18 @@ def test_rays_match_the_oracle(m, shape, cams, n_rays, px, outside):
     eg = rel_l2(out["grad"].cpu().numpy(), ref["grad"])
     record(f"rays[{shape},{n_rays},{px}]", T=eT[0], T_noalloc=eT[1], images=ei, loss=el, grad=eg)
     assert max(eT) <= 1.0 and ei < 1e-4 and el < 1e-4 and eg < 1e-3, (eT, ei, el, eg)
+
+
+@pytest.mark.parametrize("shape,cams,paths", [((1, 1, 1), 1, 33), ((5, 7, 9), 3, 64), ((33, 17, 12), 5, 200)])
+def test_backward_paths_all_end(m, shape, cams, paths):
+    """Every backward path ends in a collision or at the grid's boundary: none is abandoned, and a ray
+    crosses no more voxels than a straight line through the grid has."""
+    sc = _scene(shape, cams, 9)
+    grid = m.Grid.from_scene(sc)
+    p = synth.Params(albedo=0.95, g=0.7, sun_zenith=0.5, sun_azimuth=0.4, seed=21)
+    out = grid.render_bmc(dev(sc.beta, np.float32), m.make_params(p), paths)
+    st = grid.stats()
+    assert st["lost"] == 0 and st["bmc_paths"] == paths * sc.n_pix and st["bmc_events"] > 0
+    # one flight a path and two rays an event
+    assert st["bmc_segments"] <= (st["bmc_paths"] + 2 * st["bmc_events"]) * sum(shape)
+    assert np.isfinite(out["images"].cpu().numpy()).all()
