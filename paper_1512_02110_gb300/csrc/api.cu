@@ -646,6 +646,9 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     if (e == cudaSuccess) e = cudaMemset(g->gacc, 0, (size_t)geo.npad * 4);
     if (e == cudaSuccess) e = cudaMemset(g->gbrk, 0, (size_t)brick_bins(geo) * g->score_tiles * 4);
     if (e == cudaSuccess) e = cudaMemset(g->stats, 0, MST_NSTATS * 8 + 64);
+    // The handle's first call may run on any stream, also one that does not wait for this one: pixel rays
+    // stop at R's halo alone, and a late clear would undo what that call has written.
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         free_all(g);
         delete g;

@@ -4,6 +4,7 @@ of the score's tile), camera counts around the groups of two, four and eight, a 
 (flights along one axis only), sub-pixel ray counts that do not divide a block."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import synth
@@ -126,3 +127,23 @@ def test_backward_paths_all_end(m, shape, cams, paths):
     # one flight a path and two rays an event
     assert st["bmc_segments"] <= (st["bmc_paths"] + 2 * st["bmc_events"]) * sum(shape)
     assert np.isfinite(out["images"].cpu().numpy()).all()
+
+
+def test_a_new_handle_is_ready_for_any_stream(m):
+    """Creation leaves no work in flight: the clears of the handle's buffers (here some 0.3 GB, behind work
+    that was queued before) are done when it returns, so that a first call on a stream that does not wait
+    for the default one finds R's halo marked and the tiles empty."""
+    torch.cuda.synchronize()
+    sc = _scene((128, 128, 128), 16, 3, px=(4, 4))
+    torch.cuda._sleep(1_000_000)
+    grid = m.Grid.from_scene(sc)
+    assert torch.cuda.default_stream().query()
+    beta = dev(sc.beta, np.float32)
+    L = dev(np.ones((16, sc.nvox)), np.float64)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()  # (torch's streams do not block on the legacy one)
+    fresh = m.Grid.from_scene(sc)
+    with torch.cuda.stream(side):
+        img = fresh.form_images(beta, L)
+    side.synchronize()
+    assert torch.equal(img, grid.form_images(beta, L))
