@@ -605,8 +605,8 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         {(void**)&g->L64, C * nvox * 8},
         {(void**)&g->T, C * nvox * 4},
         {(void**)&g->R, C * geo.npad * 4},
-        {(void**)&g->bacc, C * geo.npad * 4},
-        {(void**)&g->gT, C * geo.npad * 4},
+        {(void**)&g->bacc, C * nvox * 4},
+        {(void**)&g->gT, C * nvox * 4},
         {(void**)&g->adj, nvox * g->cp * 4},
         {(void**)&g->gacc, (size_t)geo.npad * 4},
         {(void**)&g->gbrk, (size_t)brick_bins(geo) * g->score_tiles * 4},
@@ -757,7 +757,7 @@ int check_render_grad(mst_grid* g, const float* beta, const mst_params* p, const
 int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const double* meas, const uint8_t* mask,
                      double* images, double* grad, double* loss, cudaStream_t st) {
     int rc = MST_OK;
-    const size_t nL = (size_t)g->n_cams * g->geo.nvox, nP = (size_t)g->n_cams * g->geo.npad;
+    const size_t nL = (size_t)g->n_cams * g->geo.nvox;
     double* lossp = loss ? loss : g->stats + MST_NSTATS;
     g->beta_in = beta;
     {
@@ -816,12 +816,12 @@ int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const 
         Phase ph(g, MST_PH_IMAGES, st);
         MST_CK(launch_images(g, g->R, images, meas, mask, g->resid, lossp, st));
     }
-    MST_CK(cudaMemsetAsync(g->bacc, 0, sizeof(float) * nP, st));
+    MST_CK(cudaMemsetAsync(g->bacc, 0, sizeof(float) * nL, st));
     {
         Phase ph(g, MST_PH_BACKPROJECT, st);
         MST_CK(launch_backproject(g, g->resid, g->bacc, st));
     }
-    MST_CK(cudaMemsetAsync(g->gT, 0, sizeof(float) * nP, st));
+    MST_CK(cudaMemsetAsync(g->gT, 0, sizeof(float) * nL, st));
     {
         Phase ph(g, MST_PH_LOS_ADJOINT, st);
         MST_CK(launch_los_adjoint(g, g->R, g->bacc, g->gT, st));
@@ -912,7 +912,7 @@ int mst_surrogate_grad(mst_grid* g, const float* beta, const double* L_ref, cons
     DeviceGuard dg(g->device);
     cudaStream_t st = as_stream(stream);
     prof_reset(g);
-    const size_t nP = (size_t)g->n_cams * g->geo.npad;
+    const size_t nL = (size_t)g->n_cams * g->geo.nvox;
     double* lossp = loss ? loss : g->stats + MST_NSTATS;
     // two species: j = L_ref / (beta_ref + beta_air) and L = j (beta + beta_air); the terms of
     // the gradient are derivatives w.r.t. the total, which equal those w.r.t. the aerosol
@@ -932,12 +932,12 @@ int mst_surrogate_grad(mst_grid* g, const float* beta, const double* L_ref, cons
         Phase ph(g, MST_PH_IMAGES, st);
         MST_CK(launch_images(g, g->R, images, meas, mask, g->resid, lossp, st));
     }
-    MST_CK(cudaMemsetAsync(g->bacc, 0, sizeof(float) * nP, st));
+    MST_CK(cudaMemsetAsync(g->bacc, 0, sizeof(float) * nL, st));
     {
         Phase ph(g, MST_PH_BACKPROJECT, st);
         MST_CK(launch_backproject(g, g->resid, g->bacc, st));
     }
-    MST_CK(cudaMemsetAsync(g->gT, 0, sizeof(float) * nP, st));
+    MST_CK(cudaMemsetAsync(g->gT, 0, sizeof(float) * nL, st));
     {
         Phase ph(g, MST_PH_LOS_ADJOINT, st);
         MST_CK(launch_los_adjoint(g, g->R, g->bacc, g->gT, st));
@@ -1421,7 +1421,7 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
     for (int i = 0; i < n; ++i) {
         g = b->grids[i];
         cudaStream_t st = b->branch[i];
-        const size_t nP = (size_t)g->n_cams * g->geo.npad;
+        const size_t nL = (size_t)g->n_cams * g->geo.nvox;
         const uint64_t np = params[i].n_photons;
         double* lossp = losses + i;
         MST_CK(launch_fold_L(g, st));
@@ -1430,9 +1430,9 @@ int persistent_sequence(mst_batch* b, const float* const* betas, const mst_param
         MST_CK(cudaMemsetAsync(lossp, 0, sizeof(double), st));
         MST_CK(launch_images(g, g->R, images ? images[i] : nullptr, meas[i], masks ? masks[i] : nullptr, g->resid,
                              lossp, st));
-        MST_CK(cudaMemsetAsync(g->bacc, 0, sizeof(float) * nP, st));
+        MST_CK(cudaMemsetAsync(g->bacc, 0, sizeof(float) * nL, st));
         MST_CK(launch_backproject(g, g->resid, g->bacc, st));
-        MST_CK(cudaMemsetAsync(g->gT, 0, sizeof(float) * nP, st));
+        MST_CK(cudaMemsetAsync(g->gT, 0, sizeof(float) * nL, st));
         MST_CK(launch_los_adjoint(g, g->R, g->bacc, g->gT, st));
         MST_CK(launch_adjoint_tiles(g, g->T, g->bacc, g->adj, st));
         MST_CK(cudaMemsetAsync(g->g64, 0, sizeof(double) * g->geo.nvox, st));

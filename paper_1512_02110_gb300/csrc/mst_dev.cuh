@@ -182,11 +182,6 @@ __host__ __device__ __forceinline__ int pad_index(const Geo& g, int ix, int iy, 
     return (ix + kHalo) + g.p0 * (iy + kHalo) + g.p01 * (iz + kHalo);
 }
 
-// padded index of linear voxel k
-__device__ __forceinline__ int pad_of(const Geo& g, int k) {
-    return pad_index(g, k % g.nx, (k / g.nx) % g.ny, k / (g.nx * g.ny));
-}
-
 // (ix, iy, iz) of padded index q, each in [-kHalo, n + kHalo). The quotients come from FP32 reciprocals and
 // are corrected by one step: q < 2^31 and the quotients are below 2^12, so the FP32 estimate is
 // off by at most one.
@@ -419,6 +414,21 @@ struct PadWalk {
 __host__ __device__ __forceinline__ PadWalk pad_walk(const Geo& g, float3 p, float3 d, int ix, int iy, int iz) {
     return PadWalk(g, p, d, pad_index(g, ix, iy, iz), g.p0, g.p01);
 }
+
+// Faces left to the grid's boundary on each axis of a ray that starts in voxel (ix, iy, iz) along d: how
+// a walk that reads no field on its way knows that it has left the grid.
+struct FacesLeft {
+    int x, y, z;
+    __device__ __forceinline__ FacesLeft(const Geo& g, float3 d, int ix, int iy, int iz)
+        : x(d.x > 0.f ? g.nx - 1 - ix : ix), y(d.y > 0.f ? g.ny - 1 - iy : iy), z(d.z > 0.f ? g.nz - 1 - iz : iz) {}
+    // after crossing a face of x (px), of y (py) or of z: whether that was the boundary
+    __device__ __forceinline__ bool out(bool px, bool py) {
+        x -= px ? 1 : 0;
+        y -= py ? 1 : 0;
+        z -= px || py ? 0 : 1;
+        return (x | y | z) < 0;
+    }
+};
 
 // Whether a ray on the padded grid ends in a voxel of extinction b and optical depth bs = b * (distance to
 // the next face): every ray in the halo (b = +inf), a flight also where its free path tau runs out. The

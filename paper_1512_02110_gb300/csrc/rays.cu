@@ -90,10 +90,6 @@ __device__ __forceinline__ bool los_dir(const Geo& g, const Cam& c, int ix, int 
     return true;
 }
 
-__device__ __forceinline__ int camera_lin(const Geo& g, const Cam& c) {
-    return c.inside ? pad_index(g, c.ix, c.iy, c.iz) : -1;
-}
-
 // K2: tau_c(k) along the LOS from the centre of voxel k to X_c; T = exp(-tau). With L given,
 // also R_c(k) = L_c(k) T_c(k) (Eq. Rck) on the padded grid, where L = Lsrc * beta / beta_ref when
 // beta_ref is given (the j-fixed surrogate, L = j beta with j = L_ref / beta_ref). The walk ends in
@@ -118,7 +114,7 @@ __global__ void __launch_bounds__(kTB) k_los(const Geo g, const CamSet cs, const
         if (los_dir(g, cm, ix, iy, iz, p, d, rem)) {
             const int goal = !cm.inside ? -1 : (PAD ? pad_index(g, cm.ix, cm.iy, cm.iz) : lin_index(g, cm.ix, cm.iy, cm.iz));
             PadWalk w(g, p, d, PAD ? pad_index(g, ix, iy, iz) : k, PAD ? g.p0 : g.nx, PAD ? g.p01 : g.nx * g.ny);
-            int lx = d.x > 0.f ? g.nx - 1 - ix : ix, ly = d.y > 0.f ? g.ny - 1 - iy : iy, lz = d.z > 0.f ? g.nz - 1 - iz : iz;
+            FacesLeft left(g, d, ix, iy, iz);
             float b, m, bn = BetaFetch<DT>::get(ext, w.lin);
             bool px, py;
             int next;
@@ -130,7 +126,7 @@ __global__ void __launch_bounds__(kTB) k_los(const Geo g, const CamSet cs, const
                 ++nseg;
                 tau.add(__fmul_rn(b, m));
                 rem -= m;
-                if (!PAD && (px ? lx-- : (py ? ly-- : lz--)) == 0) {  // out of the grid
+                if (!PAD && left.out(px, py)) {
                     m = -1.f;
                     break;
                 }
@@ -241,37 +237,38 @@ __global__ void k_images(const Geo g, const CamSet cs, const Halton hs, float in
     if (stats) block_count(stats, MST_ST_PIXEL_SEGMENTS, nseg);
 }
 
-// K4: b_c(k) = sum_p Pi_c(p, k) resid(p)  (Pi^T, Eq. PIc transposed), on the padded grid. A thread
-// takes a pixel and walks its rays in their order. An atomic on an address that another lane of
-// the instruction holds costs another transaction (2.0e11 a second on this chip, however many
-// lanes share it); what bounds the kernel is the queue on each camera's own voxel (1.6e5 additions).
-// 9 cameras of 128^2 pixels in 64^3 voxels: 0.94-0.99 ms. A warp taking every fourth pixel, whose rays
-// part sooner, took 0.85, and adding the lanes' terms up before the atomic 0.27; neither was kept:
-// the bins next to a camera sum so many terms in FP32 that another order moves them by up to 1e-3.
+// K4: b_c(k) = sum_p Pi_c(p, k) resid(p)  (Pi^T, Eq. PIc transposed). A thread takes a pixel and walks
+// its rays in their order, counting the faces left to the boundary (stopping on the halo mark of R
+// instead, a load per voxel, took 1.37 ms for the 36 cameras of 64^2 pixels over 80 x 80 x 120 voxels
+// against 1.30, and 76 us for 3 cameras of 8^2 pixels over 96^3 against 21). An atomic on an address that
+// another lane of the instruction holds costs another transaction (2.0e11 a second on this chip,
+// however many lanes share it); what bounds the kernel is the queue on each camera's own voxel (1.6e5
+// additions). 9 cameras of 128^2 pixels in 64^3 voxels: 0.86-0.95 ms. A warp taking every fourth pixel,
+// whose rays part sooner, took 0.85, and adding the lanes' terms up before the atomic 0.27; neither was
+// kept: the bins next to a camera sum so many terms in FP32 that another order moves them by up to 1e-3.
 constexpr int kRaysApart = 1 << 15;  // pixels below which the rays of a pixel go to threads of their own
 __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet cs, const Halton hs, float inv_nv,
-                                                     const double* __restrict__ resid, const float* __restrict__ R,
-                                                     float* __restrict__ bacc, int total_pix, double* stats) {
+                                                     const double* __restrict__ resid, float* __restrict__ bacc,
+                                                     int total_pix, double* stats) {
     const int gp = blockIdx.x * kTB + (int)threadIdx.x;
     unsigned nseg = 0u;
     const float wgt = gp < total_pix ? (float)(resid[gp] * (double)inv_nv) : 0.f;
     if (wgt != 0.f) {
         const int c = cam_of_pixel(cs, gp);
-        const float* Rc = R + (size_t)c * g.npad;
-        float* bc = bacc + (size_t)c * g.npad;
+        float* bc = bacc + (size_t)c * g.nvox;
         for (int rho = blockIdx.y; rho < hs.n; rho += gridDim.y) {
             float3 p, d;
             int ix, iy, iz;
             if (!pixel_ray_start(g, cs.c[c], hs, gp, rho, p, d, ix, iy, iz)) continue;
-            PadWalk w = pad_walk(g, p, d, ix, iy, iz);
-            float rn = __ldg(Rc + w.lin);
-            for (int n = 0; n <= g.max_steps && __float_as_int(rn) != kOutside; ++n) {
+            PadWalk w(g, p, d, lin_index(g, ix, iy, iz), g.nx, g.nx * g.ny);
+            FacesLeft left(g, d, ix, iy, iz);
+            for (int n = 0; n <= g.max_steps; ++n) {
                 ++nseg;
                 bool px, py;
                 int next;
                 const float m = w.face(px, py, next);
-                rn = __ldg(Rc + next);
                 if (m > 0.f) atomicAdd(bc + w.lin, wgt * m);
+                if (left.out(px, py)) break;
                 w.cross(m, px, py, next);
             }
         }
@@ -279,10 +276,10 @@ __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet c
     if (stats) block_count(stats, MST_ST_BACKPROJ_SEGMENTS, nseg);
 }
 
-// K5: gT_c(m) = sum_k W_c(k, m) s_c(k), s = R b = L T b (Eq. DivTc transposed), on the padded grid.
+// K5: gT_c(m) = sum_k W_c(k, m) s_c(k), s = R b = L T b (Eq. DivTc transposed).
 // Every line of a camera ends in its voxel, where the atomics queue up on one address, so the
 // blocks go round the cameras and the queues run side by side (36 cameras over 80 x 80 x 120
-// voxels: 10.9 ms camera after camera, 4.1 ms in turn).
+// voxels: 12.1 ms camera after camera, 3.5 ms in turn).
 __global__ void __launch_bounds__(kTB) k_los_adjoint(const Geo g, const CamSet cs, const float* __restrict__ R,
                                                      const float* __restrict__ bacc, float* __restrict__ gT,
                                                      double* stats) {
@@ -290,30 +287,31 @@ __global__ void __launch_bounds__(kTB) k_los_adjoint(const Geo g, const CamSet c
     unsigned nseg = 0u;
     if (k < g.nvox) {
         const Cam& cm = cs.c[c];
-        const float* Rc = R + (size_t)c * g.npad;
-        float* gc = gT + (size_t)c * g.npad;
+        float* gc = gT + (size_t)c * g.nvox;
         const int ix = k % g.nx, iy = (k / g.nx) % g.ny, iz = k / (g.nx * g.ny);
-        const int own = pad_index(g, ix, iy, iz);
-        const float s = Rc[own] * bacc[(size_t)c * g.npad + own];
+        const float s = R[(size_t)c * g.npad + pad_index(g, ix, iy, iz)] * bacc[(size_t)c * g.nvox + k];
         float3 p, d;
         float rem;
         if (s != 0.f && los_dir(g, cm, ix, iy, iz, p, d, rem)) {
-            const int goal = camera_lin(g, cm);
-            PadWalk w = pad_walk(g, p, d, ix, iy, iz);
-            float m, r, rn = __ldg(Rc + w.lin);
+            const int goal = cm.inside ? lin_index(g, cm.ix, cm.iy, cm.iz) : -1;
+            PadWalk w(g, p, d, k, g.nx, g.nx * g.ny);
+            FacesLeft left(g, d, ix, iy, iz);
+            float m;
             bool px, py;
             int next;
             for (;;) {
-                r = rn;
                 m = w.face(px, py, next);
-                rn = __ldg(Rc + next);
-                if (__float_as_int(r) == kOutside || w.lin == goal || m >= rem || nseg >= (unsigned)g.max_steps) break;
+                if (w.lin == goal || m >= rem || nseg >= (unsigned)g.max_steps) break;
                 ++nseg;
                 if (m > 0.f) atomicAdd(gc + w.lin, s * m);
                 rem -= m;
+                if (left.out(px, py)) {
+                    m = -1.f;
+                    break;
+                }
                 w.cross(m, px, py, next);
             }
-            if (__float_as_int(r) != kOutside) {  // the last voxel
+            if (m >= 0.f) {  // the last voxel
                 ++nseg;
                 if (w.lin == goal) m = fmaxf(camera_leg(g, cm, w, d, p), 0.f);
                 m = fminf(m, rem);
@@ -351,36 +349,33 @@ __global__ void k_qweights(float* Q, long long n, int mode) {
 }
 
 // a_c(k) = T_c(k) b_c(k) in the [nvox][cp] layout gathered at photon events
-__global__ void k_adjoint_tiles(const Geo g, const float* __restrict__ T, const float* __restrict__ bacc,
-                                float* __restrict__ adj, int C, int cp) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < g.nvox; k += gridDim.x * blockDim.x) {
-        const int q = pad_of(g, k);
+__global__ void k_adjoint_tiles(const float* __restrict__ T, const float* __restrict__ bacc, float* __restrict__ adj,
+                                int nvox, int C, int cp) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nvox; k += gridDim.x * blockDim.x)
         for (int c0 = 0; c0 < cp; c0 += 4) {  // one 16-byte store per four cameras
             float v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int c = c0 + j;
-                v[j] = c < C ? T[(size_t)c * g.nvox + k] * bacc[(size_t)c * g.npad + q] : 0.f;
+                v[j] = c < C ? T[(size_t)c * nvox + k] * bacc[(size_t)c * nvox + k] : 0.f;
             }
             *reinterpret_cast<float4*>(adj + (size_t)k * cp + c0) = make_float4(v[0], v[1], v[2], v[3]);
         }
-    }
 }
 
 // surrogate: grad(m) = sum_c Q_c(m) [ j_c(m) T_c(m) b_c(m) - gT_c(m) ], j = Lsrc / beta_ref
-__global__ void k_combine_surrogate(const Geo g, const double* __restrict__ Lsrc, const float* __restrict__ beta_ref,
+__global__ void k_combine_surrogate(const double* __restrict__ Lsrc, const float* __restrict__ beta_ref,
                                     const float* __restrict__ T, const float* __restrict__ bacc,
                                     const float* __restrict__ gT, const float* __restrict__ Qw,
-                                    double* __restrict__ grad, int C) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < g.nvox; k += gridDim.x * blockDim.x) {
+                                    double* __restrict__ grad, int nvox, int C) {
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nvox; k += gridDim.x * blockDim.x) {
         const float br = beta_ref[k];
-        const int at = pad_of(g, k);
         double acc = 0.0;
         for (int c = 0; c < C; ++c) {
-            const size_t i = (size_t)c * g.nvox + k, ip = (size_t)c * g.npad + at;
+            const size_t i = (size_t)c * nvox + k;
             const double j = br > 0.f ? Lsrc[i] / (double)br : 0.0;
             const double q = Qw ? (double)Qw[i] : 1.0;
-            acc += q * (j * (double)T[i] * (double)bacc[ip] - (double)gT[ip]);
+            acc += q * (j * (double)T[i] * (double)bacc[i] - (double)gT[i]);
         }
         grad[k] = acc;
     }
@@ -413,7 +408,7 @@ __global__ void k_combine_full(const Geo g, const float* __restrict__ gT, const 
             }
         }
         if (gT)  // voxel estimator: the LOS term; the classic estimator has none
-            for (int c = 0; c < C; ++c) acc -= (double)gT[(size_t)c * g.npad + at];
+            for (int c = 0; c < C; ++c) acc -= (double)gT[(size_t)c * g.nvox + k];
         grad[k] = acc;
     }
 }
@@ -533,7 +528,7 @@ cudaError_t launch_backproject(const mst_grid* g, const double* resid, float* ba
     // few pixels leave the chip to single threads' chains of rays: a thread per ray then (5 cameras of
     // 32^2 pixels in 16^3 voxels: 48 us against 36)
     const dim3 nb((g->total_pix + kTB - 1) / kTB, g->total_pix < kRaysApart ? g->n_rays : 1);
-    k_backproject<<<nb, kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, g->R, bacc, g->total_pix, g->stats);
+    k_backproject<<<nb, kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, bacc, g->total_pix, g->stats);
     return cudaGetLastError();
 }
 
@@ -553,15 +548,15 @@ cudaError_t launch_ray_counts(const mst_grid* g, float* Q, int mode, cudaStream_
 }
 
 cudaError_t launch_adjoint_tiles(const mst_grid* g, const float* T, const float* bacc, float* adj, cudaStream_t st) {
-    k_adjoint_tiles<<<nblocks(g->geo.nvox, kTB, 4096), kTB, 0, st>>>(g->geo, T, bacc, adj, g->n_cams, g->cp);
+    k_adjoint_tiles<<<nblocks(g->geo.nvox, kTB, 4096), kTB, 0, st>>>(T, bacc, adj, g->geo.nvox, g->n_cams, g->cp);
     return cudaGetLastError();
 }
 
 cudaError_t launch_combine_surrogate(const mst_grid* g, const double* Lsrc, const double* /*jfix*/,
                                      const float* beta_ref, const float* /*beta*/, const float* T, const float* bacc,
                                      const float* gT, const float* Qw, double* grad, cudaStream_t st) {
-    k_combine_surrogate<<<nblocks(g->geo.nvox, kTB, 4096), kTB, 0, st>>>(g->geo, Lsrc, beta_ref, T, bacc, gT, Qw, grad,
-                                                                         g->n_cams);
+    k_combine_surrogate<<<nblocks(g->geo.nvox, kTB, 4096), kTB, 0, st>>>(Lsrc, beta_ref, T, bacc, gT, Qw, grad,
+                                                                         g->geo.nvox, g->n_cams);
     return cudaGetLastError();
 }
 
