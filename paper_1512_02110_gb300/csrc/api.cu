@@ -335,7 +335,7 @@ void drop_records(mst_grid* g) {
 // their copy has landed), within the budget. Never
 // fails the call: too many photons, no budget, a failed allocation or a call inside a stream
 // capture (no allocation there) all mean W by replay.
-bool ensure_records(mst_grid* g, uint64_t n, int dtype) {
+bool ensure_records(mst_grid* g, uint64_t n, int dtype, cudaStream_t st) {
     const uint64_t rec_bytes = (uint64_t)kEventBytes;
     if (g->capturing || n > kRecordMaxPhotons || g->rec_budget < rec_bytes * 1024) return false;
     if (!g->ev_count) {
@@ -374,6 +374,22 @@ bool ensure_records(mst_grid* g, uint64_t n, int dtype) {
         if (cudaMalloc(&g->warp_tail, sizeof(uint32_t) * (size_t)g->sm_count * kMaxWarpsPerSm) != cudaSuccess) {
             cudaGetLastError();
             g->warp_tail = nullptr;
+            return false;
+        }
+    }
+    if (!g->gbrk) {  // the score kernel's tile: a handle that only renders has none
+        const size_t bytes = (size_t)brick_bins(g->geo) * g->score_tiles * 4;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+            cudaMalloc(&g->gbrk, bytes) != cudaSuccess) {  // (a captured clear would not run now)
+            cudaGetLastError();
+            g->gbrk = nullptr;
+            return false;
+        }
+        if (cudaMemsetAsync(g->gbrk, 0, bytes, st) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(g->gbrk);
+            g->gbrk = nullptr;
             return false;
         }
     }
@@ -430,7 +446,7 @@ double radical_inverse(int base, int i) {
 
 void free_all(mst_grid* g) {
     void* ptrs[] = {g->ext, g->ext_pad, g->Lacc, g->L64, g->T, g->R, g->bacc, g->gT, g->adj, g->gacc, g->g64,
-                    g->resid, g->cimg, g->lap, g->omega, g->Qw, g->stats, g->tickets, g->wbuf, g->nevbuf, g->plist, g->score_cnt};
+                    g->resid, g->cimg, g->lap, g->omega, g->Qw, g->stats, g->wbuf, g->nevbuf, g->plist};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     drop_records(g);
@@ -596,6 +612,8 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     }
 
     const size_t nvox = (size_t)geo.nvox, C = (size_t)n_cams;
+    constexpr size_t kScoreCntAt = 512, kTicketsAt = 2048;
+    static_assert(MST_NSTATS * 8 + 64 <= kScoreCntAt && kScoreCntAt + (2 * kScoreBins + 1) * 4 <= kTicketsAt, "");
     struct A {
         void** p;
         size_t bytes;
@@ -609,15 +627,12 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         {(void**)&g->gT, C * nvox * 4},
         {(void**)&g->adj, nvox * g->cp * 4},
         {(void**)&g->gacc, (size_t)geo.npad * 4},
-        {(void**)&g->gbrk, (size_t)brick_bins(geo) * g->score_tiles * 4},
-        {(void**)&g->score_cnt, (2 * kScoreBins + 1) * 4},
         {(void**)&g->g64, nvox * 8},
         {(void**)&g->resid, (size_t)off * 8},
         {(void**)&g->cimg, (size_t)off * 8},
         {(void**)&g->lap, nvox * 8},
         {(void**)&g->omega, (size_t)off * 4},
-        {(void**)&g->stats, MST_NSTATS * 8 + 64},
-        {(void**)&g->tickets, (size_t)kMaxTickets * 4},
+        {(void**)&g->stats, kTicketsAt + (size_t)kMaxTickets * 4},
     };
     for (auto& a : allocs) {
         if (cudaMalloc(a.p, a.bytes) != cudaSuccess) {
@@ -627,6 +642,9 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
             return MST_ERR_OOM;
         }
     }
+    // statistics, list bins and tickets share an allocation
+    g->score_cnt = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(g->stats) + kScoreCntAt);
+    g->tickets = reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(g->stats) + kTicketsAt);
     // pixel solid angles for the classic estimator (exact rectangle formula, FP64 on the host)
     float* om = new float[off];
     for (int c = 0; c < n_cams; ++c) {
@@ -644,7 +662,6 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
     if (e == cudaSuccess) e = cudaMemset(g->R, 0xFF, C * geo.npad * 4);  // the halo's mark (k_los writes the rest)
     if (e == cudaSuccess) e = cudaMemset(g->Lacc, 0, nvox * g->cp * 4);
     if (e == cudaSuccess) e = cudaMemset(g->gacc, 0, (size_t)geo.npad * 4);
-    if (e == cudaSuccess) e = cudaMemset(g->gbrk, 0, (size_t)brick_bins(geo) * g->score_tiles * 4);
     if (e == cudaSuccess) e = cudaMemset(g->stats, 0, MST_NSTATS * 8 + 64);
     // The handle's first call may run on any stream, also one that does not wait for this one: pixel rays
     // stop at R's halo alone, and a late clear would undo what that call has written.
@@ -798,7 +815,7 @@ int render_grad_impl(mst_grid* g, const float* beta, const mst_params* p, const 
         if (g->capturing) {  // a batch graph: the buffers were sized before the capture
             stored = g->batch_stored;
         } else {
-            stored = ensure_records(g, p->n_photons, p->grid_dtype);
+            stored = ensure_records(g, p->n_photons, p->grid_dtype, st);
             if (stored && ensure_replay(g, p->n_photons) != MST_OK) {
                 stored = false;
                 g->err.clear();
@@ -1674,7 +1691,7 @@ int mst_batch_render_grad(mst_batch* b, const float* const* betas, const mst_par
             key_add(k, g->air);
             key_add(k, g->albedo_air);
             key_add(k, g->reg_wz);
-            const void* bufs[] = {g->wbuf, g->nevbuf, g->plist, g->evrec, g->ch_prev,
+            const void* bufs[] = {g->wbuf, g->nevbuf, g->plist, g->evrec, g->ch_prev, g->gbrk,
                                   g->warp_tail, g->Qw, g->btot, g->btot_ref};
             for (const void* q : bufs) key_add(k, q);
             key_add(k, g->ev_cap);
@@ -1696,7 +1713,7 @@ int mst_batch_render_grad(mst_batch* b, const float* const* betas, const mst_par
             if (g->batch_stored && *g->ev_seen > g->ev_cap) {
                 g->ev_last = *g->ev_seen;
                 g->ev_counted = true;
-                g->batch_stored = ensure_records(g, params[i].n_photons, params[i].grid_dtype);
+                g->batch_stored = ensure_records(g, params[i].n_photons, params[i].grid_dtype, st);
                 g->err.clear();
             }
         }
@@ -1722,7 +1739,7 @@ int mst_batch_render_grad(mst_batch* b, const float* const* betas, const mst_par
             }
             // full gradient: the forward stores its events in buffers sized here (W without pass 1)
             g->batch_stored = params[i].grad_mode == MST_GRAD_FULL &&
-                              ensure_records(g, params[i].n_photons, params[i].grid_dtype) &&
+                              ensure_records(g, params[i].n_photons, params[i].grid_dtype, st) &&
                               ensure_replay(g, params[i].n_photons) == MST_OK;
             g->err.clear();
             for (int mode = 0; mode < 7; ++mode)

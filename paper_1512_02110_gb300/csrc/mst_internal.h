@@ -126,7 +126,7 @@ struct mst_grid {
     float* gT = nullptr;          // [C][nvox]  W_c^T (L T b)
     float* adj = nullptr;         // [nvox][cp] T_c b_c
     float* gacc = nullptr;        // [npad] gradient tile on the padded grid
-    float* gbrk = nullptr;        // [score_tiles][brick_bins] gradient tile in 2 x 2 x 2 bricks
+    float* gbrk = nullptr;        // [score_tiles][brick_bins] gradient tile in 2 x 2 x 2 bricks (first call that stores events)
     uint32_t score_tiles = 1;     // its copies
     double* wbuf = nullptr;       // [replay_cap], allocated by the first full-gradient call
     uint32_t* nevbuf = nullptr;   // [replay_cap]
