@@ -690,7 +690,9 @@ constexpr int kSlots = 64;
 // Voxels a flying lane advances per loop trip, and minimum resident blocks per SM (register
 // budget), per kernel mode; set from sweeps on the 64^3 cumulus workload.
 constexpr int kStepsForward = 8;
-// The classic forward: 6 / 8 / 10 / 12 / 16 voxels ran 8.66 / 8.59 / 9.30 / 9.30 / 8.50 ms (2e6 photons, 9 cameras, 64^3)
+// Classic estimate, forward and replay passes: 6 / 8 / 10 / 12 / 16 voxels a trip ran the forward in
+// 8.66 / 8.59 / 9.30 / 9.30 / 8.50 ms (2e6 photons, 9 cameras, 64^3), pass 2 in 24.4 / 25.0 / - / 24.7 / 23.0 at
+// 5e5, where the longest photon's chain sets the time, and pass 1 in 3.8 whatever the trip.
 constexpr int kStepsClassic = 16;
 constexpr int kStepsPass1 = 8;
 constexpr int kStepsPass2 = 6;
@@ -912,7 +914,7 @@ __device__ __forceinline__ void transport_run(const TransportArgs& A, uint32_t* 
     constexpr bool PASS2 = MODE == kPass2 || MODE == kPass2C;
     constexpr bool CLASSIC = MODE == kFwdClassic || MODE == kPass1C || MODE == kPass2C;
     constexpr bool REPLAY = PASS1 || PASS2;
-    constexpr int kStepsPerTrip = TRIP > 0 ? TRIP : (PASS2 ? kStepsPass2 : (PASS1 ? kStepsPass1 : kStepsClassic));
+    constexpr int kStepsPerTrip = TRIP > 0 ? TRIP : (CLASSIC ? kStepsClassic : (PASS2 ? kStepsPass2 : kStepsPass1));
     constexpr int NW = Rec<MODE>::NW;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned warp = threadIdx.x >> 5;
