@@ -129,6 +129,30 @@ def test_backward_paths_all_end(m, shape, cams, paths):
     assert np.isfinite(out["images"].cpu().numpy()).all()
 
 
+def test_backward_paths_of_both_kernels(m):
+    """A call with few paths walks a path's rays in turn, one with many takes them in trips: the same
+    Philox streams, so the first paths of every pixel are the same whichever kernel runs. 64 x 65 x 66 voxels, 10
+    paths per resident lane and more for five cameras (one kernel), the first camera alone (the other): its means
+    and spreads agree to the rounding of FP64 sums (1e-12)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = -(-10 * sms * 1024 // (5 * 33 * 33)) + 1  # paths a pixel
+    sc = _scene((64, 65, 66), 5, 9, px=(33, 33))
+    p = m.make_params(synth.Params(albedo=0.95, g=0.7, sun_zenith=0.5, sun_azimuth=0.4, seed=21))
+    beta = dev(sc.beta, np.float32)
+    grid = m.Grid.from_scene(sc)
+    a = grid.render_bmc(beta, p, n)
+    st = grid.stats()
+    assert st["lost"] == 0 and st["bmc_paths"] == n * sc.n_pix >= 10 * sms * 1024
+    first = m.Grid(sc.shape, sc.h, sc.origin, sc.cam_pos[:1], sc.cam_rot[:1], sc.cam_w[:1], sc.cam_h[:1], sc.cam_fov[:1],
+                   sc.n_rays)
+    c = first.render_bmc(beta, p, n)
+    st = first.stats()
+    assert st["lost"] == 0 and st["bmc_paths"] == n * 33 * 33 < 10 * sms * 1024
+    for k in ("images", "var"):
+        x, y = a[k][: 33 * 33].cpu().numpy(), c[k].cpu().numpy()
+        assert np.abs(x - y).max() <= 1e-12 * np.abs(x).max(), k
+
+
 def test_a_new_handle_is_ready_for_any_stream(m):
     """Creation leaves no work in flight: the clears of the handle's buffers (here some 0.3 GB, behind work
     that was queued before) are done when it returns, so that a first call on a stream that does not wait
