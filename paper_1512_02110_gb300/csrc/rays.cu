@@ -246,7 +246,12 @@ __global__ void k_images(const Geo g, const CamSet cs, const Halton hs, float in
 // additions). 9 cameras of 128^2 pixels in 64^3 voxels: 0.86-0.95 ms. A warp taking every fourth pixel,
 // whose rays part sooner, took 0.85, and adding the lanes' terms up before the atomic 0.27; neither was
 // kept: the bins next to a camera sum so many terms in FP32 that another order moves them by up to 1e-3.
-constexpr int kRaysApart = 1 << 15;  // pixels below which the rays of a pixel go to threads of their own
+// Below this many pixels a camera, the rays of a pixel go to threads of their own: few pixels leave the
+// chip to single threads' chains of rays, many of them queue longer on the camera's voxel when all their
+// rays come at once. us apart / in one thread by pixels a camera: 1024: 41 / 137 (1 camera, 64^3), 37 / 39 (5,
+// 16^3), 101 / 105 (36, 32^3); 2025: 64 / 135, 56 / 60, 121 / 152; 4096: 127 / 160, 146 / 109, 429 / 441, 244 / 236
+// (9 cameras, 64^3), 211 / 254 (3, 96^3); 8100: 248 / 217 (1, 64^3), 390 / 316 (3, 96^3).
+constexpr int kRaysApart = 3072;
 __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet cs, const Halton hs, float inv_nv,
                                                      const double* __restrict__ resid, float* __restrict__ bacc,
                                                      int total_pix, double* stats) {
@@ -525,9 +530,7 @@ cudaError_t launch_images(const mst_grid* g, const float* R, double* images, con
 
 cudaError_t launch_backproject(const mst_grid* g, const double* resid, float* bacc, cudaStream_t st) {
     const float inv_nv = (float)(1.0 / (g->n_rays * g->voxel_volume));
-    // few pixels leave the chip to single threads' chains of rays: a thread per ray then (5 cameras of
-    // 32^2 pixels in 16^3 voxels: 48 us against 36)
-    const dim3 nb((g->total_pix + kTB - 1) / kTB, g->total_pix < kRaysApart ? g->n_rays : 1);
+    const dim3 nb((g->total_pix + kTB - 1) / kTB, g->total_pix / g->n_cams < kRaysApart ? g->n_rays : 1);
     k_backproject<<<nb, kTB, 0, st>>>(g->geo, g->cams, g->halton, inv_nv, resid, bacc, g->total_pix, g->stats);
     return cudaGetLastError();
 }
