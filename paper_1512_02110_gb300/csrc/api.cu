@@ -1550,9 +1550,9 @@ int mst_batch_set_wavefront(mst_batch* b, int forward_trip, int forward_blocks, 
         b->err = "forward trip in {0, 8, 10, 12, 16}, pass-2 trip in {0, 4, 6, 8, 10}, blocks per SM in 0..8";
         return MST_ERR_INVALID_ARG;
     }
-    b->trip_fwd = forward_trip == 8 ? 0 : forward_trip;  // 8 and 6 are the kernels' defaults
+    b->trip_fwd = forward_trip == kForwardTrip ? 0 : forward_trip;  // 0: the kernels' defaults
     b->blocks_fwd = forward_blocks;
-    b->trip_p2 = replay_trip == 6 ? 0 : replay_trip;
+    b->trip_p2 = replay_trip == kScoreTrip ? 0 : replay_trip;
     b->blocks_p2 = replay_blocks;
     return MST_OK;
 }
@@ -1604,9 +1604,9 @@ int mst_batch_autotune(mst_batch* b, const float* const* betas, const mst_params
         return MST_OK;
     };
     // one axis at a time: the forward's trip and blocks, then pass 2's
-    int best[4] = {12, 0, 6, 0};
+    int best[4] = {kForwardTrip, 0, kScoreTrip, 0};
     double ms = 0.0;
-    if (rc == MST_OK) rc = mst_batch_set_wavefront(b, 12, 0, 6, 0);
+    if (rc == MST_OK) rc = mst_batch_set_wavefront(b, kForwardTrip, 0, kScoreTrip, 0);
     if (rc == MST_OK) rc = timed(ms);  // warm-up: buffers sized, graph captured
     const int occ_f = transport_batch_blocks_per_sm(0);
     const int occ_r = transport_batch_blocks_per_sm(4);

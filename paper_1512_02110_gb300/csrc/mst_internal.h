@@ -31,6 +31,9 @@ constexpr unsigned kEventChunk = 256;  // record slots a warp of the forward res
 // which both kernels need: the forward ran 37.1 ms with 24 warps at 80 registers, 34.7 with 28,
 // 35.4 with 32 at 64 registers and their spills (64^3, 1e8 photons).
 constexpr int kTransportWarps = 7;
+// Voxels a lane of the forward walks, and entries a lane of the score kernel adds, per loop trip unless
+// mst_set_wavefront or an autotuner says otherwise
+constexpr int kForwardTrip = 8, kScoreTrip = 6;
 constexpr uint32_t kEndChunk = 0xFFFFFFFFu;  // end of a warp's chunk list
 constexpr int kMaxWarpsPerSm = 64;     // warp_tail entries per SM (the forward runs 24)
 constexpr uint64_t kDefaultRecordBytes = 32ull << 30;

@@ -688,15 +688,14 @@ constexpr uint32_t kNoPhoton = 0xFFFFFFFFu;  // photon word of a chunk's unused 
 constexpr uint32_t kNoEvent = 0xFFFFFFFFu;   // previous record of a photon's first event
 constexpr int kSlots = 64;
 // Voxels a flying lane advances per loop trip, and minimum resident blocks per SM (register
-// budget), per kernel mode; set from sweeps on the 64^3 cumulus workload.
-constexpr int kStepsForward = 8;
+// budget), per kernel mode (the forward's and the score's trips: kForwardTrip, kScoreTrip); set from
+// sweeps on the 64^3 cumulus workload.
 // Classic estimate, forward and replay passes: 6 / 8 / 10 / 12 / 16 voxels a trip ran the forward in
 // 8.66 / 8.59 / 9.30 / 9.30 / 8.50 ms (2e6 photons, 9 cameras, 64^3), pass 2 in 24.4 / 25.0 / - / 24.7 / 23.0 at
 // 5e5, where the longest photon's chain sets the time, and pass 1 in 3.8 whatever the trip.
 constexpr int kStepsClassic = 16;
 constexpr int kStepsPass1 = 8;
 constexpr int kStepsPass2 = 6;
-constexpr int kStepsScore = 6;  // list entries a score lane adds per loop trip
 // A draining warp of the forward takes its queued events once they are no fewer than the flights
 // still under way.
 constexpr int kDrain = 1;
@@ -2028,7 +2027,7 @@ cudaError_t launch_trip(const TransportArgs& a, int trip, int blocks, cudaStream
 
 template <int DT, bool TWO, int TRIP>
 cudaError_t launch_forward_t(const TransportArgs& a, int blocks, cudaStream_t st) {
-    if constexpr (TRIP != kStepsForward) {  // the default's attributes are set by occupancy()
+    if constexpr (TRIP != kForwardTrip) {  // the default's attributes are set by occupancy()
         static const int once = occupancy(k_forward<DT, TWO, TRIP>, forward_smem(), kMinBlocksForward, kFT);
         (void)once;
     }
@@ -2048,16 +2047,16 @@ cudaError_t launch_forward(const TransportArgs& a, int trip, int blocks, cudaStr
             default: break;
         }
     }
-    return launch_forward_t<DT, TWO, kStepsForward>(a, blocks, st);
+    return launch_forward_t<DT, TWO, kForwardTrip>(a, blocks, st);
 }
 
 template <int DT, bool TWO>
 int occupancy_mode(int mode) {
     switch (mode) {
-        case kFwdVoxel: return occupancy(k_forward<DT, TWO, kStepsForward>, forward_smem(), kMinBlocksForward, kFT);
+        case kFwdVoxel: return occupancy(k_forward<DT, TWO, kForwardTrip>, forward_smem(), kMinBlocksForward, kFT);
         case kFwdClassic: return occupancy(k_transport<DT, kFwdClassic, TWO>, smem_bytes<kFwdClassic>());
         case kPass2: return occupancy(k_transport<DT, kPass2, TWO>, smem_bytes<kPass2>());
-        case kScore: return occupancy(k_score<DT, TWO, kStepsScore>, score_smem<kStepsScore>(), kMinBlocksScore, kFT);
+        case kScore: return occupancy(k_score<DT, TWO, kScoreTrip>, score_smem<kScoreTrip>(), kMinBlocksScore, kFT);
         case kPass1C: return occupancy(k_transport<DT, kPass1C, TWO>, smem_bytes<kPass1C>());
         case kPass2C: return occupancy(k_transport<DT, kPass2C, TWO>, smem_bytes<kPass2C>());
         default: return occupancy(k_transport<DT, kPass1, TWO>, smem_bytes<kPass1>());
@@ -2110,7 +2109,7 @@ cudaError_t launch_transport_batch(const TransportArgs* table, int n, int mode, 
                 case 12: k_forward_batch<12><<<blocks, kFT, forward_smem(), st>>>(table, n); break;
                 case 10: k_forward_batch<10><<<blocks, kFT, forward_smem(), st>>>(table, n); break;
                 case 16: k_forward_batch<16><<<blocks, kFT, forward_smem(), st>>>(table, n); break;
-                default: k_forward_batch<kStepsForward><<<blocks, kFT, forward_smem(), st>>>(table, n);
+                default: k_forward_batch<kForwardTrip><<<blocks, kFT, forward_smem(), st>>>(table, n);
             }
             return cudaGetLastError();
         case kPass2: return launch_batch_mode<kPass2>(table, n, blocks, st);
@@ -2123,11 +2122,11 @@ int transport_batch_blocks_per_sm(int mode) {
     static int occ[7] = {0, 0, 0, 0, 0, 0, 0};
     static bool ready = false;
     if (!ready) {  // every instantiation's attributes, once; the default trips give the occupancy
-        occ[kFwdVoxel] = occupancy(k_forward_batch<kStepsForward>, forward_smem(), kMinBlocksForward, kFT);
+        occ[kFwdVoxel] = occupancy(k_forward_batch<kForwardTrip>, forward_smem(), kMinBlocksForward, kFT);
         occupancy(k_forward_batch<12>, forward_smem(), kMinBlocksForward, kFT);
         occupancy(k_forward_batch<10>, forward_smem(), kMinBlocksForward, kFT);
         occupancy(k_forward_batch<16>, forward_smem(), kMinBlocksForward, kFT);
-        occ[kScore] = occupancy(k_score_batch<kStepsScore>, score_smem<kStepsScore>(), kMinBlocksScore, kFT);
+        occ[kScore] = occupancy(k_score_batch<kScoreTrip>, score_smem<kScoreTrip>(), kMinBlocksScore, kFT);
         occupancy(k_score_batch<4>, score_smem<4>(), kMinBlocksScore, kFT);
         occupancy(k_score_batch<8>, score_smem<8>(), kMinBlocksScore, kFT);
         occupancy(k_score_batch<10>, score_smem<10>(), kMinBlocksScore, kFT);
@@ -2143,7 +2142,7 @@ cudaError_t launch_score_batch(const TransportArgs* table, int n, int trip, int 
         case 4: k_score_batch<4><<<blocks, kFT, score_smem<4>(), st>>>(table, n); break;
         case 8: k_score_batch<8><<<blocks, kFT, score_smem<8>(), st>>>(table, n); break;
         case 10: k_score_batch<10><<<blocks, kFT, score_smem<10>(), st>>>(table, n); break;
-        default: k_score_batch<kStepsScore><<<blocks, kFT, score_smem<kStepsScore>(), st>>>(table, n);
+        default: k_score_batch<kScoreTrip><<<blocks, kFT, score_smem<kScoreTrip>(), st>>>(table, n);
     }
     return cudaGetLastError();
 }
@@ -2184,7 +2183,7 @@ namespace {
 
 template <int DT, bool TWO, int K>
 cudaError_t launch_score_k(const TransportArgs& a, int blocks, cudaStream_t st) {
-    if constexpr (K != kStepsScore) {  // the default's attributes are set by occupancy()
+    if constexpr (K != kScoreTrip) {  // the default's attributes are set by occupancy()
         static const int once = occupancy(k_score<DT, TWO, K>, score_smem<K>(), kMinBlocksScore, kFT);
         (void)once;
     }
@@ -2194,13 +2193,13 @@ cudaError_t launch_score_k(const TransportArgs& a, int blocks, cudaStream_t st) 
 
 template <bool TWO>
 cudaError_t launch_score_dt(const TransportArgs& a, int dtype, int trip, int blocks, cudaStream_t st) {
-    if (dtype == 1) return launch_score_k<1, TWO, kStepsScore>(a, blocks, st);
-    if (dtype == 2) return launch_score_k<2, TWO, kStepsScore>(a, blocks, st);
+    if (dtype == 1) return launch_score_k<1, TWO, kScoreTrip>(a, blocks, st);
+    if (dtype == 2) return launch_score_k<2, TWO, kScoreTrip>(a, blocks, st);
     switch (trip) {
         case 4: return launch_score_k<0, TWO, 4>(a, blocks, st);
         case 8: return launch_score_k<0, TWO, 8>(a, blocks, st);
         case 10: return launch_score_k<0, TWO, 10>(a, blocks, st);
-        default: return launch_score_k<0, TWO, kStepsScore>(a, blocks, st);
+        default: return launch_score_k<0, TWO, kScoreTrip>(a, blocks, st);
     }
 }
 
