@@ -250,98 +250,7 @@ struct BetaFetch<2> {
     static __device__ __forceinline__ T make(float v) { return __float2bfloat16_rn(v); }
 };
 
-// ------------------------------------------------------------------------------------------
-// Voxel walk in voxel-local form. A point is (voxel index, offset inside the voxel); the walk
-// keeps, per axis, the distance along the ray from the current point to the next face. A step
-// of length s across axis a subtracts s from the other two axes and resets axis a to h_a/|d_a|,
-// so every quantity stays of the size of one voxel and FP32 keeps ~1e-6 m resolution however
-// large the grid. Ties go to x, then y, then z.
-
-struct Walk {
-    float tx, ty, tz;     // distance to the next face per axis (INF when parallel)
-    float qx, qy, qz;     // h / |d| per axis
-    float ax, ay, az;     // |d| per axis
-    float p0x, p0y, p0z;  // offset at the start (kept on axes the ray does not move along)
-    int ix, iy, iz;       // current voxel
-    int sx, sy, sz;       // step per axis (0 when the direction component is 0)
-    int lin;              // linear index ix + nx (iy + ny iz) of the current voxel (its extinction's address)
-    int left;             // face crossings left before the walk is abandoned
-};
-
-// kFastRcp: 1/|d| by the hardware reciprocal (__fdividef, within 2 ulp) instead of the
-// correctly rounded division; photon flights use it, camera and LOS rays keep the division.
-template <bool kFastRcp>
-__device__ __forceinline__ void axis_init(float p, float d, float h, float& t, float& q, float& a, int& s) {
-    if (d > 0.f) {
-        a = d;
-        const float inv = kFastRcp ? __fdividef(1.f, d) : 1.f / d;
-        t = (h - p) * inv;
-        q = h * inv;
-        s = 1;
-    } else if (d < 0.f) {
-        a = -d;
-        const float inv = kFastRcp ? __fdividef(1.f, a) : 1.f / a;
-        t = p * inv;
-        q = h * inv;
-        s = -1;
-    } else {
-        a = 0.f;
-        t = CUDART_INF_F;
-        q = CUDART_INF_F;
-        s = 0;
-    }
-}
-
-// p: offset of the start point inside voxel (ix, iy, iz), each in [0, h]
-template <bool kFastRcp = false>
-__device__ __forceinline__ void walk_init(Walk& w, const Geo& g, float3 p, float3 d, int ix, int iy, int iz) {
-    axis_init<kFastRcp>(fminf(fmaxf(p.x, 0.f), g.hx), d.x, g.hx, w.tx, w.qx, w.ax, w.sx);
-    axis_init<kFastRcp>(fminf(fmaxf(p.y, 0.f), g.hy), d.y, g.hy, w.ty, w.qy, w.ay, w.sy);
-    axis_init<kFastRcp>(fminf(fmaxf(p.z, 0.f), g.hz), d.z, g.hz, w.tz, w.qz, w.az, w.sz);
-    w.p0x = p.x; w.p0y = p.y; w.p0z = p.z;
-    w.ix = ix; w.iy = iy; w.iz = iz;
-    w.lin = lin_index(g, ix, iy, iz);
-    w.left = g.max_steps;
-}
-
-// distance to the next face and its axis
-__device__ __forceinline__ int walk_axis(const Walk& w, float& tn) {
-    int a = 0;
-    tn = w.tx;
-    if (w.ty < tn) { a = 1; tn = w.ty; }
-    if (w.tz < tn) { a = 2; tn = w.tz; }
-    tn = fmaxf(tn, 0.f);
-    return a;
-}
-
-constexpr int kWalkOverflow = 6;
-
-// Moves seg along the ray and crosses the face on axis a. Returns the exit face (0..5: x-, x+,
-// y-, y+, z-, z+) if the walk left the grid, kWalkOverflow if it made more crossings than any
-// straight line through the grid can (only possible with a non-finite direction), else -1.
-// Branch-free in the axis, so lanes that cross different faces do not diverge. Callers that
-// bound the crossings themselves (the transport, once per trip) pass kGuard = false.
-template <bool kGuard = true>
-__device__ __forceinline__ int walk_step(Walk& w, const Geo& g, int a, float seg) {
-    const bool bx = a == 0, by = a == 1, bz = a == 2;
-    w.tx = bx ? w.qx : w.tx - seg;
-    w.ty = by ? w.qy : w.ty - seg;
-    w.tz = bz ? w.qz : w.tz - seg;
-    const int s = bx ? w.sx : (by ? w.sy : w.sz);
-    w.ix += bx ? s : 0;
-    w.iy += by ? s : 0;
-    w.iz += bz ? s : 0;
-    w.lin += s * (bx ? 1 : (by ? g.nx : g.nx * g.ny));
-    const bool out = ((unsigned)w.ix >= (unsigned)g.nx) | ((unsigned)w.iy >= (unsigned)g.ny) |
-                     ((unsigned)w.iz >= (unsigned)g.nz);
-    if (kGuard && --w.left < 0) return kWalkOverflow;
-    return out ? 2 * a + (s > 0) : -1;
-}
-
-__device__ __forceinline__ float axis_local(float t, float a, int s, float h, float p0, float l) {
-    const float v = s > 0 ? h - (t - l) * a : (s < 0 ? (t - l) * a : p0);
-    return fminf(fmaxf(v, 0.f), h);
-}
+constexpr int kWalkOverflow = 6;  // "exit face" of a walk that was abandoned
 
 // A sum of FP32 terms held as an unevaluated pair hi + lo: each addition's rounding error is
 // recovered exactly (Knuth's TwoSum, six additions) and summed beside it, so n terms keep about
@@ -360,11 +269,14 @@ struct PairSum {
     __device__ __forceinline__ double value() const { return isfinite(lo) ? (double)hi + (double)lo : (double)hi; }
 };
 
-// A camera ray or line of sight on the padded grid (its halo tells the walk that it has left): per
-// axis the distance to the next face (t), between faces (q) and the padded index's change at a
-// crossing, and the current padded index. The distances are those of axis_init with the rounded
-// division, and a step moves them as walk_step does; the voxel indices, the three bounds tests and
-// the exit face of that walk are gone.
+// ------------------------------------------------------------------------------------------
+// Voxel walk of camera rays and lines of sight, in voxel-local form. A point is (voxel, offset inside
+// the voxel); the walk keeps, per axis, the distance along the ray from the current point to the next
+// face (t), the distance between faces (q = h / |d|) and the change of the voxel's index at a crossing. A
+// step of length s subtracts s from two axes and resets the crossed one to q, so every quantity
+// stays of the size of one voxel and FP32 keeps ~1e-6 m resolution however large the grid. Ties go to x,
+// then y, then z. The index runs over the padded grid, whose halo tells the walk that it has left, or
+// over the linear one beside a FacesLeft.
 struct PadWalk {
     float tx, ty, tz, qx, qy, qz;
     int dx, dy, dz, lin;
@@ -438,16 +350,6 @@ __host__ __device__ __forceinline__ bool ray_ends(bool flight, float tau, float 
     return isinf(b) || (flight && tau <= bs);
 }
 
-// offset inside the current voxel of the point a distance l past the current point
-__device__ __forceinline__ float3 walk_local(const Walk& w, const Geo& g, float l) {
-    return make_float3(axis_local(w.tx, w.ax, w.sx, g.hx, w.p0x, l), axis_local(w.ty, w.ay, w.sy, g.hy, w.p0y, l),
-                       axis_local(w.tz, w.az, w.sz, g.hz, w.p0z, l));
-}
-
-__device__ __forceinline__ bool walk_at(const Walk& w, int ix, int iy, int iz) {
-    return w.ix == ix && w.iy == iy && w.iz == iz;
-}
-
 // vector from the point (voxel i, offset p) to the point (voxel j, offset q)
 __device__ __forceinline__ float3 local_delta(const Geo& g, int ix, int iy, int iz, float3 p, int jx, int jy, int jz,
                                               float3 q) {
@@ -516,60 +418,6 @@ __device__ __forceinline__ int cam_of_pixel(const CamSet& cs, int gp) {
     for (int i = 1; i < cs.n; ++i)
         if (gp >= cs.c[i].pix_off) c = i;
     return c;
-}
-
-// Walks the segment from the point (voxel i, offset p) to the centre of projection of camera c,
-// calling fn(walk, length) for every voxel it crosses (walk.lin names the voxel). The walk ends in the
-// camera's voxel (last length = distance to the camera inside it) or, for a camera outside the
-// grid, at the grid face; the remaining distance guards both ends against rounding.
-template <typename F>
-__device__ __forceinline__ void walk_to_camera(const Geo& g, const Cam& c, int ix, int iy, int iz, float3 p, F&& fn,
-                                               unsigned long long& nseg) {
-    const float3 lc = make_float3(c.lx, c.ly, c.lz);
-    const float3 v = local_delta(g, ix, iy, iz, p, c.ix, c.iy, c.iz, lc);
-    const float dist = sqrtf(v.x * v.x + v.y * v.y + v.z * v.z);
-    if (!(dist > 0.f)) return;
-    const float inv = 1.f / dist;
-    const float3 d = make_float3(v.x * inv, v.y * inv, v.z * inv);
-    Walk w;
-    walk_init(w, g, p, d, ix, iy, iz);
-    float rem = dist;
-    for (;;) {
-        ++nseg;
-        if (walk_at(w, c.ix, c.iy, c.iz)) {
-            const float3 q = walk_local(w, g, 0.f);
-            const float len = (lc.x - q.x) * d.x + (lc.y - q.y) * d.y + (lc.z - q.z) * d.z;
-            fn(w, fminf(fmaxf(len, 0.f), rem));
-            return;
-        }
-        float seg;
-        const int a = walk_axis(w, seg);
-        if (seg >= rem) {
-            fn(w, rem);
-            return;
-        }
-        fn(w, seg);
-        rem -= seg;
-        if (walk_step(w, g, a, seg) >= 0) return;
-    }
-}
-
-// Walks the pixel ray from camera c along d to the grid exit, calling fn(walk, length).
-template <typename F>
-__device__ __forceinline__ void walk_from_camera(const Geo& g, const Cam& c, float3 d, F&& fn,
-                                                 unsigned long long& nseg) {
-    float3 p;
-    int ix, iy, iz;
-    if (!ray_start(g, c, d, p, ix, iy, iz)) return;
-    Walk w;
-    walk_init(w, g, p, d, ix, iy, iz);
-    for (;;) {
-        ++nseg;
-        float seg;
-        const int a = walk_axis(w, seg);
-        fn(w, seg);
-        if (walk_step(w, g, a, seg) >= 0) return;
-    }
 }
 
 __device__ __forceinline__ double warp_sum(double v) {

@@ -335,15 +335,21 @@ __global__ void __launch_bounds__(kTB) k_ray_counts(const Geo g, const CamSet cs
     const int gp = blockIdx.x * blockDim.x + threadIdx.x;
     if (gp >= total_pix) return;
     const int c = cam_of_pixel(cs, gp);
-    const Cam& cm = cs.c[c];
-    const int p = gp - cm.pix_off, i = p % cm.w, j = p / cm.w;
     float* qc = Q + (size_t)c * g.nvox;
-    unsigned long long nseg = 0;
     for (int rho = 0; rho < hs.n; ++rho) {
-        const float3 d = pixel_dir(cm, (float)i + hs.a[rho], (float)j + hs.b[rho]);
-        walk_from_camera(g, cm, d, [&](const Walk& w, float len) {
-            if (len >= eps) atomicAdd(qc + w.lin, 1.f);
-        }, nseg);
+        float3 p, d;
+        int ix, iy, iz;
+        if (!pixel_ray_start(g, cs.c[c], hs, gp, rho, p, d, ix, iy, iz)) continue;
+        PadWalk w(g, p, d, lin_index(g, ix, iy, iz), g.nx, g.nx * g.ny);
+        FacesLeft left(g, d, ix, iy, iz);
+        for (int n = 0; n <= g.max_steps; ++n) {
+            bool px, py;
+            int next;
+            const float m = w.face(px, py, next);
+            if (m >= eps) atomicAdd(qc + w.lin, 1.f);
+            if (left.out(px, py)) break;
+            w.cross(m, px, py, next);
+        }
     }
 }
 

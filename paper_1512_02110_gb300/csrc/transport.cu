@@ -696,9 +696,6 @@ constexpr int kSlots = 64;
 constexpr int kStepsClassic = 16;
 constexpr int kStepsPass1 = 8;
 constexpr int kStepsPass2 = 6;
-// A draining warp of the forward takes its queued events once they are no fewer than the flights
-// still under way.
-constexpr int kDrain = 1;
 // The forward launches photons when this many slots are free: 1 / 8 / 16 / 24 / 32 ran 37.0 / 36.9 /
 // 37.1 / 39.2 / 42.8 ms at 1e8 photons (64^3): waiting for more leaves lanes idle.
 constexpr int kLaunchFrom = 8;
@@ -1444,8 +1441,9 @@ __device__ __forceinline__ void forward_run(const TransportArgs& A, uint32_t* sm
         __syncwarp();
 
         const int fly_n = __popc(fly);
-        // (4) events, 32 at a time; while the warp drains, whatever is queued once no photon is ready
-        while (ev_n >= 32 || (ev_n > 0 && dry && rd_n == 0 && fly_n <= kDrain * ev_n)) {
+        // (4) events, 32 at a time; while the warp drains, whatever is queued once no photon is ready and the
+        // events are no fewer than the flights still under way
+        while (ev_n >= 32 || (ev_n > 0 && dry && rd_n == 0 && fly_n <= ev_n)) {
             const int n = min(32, ev_n);
             unsigned long long ev_slot = 0ull;  // storing events: this lane's record slot
             if (A.ev_cap) {
