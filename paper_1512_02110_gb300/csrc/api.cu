@@ -174,8 +174,9 @@ void set_fold(TransportArgs& a, uint64_t bins) {
     a.fold_nslices = (uint32_t)((bins + slice - 1) / slice);
 }
 
-// The score kernel folds one slice of its brick tile per chunk of stored events. A photon makes
-// a few events at most on average; counting one per photon keeps a sweep within kFoldSweep photons.
+// The score kernel folds one slice of its brick tile per chunk of stored events, so a sweep takes
+// kFoldSweep events, each with one flight. (The replay's sweep takes kFoldSweep listed photons, of one
+// flight and more each: in no medium does a bin sum more flights here than there.)
 void set_score_fold(TransportArgs& a) {
     const uint64_t bins = (uint64_t)brick_bins(a.g) * a.score_tiles, chunks = kFoldSweep / kEventChunk;
     const uint64_t slice = std::max<uint64_t>(32, ((bins + chunks - 1) / chunks + 31) / 32 * 32);

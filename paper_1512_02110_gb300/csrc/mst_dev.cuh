@@ -254,9 +254,13 @@ constexpr int kWalkOverflow = 6;  // "exit face" of a walk that was abandoned
 
 // A sum of FP32 terms held as an unevaluated pair hi + lo: each addition's rounding error is
 // recovered exactly (Knuth's TwoSum, six additions) and summed beside it, so n terms keep about
-// 48 - log2(n) bits. This chip's FP64 pipe takes 2.6e11 conversions with their additions a second
-// against 3.2e13 FP32 operations, and the ray kernels add one term per voxel segment: k_los took
-// 0.93 ms for 1.8e8 segments with FP64 sums, 0.32 ms with this and the walk below.
+// 48 - log2(n) bits of the 53 that an FP64 sum keeps. The terms are products rounded to 24 bits, and
+// that rounding is what the results show: their distance from a 64-bit evaluation is the same to four
+// digits and more with either sum (T 7.07e-7, images 1.70e-7 and 2.97e-7, at 64^3 and 95 x 77 x 61 voxels; haze T
+// 3.44e-8, images 6.37e-8), T is the same FP32 number, and images differ by 1e-15 to 3e-14 of a pixel.
+// This chip's FP64 pipe takes 2.6e11 conversions with their additions a second against 3.2e13 FP32
+// operations, and the ray kernels add one term per voxel segment: k_los took 0.93 ms for 1.8e8
+// segments with FP64 sums, 0.32 ms with this and the walk below.
 struct PairSum {
     float hi = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(float x) {

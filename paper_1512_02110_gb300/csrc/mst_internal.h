@@ -14,14 +14,15 @@ namespace mst {
 
 // The transport accumulates into FP32 tiles. While a launch runs, every new ticket batch of a
 // warp also folds one slice of the tile into the FP64 result (swap to zero, add in FP64), the
-// slices sized so that a sweep over the whole tile takes at most about kFoldSweep photons:
-// no FP32 bin sums more than a sweep's contributions, however many photons a launch traces.
+// slices sized so that a sweep over the whole tile takes at most about kFoldSweep photons (the score
+// kernel: a slice per chunk of records, kFoldSweep stored events a sweep): no FP32 bin sums more than a
+// sweep's contributions, however many photons a launch traces.
 constexpr uint64_t kMaxPhotons = 1ull << 34;    // photons per call
 constexpr uint64_t kLaunchPhotons = 1ull << 30;  // photons per forward launch (32-bit ticket)
 constexpr uint64_t kReplayChunk = 1ull << 24;    // photons per replay pass-1 / pass-2 pair
-// Full gradient: the forward stores its events (kEventWords words each, structure of arrays)
-// for calls of at most kRecordMaxPhotons photons; W then comes from the stored events and the
-// replay is one pass-2 launch over the call's photons.
+// Full gradient: the forward stores its events (kEventBytes each, three 16-byte words in arrays of
+// their own) for calls of at most kRecordMaxPhotons photons, and the score kernel computes the gradient from
+// them alone; replay passes 1 and 2 run only when the events are not held.
 constexpr uint64_t kRecordMaxPhotons = 1ull << 27;
 // packed voxel, offset (3) | incoming direction (3), albedo * weight | photon, event number, the free
 // path left when the flight entered the event's voxel, the photon's previous record
@@ -35,7 +36,7 @@ constexpr int kTransportWarps = 7;
 // mst_set_wavefront or an autotuner says otherwise
 constexpr int kForwardTrip = 8, kScoreTrip = 6;
 constexpr uint32_t kEndChunk = 0xFFFFFFFFu;  // end of a warp's chunk list
-constexpr int kMaxWarpsPerSm = 64;     // warp_tail entries per SM (the forward runs 24)
+constexpr int kMaxWarpsPerSm = 64;     // warp_tail entries per SM (the forward runs 28)
 constexpr uint64_t kDefaultRecordBytes = 32ull << 30;
 constexpr uint64_t kFoldSweep = 1ull << 21;
 constexpr int kTicketBatch = 64;  // photon ids a warp takes from the global ticket at a time

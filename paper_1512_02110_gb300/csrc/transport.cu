@@ -134,7 +134,7 @@ __device__ __forceinline__ void launch_photon(const TransportArgs& A, Photon& ph
 
 // A free flight (steps ii-iii) on the padded grid. Per axis: the distance along the ray from
 // the current point to the next face (t), the distance between faces (q = h / |d|), and the change
-// of the padded index when a face is crossed (+-1, +-(nx + 2), +-(nx + 2)(ny + 2); 0 for an axis
+// of the padded index when a face is crossed (+-1, +-(nx + 4), +-(nx + 4)(ny + 4); 0 for an axis
 // the ray does not move along, whose t stays +inf); `lin` is the current voxel's padded index.
 // A voxel step subtracts the step from two axes and resets the crossed one to q, so every
 // quantity stays of the size of one voxel and FP32 keeps ~1e-6 m resolution anywhere in the grid.
