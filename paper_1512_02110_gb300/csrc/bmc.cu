@@ -188,8 +188,8 @@ __global__ void __launch_bounds__(kTB, kBmcBlocks) k_bmc(const BmcArgs A) {
             unpad(A.g, w.lin, jx, jy, jz);
             const bool in = inside(A.g, jx, jy, jz);
             if (ray == kFlight) {
-                done = !in;
-                if (in) {  // a collision: the sun's local estimate
+                done = !in || isnan(b);  // (no path collides in a voxel without an extinction)
+                if (!done) {  // a collision: the sun's local estimate
                     ++nseg;
                     ++events;
                     path_collide(A, s, w, s.tau / b, jx, jy, jz);
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kTB, kBmcBlocks) k_bmc_small(const BmcArgs A) 
             unpad(A.g, w.lin, jx, jy, jz);
             return true;
         };
-        while (walk(false) && inside(A.g, jx, jy, jz)) {
+        while (walk(false) && inside(A.g, jx, jy, jz) && !isnan(b)) {
             ++nseg;
             ++events;
             path_collide(A, s, w, s.tau / b, jx, jy, jz);

@@ -347,11 +347,12 @@ struct FacesLeft {
 };
 
 // Whether a ray on the padded grid ends in a voxel of extinction b and optical depth bs = b * (distance to
-// the next face): every ray in the halo (b = +inf), a flight also where its free path tau runs out. The
-// halo is told by b alone: a ray that leaves the grid exactly on a voxel's edge crosses its first
-// halo voxel over no distance, where bs is inf * 0 = NaN and no comparison with it ends the walk.
+// the next face): a flight where its free path tau is not above bs, another ray in the halo (b = +inf). A
+// ray that leaves the grid exactly on a voxel's edge crosses its first halo voxel over no distance, where bs
+// is inf * 0 = NaN: not above is true there, at most would be false, and the walk would go on past the
+// array. (Testing the halo for both kinds costs the backward paths 3 %.)
 __host__ __device__ __forceinline__ bool ray_ends(bool flight, float tau, float b, float bs) {
-    return isinf(b) || (flight && tau <= bs);
+    return flight ? !(tau > bs) : isinf(b);
 }
 
 // vector from the point (voxel i, offset p) to the point (voxel j, offset q)

@@ -202,3 +202,19 @@ def test_back_projection_on_both_sides_of_its_rule(m, px):
     eg = rel_l2(out["grad"].cpu().numpy(), oracle.surrogate_grad(sc, L, sc.beta, meas)["grad"])
     record(f"back_projection{px}", grad=eg)
     assert eg < 1e-3, eg
+
+
+@pytest.mark.parametrize("shape,paths", [((5, 7, 9), 64), ((64, 65, 66), 400)])
+def test_backward_paths_end_in_fields_with_unusable_voxels(m, shape, paths):
+    """A NaN or an infinite extinction in the field stops or blinds paths and costs no others: every
+    path ends (both kernels), and pixels that no path of theirs brings near stay finite."""
+    sc = _scene(shape, 5, 9, px=(33, 33))
+    beta = dev(sc.beta, np.float32)
+    beta[shape[0] * shape[1] * (shape[2] - 1)] = float("nan")
+    beta[-1] = float("inf")
+    grid = m.Grid.from_scene(sc)
+    p = synth.Params(albedo=0.95, g=0.7, sun_zenith=0.5, sun_azimuth=0.4, seed=21)
+    out = grid.render_bmc(beta, m.make_params(p), paths)
+    st = grid.stats()
+    assert st["lost"] == 0 and st["bmc_paths"] == paths * sc.n_pix and st["bmc_events"] > 0
+    assert torch.isfinite(out["images"]).any()
