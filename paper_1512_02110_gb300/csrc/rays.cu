@@ -247,11 +247,11 @@ __global__ void k_images(const Geo g, const CamSet cs, const Halton hs, float in
 // whose rays part sooner, took 0.85, and adding the lanes' terms up before the atomic 0.27; neither was
 // kept: the bins next to a camera sum so many terms in FP32 that another order moves them by up to 1e-3.
 // Below this many pixels a camera, the rays of a pixel go to threads of their own: few pixels leave the
-// chip to single threads' chains of rays, many of them queue longer on the camera's voxel when all their
-// rays come at once. us apart / in one thread by pixels a camera: 1024: 41 / 137 (1 camera, 64^3), 37 / 39 (5,
-// 16^3), 101 / 105 (36, 32^3); 2025: 64 / 135, 56 / 60, 121 / 152; 4096: 127 / 160, 146 / 109, 429 / 441, 244 / 236
-// (9 cameras, 64^3), 211 / 254 (3, 96^3); 8100: 248 / 217 (1, 64^3), 390 / 316 (3, 96^3).
-constexpr int kRaysApart = 3072;
+// chip to single threads' chains of rays (us apart / in one thread, by pixels a camera: 64: 15 / 82 (1 camera, 64^3),
+// 9 / 35 (5, 16^3); 576: 31 / 123, 23 / 37). They are faster apart up to some 3000 pixels (2025: 64 / 135, 56 / 60;
+// 4096: 127 / 160, 146 / 109), but from 32^2 on the order of the FP32 sums decides: apart, the bins next to a
+// camera move by two to five times what two runs of one form differ by.
+constexpr int kRaysApart = 1024;
 __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet cs, const Halton hs, float inv_nv,
                                                      const double* __restrict__ resid, float* __restrict__ bacc,
                                                      int total_pix, double* stats) {
@@ -282,13 +282,18 @@ __global__ void __launch_bounds__(kTB) k_backproject(const Geo g, const CamSet c
 }
 
 // K5: gT_c(m) = sum_k W_c(k, m) s_c(k), s = R b = L T b (Eq. DivTc transposed).
-// Every line of a camera ends in its voxel, where the atomics queue up on one address, so the
-// blocks go round the cameras and the queues run side by side (36 cameras over 80 x 80 x 120
-// voxels: 12.1 ms camera after camera, 3.5 ms in turn).
+// Every line of a camera ends in its voxel, where the atomics queue up on one address. With more voxels
+// than the chip has threads at once the blocks therefore go round the cameras (TURN), so that the
+// queues run side by side (36 cameras over 80 x 80 x 120 voxels: 12.1 ms camera after camera, 3.3 ms
+// in turn). On smaller grids the lines of several cameras are under way anyway (64^3, 9 cameras: 0.13
+// against 0.10 ms), and camera after camera keeps the order in which a bin's FP32 terms arrive.
+template <bool TURN>
 __global__ void __launch_bounds__(kTB) k_los_adjoint(const Geo g, const CamSet cs, const float* __restrict__ R,
                                                      const float* __restrict__ bacc, float* __restrict__ gT,
                                                      double* stats) {
-    const int c = blockIdx.x % cs.n, k = (int)(blockIdx.x / cs.n) * kTB + (int)threadIdx.x;
+    const int nb = gridDim.x / cs.n;  // blocks of a camera
+    const int c = TURN ? blockIdx.x % cs.n : blockIdx.x / nb;
+    const int k = (int)(TURN ? blockIdx.x / cs.n : blockIdx.x % nb) * kTB + (int)threadIdx.x;
     unsigned nseg = 0u;
     if (k < g.nvox) {
         const Cam& cm = cs.c[c];
@@ -542,8 +547,11 @@ cudaError_t launch_backproject(const mst_grid* g, const double* resid, float* ba
 }
 
 cudaError_t launch_los_adjoint(const mst_grid* g, const float* R, const float* bacc, float* gT, cudaStream_t st) {
-    const int nb = (g->geo.nvox + kTB - 1) / kTB * g->n_cams;
-    k_los_adjoint<<<nb, kTB, 0, st>>>(g->geo, g->cams, R, bacc, gT, g->stats);
+    const int nb = (g->geo.nvox + kTB - 1) / kTB;
+    if (nb > g->sm_count * (2048 / kTB))
+        k_los_adjoint<true><<<nb * g->n_cams, kTB, 0, st>>>(g->geo, g->cams, R, bacc, gT, g->stats);
+    else
+        k_los_adjoint<false><<<nb * g->n_cams, kTB, 0, st>>>(g->geo, g->cams, R, bacc, gT, g->stats);
     return cudaGetLastError();
 }
 

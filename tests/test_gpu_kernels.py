@@ -186,9 +186,27 @@ def test_thin_grids_hold_no_halo_per_camera(m):
     assert used < 0.5e9, used
 
 
-@pytest.mark.parametrize("px", [(55, 55), (56, 55), (3072, 1)])
+def test_line_adjoint_on_both_sides_of_its_rule(m):
+    """The fixed-field gradient on grids of more and of fewer voxels than the chip has threads at once
+    (blocks in turn over the cameras, or camera after camera), against the FP64 oracle at the
+    repository's 1e-3."""
+    threads = 2048 * torch.cuda.get_device_properties(0).multi_processor_count
+    for shape, more in (((32, 32, 38), False), ((threads // 4096 + 1, 64, 64), True)):
+        assert (np.prod(shape) > threads) == more
+        sc = _scene(shape, 2, 3, px=(5, 4))
+        rng = np.random.default_rng(5)
+        L = rng.uniform(0.5, 2.0, (2, sc.nvox)) * sc.beta
+        meas = rng.uniform(0.0, 1e-4, sc.n_pix)
+        grid, beta = m.Grid.from_scene(sc), dev(sc.beta, np.float32)
+        out = grid.surrogate_grad(beta, dev(L, np.float64).view(2, -1), beta, m.make_params(synth.Params()), dev(meas, np.float64))
+        eg = rel_l2(out["grad"].cpu().numpy(), oracle.surrogate_grad(sc, L, sc.beta, meas)["grad"])
+        record(f"line_adjoint{shape}", grad=eg)
+        assert eg < 1e-3, (shape, eg)
+
+
+@pytest.mark.parametrize("px", [(32, 32), (31, 33), (1024, 1)])
 def test_back_projection_on_both_sides_of_its_rule(m, px):
-    """The fixed-field gradient with a pixel's rays in one thread (3072 pixels a camera and more) and in
+    """The fixed-field gradient with a pixel's rays in one thread (1024 pixels a camera and more) and in
     threads of their own, against the FP64 oracle at the repository's 1e-3; the ray segments are counted
     alike."""
     sc = _scene((9, 11, 7), 2, 3, px=px)
