@@ -297,10 +297,16 @@ int run_replay_stored(mst_grid* g, const mst_params* p, cudaStream_t st) {
     return MST_OK;  // what is left in the tiles is folded by launch_combine_full
 }
 
-// Per-photon buffers of the replay for n photons (at least kReplayChunk), allocated by the
-// first full-gradient call that needs them and grown when a call needs more.
+// What a full gradient needs beside the other calls' buffers: the adjoint tile and the per-photon buffers
+// for n photons (at least kReplayChunk), allocated by the first call that needs them, the latter grown
+// when a call needs more.
 int ensure_replay(mst_grid* g, uint64_t n) {
     n = std::max<uint64_t>(n, kReplayChunk);
+    if (!g->adj && cudaMalloc(&g->adj, (size_t)g->geo.nvox * g->cp * 4) != cudaSuccess) {
+        cudaGetLastError();
+        g->adj = nullptr;
+        return fail(g, MST_ERR_OOM, "adjoint tile: out of device memory");
+    }
     if (g->wbuf && g->replay_cap >= n) return MST_OK;
     auto drop = [g]() {
         cudaFree(g->wbuf);
@@ -626,7 +632,6 @@ int mst_create_grid(const mst_grid_desc* d, int n_cams, const mst_camera* cams, 
         {(void**)&g->R, C * geo.npad * 4},
         {(void**)&g->bacc, C * nvox * 4},
         {(void**)&g->gT, C * nvox * 4},
-        {(void**)&g->adj, nvox * g->cp * 4},
         {(void**)&g->gacc, (size_t)geo.npad * 4},
         {(void**)&g->g64, nvox * 8},
         {(void**)&g->resid, (size_t)off * 8},
@@ -1692,7 +1697,7 @@ int mst_batch_render_grad(mst_batch* b, const float* const* betas, const mst_par
             key_add(k, g->air);
             key_add(k, g->albedo_air);
             key_add(k, g->reg_wz);
-            const void* bufs[] = {g->wbuf, g->nevbuf, g->plist, g->evrec, g->ch_prev, g->gbrk,
+            const void* bufs[] = {g->wbuf, g->nevbuf, g->plist, g->evrec, g->ch_prev, g->gbrk, g->adj,
                                   g->warp_tail, g->Qw, g->btot, g->btot_ref};
             for (const void* q : bufs) key_add(k, q);
             key_add(k, g->ev_cap);

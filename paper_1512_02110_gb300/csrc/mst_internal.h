@@ -128,7 +128,7 @@ struct mst_grid {
     float* R = nullptr;           // [C][npad]  L_c T_c on the padded grid, halo all one bits
     float* bacc = nullptr;        // [C][nvox]  Pi_c^T (2 r_c)
     float* gT = nullptr;          // [C][nvox]  W_c^T (L T b)
-    float* adj = nullptr;         // [nvox][cp] T_c b_c
+    float* adj = nullptr;         // [nvox][cp] T_c b_c (first full gradient)
     float* gacc = nullptr;        // [npad] gradient tile on the padded grid
     float* gbrk = nullptr;        // [score_tiles][brick_bins] gradient tile in 2 x 2 x 2 bricks (first call that stores events)
     uint32_t score_tiles = 1;     // its copies

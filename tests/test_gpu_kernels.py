@@ -175,7 +175,7 @@ def test_a_new_handle_is_ready_for_any_stream(m):
 
 def test_thin_grids_hold_no_halo_per_camera(m):
     """Only the ray field R is padded: with every other field of [cameras][voxels] unpadded, one layer of
-    512 x 512 voxels and 32 cameras take 0.41 GB (R: 5 x 516^2 x 32 x 4 B; 0.69 GB with two more padded)."""
+    512 x 512 voxels and 32 cameras take 0.37 GB (R: 5 x 516^2 x 32 x 4 B; 0.65 GB with two more padded)."""
     torch.cuda.synchronize()
     sc = _scene((512, 512, 1), 32, 3, px=(4, 4))
     m.Grid.from_scene(sc).close()
